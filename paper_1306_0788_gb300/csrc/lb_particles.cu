@@ -12,197 +12,206 @@ constexpr int kPBlock = 128;
 
 inline unsigned pgrid(long long n) { return (unsigned)((n + kPBlock - 1) / kPBlock); }
 
-// Lattice row (z, y) of each particle and the row histogram.
-__global__ void k_bin(StepParams P, ParticleArrays pa, int *__restrict__ row_of, int *__restrict__ row_count,
-                      unsigned *err) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= P.np) return;
-  int4 c = pa.cell[p];
-  if (c.x < 0 || c.x >= P.nx || c.y < 0 || c.y >= P.ny || c.z < 0 || c.z >= P.nz) {
-    atomicOr(err, kErrParticle);  // cannot happen for states written by this library
-    c.x = wrapi(c.x, P.nx); c.y = wrapi(c.y, P.ny); c.z = wrapi(c.z, P.nz);
-    pa.cell[p] = c;
-  }
-  const int row = c.z * P.ny + c.y;
-  row_of[p] = row;
-  atomicAdd(row_count + row, 1);
-}
-
-// Exclusive scan of the row histogram (rows -> first sorted slot) in three passes: per-block
-// sums of 2048 rows, a scan of the block sums, and the in-block scans.  Also primes the
-// scatter cursors.
+// ------------------------------------------------------------------ particle sort
+//
+// Particles (and the reaction records of MD sub-stepping) are kept sorted by lattice row (z, y),
+// then x cell, then id: a counting sort by row whose order within a row comes from ranks.
+//   bin      the row of each particle, its rank of arrival in the row (the histogram's counter
+//            before it), and the histogram summed over the kScanRows rows of each scan block
+//   scan     rows -> first sorted slot: a block scans its rows from the sum of the block totals
+//            before it (one launch; the totals are few), and clears the counters for the next sort
+//   scatter  each particle's sort key to a slot of its row, in arrival order
+//   place    a particle's slot in its row is the number of smaller keys there; it moves
+// The keys of a row are distinct, so the order, and every gather after it, is deterministic
+// whatever the order of arrival.  Every pass is bound by latency.  Placing by rank reads a row's
+// keys from one contiguous run, a thread per particle: the insertion sort it replaces (a thread per
+// row, each move a chain of dependent loads) took 80-90 us on the records of ten substeps of 800
+// chain beads on 80^3, and a coupled step there 923 us where it now takes 450.
 using site::block_exclusive_scan;
-using site::kScanThreads;
 using site::kScanPerThread;
 using site::kScanRows;
+using site::kScanThreads;
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_partial(int nrows, const int *__restrict__ count,
-                                                               int *__restrict__ bsum) {
-  __shared__ int wt[kScanThreads / 32];
-  const int base = blockIdx.x * kScanRows + threadIdx.x * kScanPerThread;
-  int sum = 0;
-#pragma unroll
-  for (int k = 0; k < kScanPerThread; ++k)
-    if (base + k < nrows) sum += count[base + k];
-  int total;
-  block_exclusive_scan(sum, wt, total);
-  if (threadIdx.x == 0) bsum[blockIdx.x] = total;
+using SortKey = unsigned long long;
+
+__device__ __forceinline__ SortKey sort_key(int cx, int id) {
+  return ((SortKey)(unsigned)cx << 32) | (unsigned)id;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_top(int nb, int *__restrict__ bsum) {
-  __shared__ int wt[kScanThreads / 32];
-  const int per = (nb + kScanThreads - 1) / kScanThreads;
-  const int b = threadIdx.x * per;
-  int sum = 0;
-  for (int k = 0; k < per; ++k)
-    if (b + k < nb) sum += bsum[b + k];
-  int total;
-  int run = block_exclusive_scan(sum, wt, total);
-  for (int k = 0; k < per; ++k)
-    if (b + k < nb) {
-      const int c = bsum[b + k];
-      bsum[b + k] = run;
-      run += c;
+// Counts particle p (in cell c) in its row, if `valid`.  Every thread of the warp calls it.
+__device__ __forceinline__ void bin_particle(const StepParams &P, int p, bool valid, int4 c, const SortScratch &S) {
+  const int row = valid ? c.z * P.ny + c.y : -1;
+  if (valid) {
+    S.row_of[p] = row;
+    S.rank_of[p] = atomicAdd(S.row_count + row, 1);
+  }
+  // one addition per scan block a warp's particles fall in (they come nearly sorted: mostly one)
+  const int blk = valid ? row / kScanRows : -1;
+  const unsigned same = __match_any_sync(0xffffffffu, blk);
+  if (valid && (int)(threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(S.block_count + blk, __popc(same));
+}
+
+__global__ void __launch_bounds__(kPBlock) k_bin(StepParams P, ParticleArrays pa, SortScratch S, unsigned *err) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool valid = p < P.np;
+  int4 c = make_int4(0, 0, 0, 0);
+  if (valid) {
+    c = pa.cell[p];
+    if (c.x < 0 || c.x >= P.nx || c.y < 0 || c.y >= P.ny || c.z < 0 || c.z >= P.nz) {
+      atomicOr(err, kErrParticle);  // cannot happen for states written by this library
+      c.x = wrapi(c.x, P.nx); c.y = wrapi(c.y, P.ny); c.z = wrapi(c.z, P.nz);
+      pa.cell[p] = c;
     }
-  if (threadIdx.x == 0) bsum[nb] = total;
+  }
+  bin_particle(P, p, valid, c, S);
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_final(int nrows, int nb, const int *__restrict__ count,
-                                                             const int *__restrict__ bsum, int *__restrict__ start,
-                                                             int *__restrict__ cursor) {
+// Particle update (site::integrate) from src into dst, in the same order, and the bin pass of the
+// sort that follows it.
+__global__ void __launch_bounds__(kPBlock) k_integrate_bin(StepParams P, ParticleArrays src, ParticleArrays dst,
+                                                           ParticleForces pf, SortScratch S, unsigned *err) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool valid = p < P.np;
+  bin_particle(P, p, valid, valid ? site::integrate(P, p, src, dst, pf, err) : make_int4(0, 0, 0, 0), S);
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_rows(int nrows, SortScratch S, int *__restrict__ start) {
   __shared__ int wt[kScanThreads / 32];
+  int total;
+  int before = 0;
+  for (int b = threadIdx.x; b < (int)blockIdx.x; b += kScanThreads) before += S.block_count[b];
+  block_exclusive_scan(before, wt, total);
+  before = total;  // particles in the rows of the blocks before this one
+  __syncthreads();
   const int base = blockIdx.x * kScanRows + threadIdx.x * kScanPerThread;
   int c[kScanPerThread];
   int sum = 0;
 #pragma unroll
   for (int k = 0; k < kScanPerThread; ++k) {
-    c[k] = base + k < nrows ? count[base + k] : 0;
+    c[k] = base + k < nrows ? S.row_count[base + k] : 0;
     sum += c[k];
   }
-  int total;
-  int run = bsum[blockIdx.x] + block_exclusive_scan(sum, wt, total);
+  int run = before + block_exclusive_scan(sum, wt, total);
 #pragma unroll
   for (int k = 0; k < kScanPerThread; ++k)
     if (base + k < nrows) {
       start[base + k] = run;
-      cursor[base + k] = run;
+      S.row_count[base + k] = 0;
       run += c[k];
     }
-  if (blockIdx.x == nb - 1 && threadIdx.x == 0) start[nrows] = bsum[nb];
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) start[nrows] = before + total;
 }
 
-__global__ void k_scatter(int np, const int *__restrict__ row_of, int *__restrict__ cursor, int *__restrict__ perm) {
+__global__ void __launch_bounds__(kPBlock) k_scatter(int np, int nblocks, SortScratch S, const int *__restrict__ start,
+                                                     const int4 *__restrict__ cell, const int *__restrict__ id) {
+  if (blockIdx.x == 0)  // the block totals have been read: cleared for the next sort
+    for (int b = threadIdx.x; b < nblocks; b += kPBlock) S.block_count[b] = 0;
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= np) return;
-  perm[atomicAdd(cursor + row_of[p], 1)] = p;
+  const int row = S.row_of[p];
+  const int j = start[row] + S.rank_of[p];
+  S.perm[j] = p;
+  S.row_at[j] = row;
+  S.key[j] = sort_key(cell[p].x, id[p]);
 }
 
-// Order each row by (x cell, particle id) so the sort, and every gather after it, is
-// deterministic.  Rows hold few particles: insertion sort, one thread per row.
-__global__ void k_row_sort(StepParams P, const int *__restrict__ start, ParticleArrays pa, int *__restrict__ perm) {
-  const int row = blockIdx.x * blockDim.x + threadIdx.x;
-  if (row >= P.nrows) return;
+// The slot of the entry scattered to j: the first slot of its row plus its rank there.
+__device__ __forceinline__ int placed_slot(int j, const SortScratch &S, const int *__restrict__ start) {
+  const int row = S.row_at[j];
+  const SortKey key = S.key[j];
   const int b = start[row], e = start[row + 1];
-  for (int i = b + 1; i < e; ++i) {
-    const int v = perm[i];
-    const long long kv = ((long long)pa.cell[v].x << 32) | (unsigned)pa.pid[v];
-    int j = i - 1;
-    while (j >= b) {
-      const int w = perm[j];
-      const long long kw = ((long long)pa.cell[w].x << 32) | (unsigned)pa.pid[w];
-      if (kw <= kv) break;
-      perm[j + 1] = w;
-      --j;
-    }
-    perm[j + 1] = v;
-  }
+  int slot = b;
+  for (int q = b; q < e; ++q) slot += S.key[q] < key;
+  return slot;
 }
 
-__global__ void k_permute(int np, const int *__restrict__ perm, ParticleArrays src, ParticleArrays dst,
-                          int *__restrict__ slot_of_id) {
+__device__ __forceinline__ void move_particle(const ParticleArrays &src, int p, const ParticleArrays &dst, int slot,
+                                              int *__restrict__ slot_of_id) {
+  const int id = src.pid[p];
+  dst.cell[slot] = src.cell[p];
+  dst.frac[slot] = src.frac[p];
+  dst.vel[slot] = src.vel[p];
+  dst.pid[slot] = id;
+  slot_of_id[id] = slot;
+}
+
+__global__ void __launch_bounds__(kPBlock) k_place(int np, SortScratch S, const int *__restrict__ start,
+                                                   ParticleArrays src, ParticleArrays dst,
+                                                   int *__restrict__ slot_of_id) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= np) return;
-  const int p = perm[j];
-  dst.cell[j] = src.cell[p];
-  dst.frac[j] = src.frac[p];
-  dst.vel[j] = src.vel[p];
-  const int id = src.pid[p];
-  dst.pid[j] = id;
-  slot_of_id[id] = j;
+  move_particle(src, S.perm[j], dst, placed_slot(j, S, start), slot_of_id);
 }
 
-// The whole counting sort of a small system in one block: the steps of k_bin ... k_permute
-// (histogram with the same range check, exclusive scan, scatter, order by (x cell, id) within a
-// row, permutation) with the counts and the permutation in shared memory, one launch instead of
-// a chain of seven that a step of a small lattice would wait for.  The order is unique, so the
-// result is that of the chain.
-constexpr int kSortSmallRows = 4096, kSortSmallNp = 2048;
+// The particle update (kUpdate) and the whole sort of a small system in one block, the counters,
+// keys and slots in shared memory: one launch instead of four that a step of a small lattice would
+// wait for.  The order is unique, so the result is that of the chain.  With 256 threads, insertion
+// sorts per row and the update in a kernel before it, 1000 particles on 64^3 took 23 + 4 us and a
+// coupled step 45 us; now the step takes 29.  The limits are what one block's shared memory holds
+// with room to spare (112 KB); a step of 100 x 90 x 110 (9900 rows, 1000 particles) hides the four
+// launches of the chain behind its lattice update.
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallRows = 8192, kSmallNp = 4096;
 
-__global__ void __launch_bounds__(kScanThreads) k_sort_small(StepParams P, ParticleArrays src, ParticleArrays dst,
-                                                             int *__restrict__ start, int *__restrict__ slot_of_id,
-                                                             unsigned *err) {
-  __shared__ int count[kSortSmallRows];  // histogram, then the scatter cursors (= row ends)
-  __shared__ int row_of[kSortSmallNp];
-  __shared__ int perm[kSortSmallNp];
-  __shared__ int wt[kScanThreads / 32];
+inline size_t small_smem(int nrows, int np) { return sizeof(int) * (size_t)(nrows + 1) + (size_t)np * 20 + 16; }
+
+template <bool kUpdate>
+__global__ void __launch_bounds__(kSmallThreads) k_sort_small(StepParams P, ParticleArrays src, ParticleArrays mid,
+                                                              ParticleForces pf, ParticleArrays dst,
+                                                              int *__restrict__ start, int *__restrict__ slot_of_id,
+                                                              unsigned *err) {
+  extern __shared__ SortKey small_keys[];
+  __shared__ int wt[kSmallThreads / 32];
   const int np = P.np, nrows = P.nrows;
-  for (int r = threadIdx.x; r < nrows; r += kScanThreads) count[r] = 0;
+  SortKey *key = small_keys;                            // [np] by particle
+  int *row_of = reinterpret_cast<int *>(key + np);      // [np]
+  int *rank_of = row_of + np;                           // [np]
+  int *list = rank_of + np;                             // [np] the particles of each row, in arrival order
+  int *row = list + np;                                 // [nrows + 1] counters, then first slots
+  for (int r = threadIdx.x; r <= nrows; r += kSmallThreads) row[r] = 0;
   __syncthreads();
-  for (int p = threadIdx.x; p < np; p += kScanThreads) {
-    int4 c = src.cell[p];
-    if (c.x < 0 || c.x >= P.nx || c.y < 0 || c.y >= P.ny || c.z < 0 || c.z >= P.nz) {
-      atomicOr(err, kErrParticle);  // cannot happen for states written by this library
-      c.x = wrapi(c.x, P.nx); c.y = wrapi(c.y, P.ny); c.z = wrapi(c.z, P.nz);
-      src.cell[p] = c;
+  for (int p = threadIdx.x; p < np; p += kSmallThreads) {
+    int4 c;
+    if (kUpdate) {
+      c = site::integrate(P, p, src, mid, pf, err);
+    } else {
+      c = mid.cell[p];
+      if (c.x < 0 || c.x >= P.nx || c.y < 0 || c.y >= P.ny || c.z < 0 || c.z >= P.nz) {
+        atomicOr(err, kErrParticle);  // cannot happen for states written by this library
+        c.x = wrapi(c.x, P.nx); c.y = wrapi(c.y, P.ny); c.z = wrapi(c.z, P.nz);
+        mid.cell[p] = c;
+      }
     }
-    const int row = c.z * P.ny + c.y;
-    row_of[p] = row;
-    atomicAdd(&count[row], 1);
+    const int r = c.z * P.ny + c.y;
+    row_of[p] = r;
+    rank_of[p] = atomicAdd(&row[r], 1);
+    key[p] = sort_key(c.x, (kUpdate ? src : mid).pid[p]);
   }
   __syncthreads();
-  const int per = (nrows + kScanThreads - 1) / kScanThreads;  // consecutive rows of a thread
-  const int b = threadIdx.x * per;
+  const int per = (nrows + kSmallThreads - 1) / kSmallThreads;  // consecutive rows of a thread
+  const int b0 = threadIdx.x * per;
   int sum = 0;
   for (int k = 0; k < per; ++k)
-    if (b + k < nrows) sum += count[b + k];
+    if (b0 + k < nrows) sum += row[b0 + k];
   int total;
-  int run = block_exclusive_scan(sum, wt, total);
+  int run = block_exclusive_scan<kSmallThreads>(sum, wt, total);
   for (int k = 0; k < per; ++k)
-    if (b + k < nrows) {
-      const int n = count[b + k];
-      start[b + k] = run;
-      count[b + k] = run;
+    if (b0 + k < nrows) {
+      const int n = row[b0 + k];
+      row[b0 + k] = run;
+      start[b0 + k] = run;
       run += n;
     }
-  if (threadIdx.x == 0) start[nrows] = total;
+  if (threadIdx.x == 0) row[nrows] = start[nrows] = total;
   __syncthreads();
-  for (int p = threadIdx.x; p < np; p += kScanThreads) perm[atomicAdd(&count[row_of[p]], 1)] = p;
+  for (int p = threadIdx.x; p < np; p += kSmallThreads) list[row[row_of[p]] + rank_of[p]] = p;
   __syncthreads();
-  for (int r = threadIdx.x; r < nrows; r += kScanThreads) {  // row r holds slots [end of r-1, end of r)
-    const int b0 = r == 0 ? 0 : count[r - 1], e0 = count[r];
-    for (int i = b0 + 1; i < e0; ++i) {
-      const int v = perm[i];
-      const long long kv = ((long long)src.cell[v].x << 32) | (unsigned)src.pid[v];
-      int j = i - 1;
-      while (j >= b0) {
-        const int w = perm[j];
-        const long long kw = ((long long)src.cell[w].x << 32) | (unsigned)src.pid[w];
-        if (kw <= kv) break;
-        perm[j + 1] = w;
-        --j;
-      }
-      perm[j + 1] = v;
-    }
-  }
-  __syncthreads();
-  for (int j = threadIdx.x; j < np; j += kScanThreads) {
-    const int p = perm[j];
-    dst.cell[j] = src.cell[p];
-    dst.frac[j] = src.frac[p];
-    dst.vel[j] = src.vel[p];
-    const int id = src.pid[p];
-    dst.pid[j] = id;
-    slot_of_id[id] = j;
+  for (int p = threadIdx.x; p < np; p += kSmallThreads) {
+    const int b = row[row_of[p]], e = row[row_of[p] + 1];
+    const SortKey mine = key[p];
+    int slot = b;
+    for (int q = b; q < e; ++q) slot += key[list[q]] < mine;
+    move_particle(mid, p, dst, slot, slot_of_id);  // (this thread wrote entry p of mid)
   }
 }
 
@@ -254,13 +263,6 @@ __global__ void __launch_bounds__(kPBlock) k_pairs(StepParams P, ParticleArrays 
   site::pairs8(P, p, k, 0xFFu << (threadIdx.x & 24), pa, ci, bond_start, bond_other, slot_of_id, pf, err);
 }
 
-// Particle update (site::integrate) from src into dst, in the same order (dst may be src).
-__global__ void k_integrate(StepParams P, ParticleArrays src, ParticleArrays dst, ParticleForces pf, unsigned *err) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= P.np) return;
-  site::integrate(P, p, src, dst, pf, err);
-}
-
 // ------------------------------------------------------------------ MD sub-stepping
 
 // Coupling forces of substep `sub` at the particles' current positions C (in the order of the
@@ -301,16 +303,19 @@ __global__ void k_integrate_sub(StepParams P, ParticleArrays C, ParticleArrays S
   if (dx > 1 || dx < -1 || dy > 1 || dy < -1 || dz > 1 || dz < -1) atomicOr(err, kErrTooFast);
 }
 
-__global__ void k_rec_permute(int n, const int *__restrict__ perm, ReactionRecords src, ReactionRecords dst) {
+__global__ void __launch_bounds__(kPBlock) k_rec_place(int n, SortScratch S, const int *__restrict__ start,
+                                                       ReactionRecords src, ReactionRecords dst) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
-  const int p = perm[j];
-  dst.cell[j] = src.cell[p];
-  dst.frac[j] = src.frac[p];
-  dst.key[j] = src.key[p];
-  dst.fric[j] = src.fric[p];
-  dst.psA[j] = src.psA[p];
-  dst.psB[j] = src.psB[p];
+  const int p = S.perm[j];
+  const int4 c = src.cell[p];
+  const float4 fr = src.frac[p], a = src.fric[p], b = src.psA[p], d = src.psB[p];
+  const int slot = placed_slot(j, S, start);
+  dst.cell[slot] = c;
+  dst.frac[slot] = fr;
+  dst.fric[slot] = a;
+  dst.psA[slot] = b;
+  dst.psB[slot] = d;
 }
 
 constexpr int kMomBlock = 256;
@@ -373,35 +378,49 @@ __global__ void __launch_bounds__(kPBlock) k_particles_out(int n, ParticleArrays
 
 }  // namespace
 
-void launch_bin(const StepParams &P, const ParticleArrays &pa, int *row_of, int *row_count, unsigned *err,
-                cudaStream_t st) {
-  k_bin<<<pgrid(P.np), kPBlock, 0, st>>>(P, pa, row_of, row_count, err);
-}
 int scan_blocks(int nrows) { return (nrows + kScanRows - 1) / kScanRows; }
-void launch_scan_rows(int nrows, const int *row_count, int *row_start, int *row_cursor, int *bsum, cudaStream_t st) {
-  const int nb = scan_blocks(nrows);
-  k_scan_partial<<<nb, kScanThreads, 0, st>>>(nrows, row_count, bsum);
-  k_scan_top<<<1, kScanThreads, 0, st>>>(nb, bsum);
-  k_scan_final<<<nb, kScanThreads, 0, st>>>(nrows, nb, row_count, bsum, row_start, row_cursor);
-}
-bool sort_fits_one_block(int nrows, int np) { return nrows <= kSortSmallRows && np <= kSortSmallNp; }
 
-void launch_sort_small(const StepParams &P, const ParticleArrays &src, const ParticleArrays &dst, int *row_start,
-                       int *slot_of_id, unsigned *err, cudaStream_t st) {
-  k_sort_small<<<1, kScanThreads, 0, st>>>(P, src, dst, row_start, slot_of_id, err);
+void launch_bin(const StepParams &P, const ParticleArrays &pa, const SortScratch &S, unsigned *err, cudaStream_t st) {
+  k_bin<<<pgrid(P.np), kPBlock, 0, st>>>(P, pa, S, err);
+}
+void launch_integrate_bin(const StepParams &P, const ParticleArrays &src, const ParticleArrays &dst,
+                          const ParticleForces &pf, const SortScratch &S, unsigned *err, cudaStream_t st) {
+  k_integrate_bin<<<pgrid(P.np), kPBlock, 0, st>>>(P, src, dst, pf, S, err);
+}
+// The scan and scatter passes of np binned entries.
+static void scan_scatter(const StepParams &P, int np, const SortScratch &S, int *row_start, const int4 *cell,
+                         const int *id, cudaStream_t st) {
+  const int nb = scan_blocks(P.nrows);
+  k_scan_rows<<<nb, kScanThreads, 0, st>>>(P.nrows, S, row_start);
+  k_scatter<<<pgrid(np), kPBlock, 0, st>>>(np, nb, S, row_start, cell, id);
+}
+void launch_place(const StepParams &P, const SortScratch &S, const ParticleArrays &src, const ParticleArrays &dst,
+                  int *row_start, int *slot_of_id, cudaStream_t st) {
+  scan_scatter(P, P.np, S, row_start, src.cell, src.pid, st);
+  k_place<<<pgrid(P.np), kPBlock, 0, st>>>(P.np, S, row_start, src, dst, slot_of_id);
+}
+void launch_rec_place(const StepParams &P, int n, const SortScratch &S, const ReactionRecords &src,
+                      const ReactionRecords &dst, int *row_start, cudaStream_t st) {
+  scan_scatter(P, n, S, row_start, src.cell, src.key, st);
+  k_rec_place<<<pgrid(n), kPBlock, 0, st>>>(n, S, row_start, src, dst);
 }
 
-void launch_scatter(int np, const int *row_of, int *row_cursor, int *perm, cudaStream_t st) {
-  k_scatter<<<pgrid(np), kPBlock, 0, st>>>(np, row_of, row_cursor, perm);
+bool sort_fits_one_block(int nrows, int np) { return nrows <= kSmallRows && np <= kSmallNp; }
+
+void launch_sort_small(const StepParams &P, const ParticleArrays *update_from, const ParticleArrays &mid,
+                       const ParticleForces &pf, const ParticleArrays &dst, int *row_start, int *slot_of_id,
+                       unsigned *err, cudaStream_t st) {
+  const size_t smem = small_smem(P.nrows, P.np);
+  const int most = (int)small_smem(kSmallRows, kSmallNp);
+  if (update_from) {
+    cudaFuncSetAttribute(k_sort_small<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    k_sort_small<true><<<1, kSmallThreads, smem, st>>>(P, *update_from, mid, pf, dst, row_start, slot_of_id, err);
+  } else {
+    cudaFuncSetAttribute(k_sort_small<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    k_sort_small<false><<<1, kSmallThreads, smem, st>>>(P, mid, mid, pf, dst, row_start, slot_of_id, err);
+  }
 }
-void launch_row_sort(const StepParams &P, const int *row_start, const ParticleArrays &pa, int *perm,
-                     cudaStream_t st) {
-  k_row_sort<<<pgrid(P.nrows), kPBlock, 0, st>>>(P, row_start, pa, perm);
-}
-void launch_permute(int np, const int *perm, const ParticleArrays &src, const ParticleArrays &dst, int *slot_of_id,
-                    cudaStream_t st) {
-  k_permute<<<pgrid(np), kPBlock, 0, st>>>(np, perm, src, dst, slot_of_id);
-}
+
 void launch_couple(const StepParams &P, const ParticleArrays &pa, CellIndex ci, const float *rho, const float *jp,
                    const ParticleForces &pf, cudaStream_t st) {
   k_couple<<<pgrid(8LL * P.np), kPBlock, 0, st>>>(P, pa, ci, rho, jp, pf);
@@ -430,10 +449,6 @@ void launch_pairs(const StepParams &P, const ParticleArrays &pa, CellIndex ci, c
                   cudaStream_t st) {
   k_pairs<<<pgrid(8LL * P.np), kPBlock, 0, st>>>(P, pa, ci, bond_start, bond_other, slot_of_id, pf, err);
 }
-void launch_integrate(const StepParams &P, const ParticleArrays &src, const ParticleArrays &dst,
-                      const ParticleForces &pf, unsigned *err, cudaStream_t st) {
-  k_integrate<<<pgrid(P.np), kPBlock, 0, st>>>(P, src, dst, pf, err);
-}
 void launch_couple_sub(const StepParams &P, const ParticleArrays &C, const ParticleArrays &S, CellIndex ci,
                        const float *rho, const float *jp, const ParticleForces &pf, int sub,
                        const ReactionRecords &rec, cudaStream_t st) {
@@ -442,10 +457,6 @@ void launch_couple_sub(const StepParams &P, const ParticleArrays &C, const Parti
 void launch_integrate_sub(const StepParams &P, const ParticleArrays &C, const ParticleArrays &S,
                           const ParticleForces &pf, unsigned *err, cudaStream_t st) {
   k_integrate_sub<<<pgrid(P.np), kPBlock, 0, st>>>(P, C, S, pf, err);
-}
-void launch_rec_permute(int n, const int *perm, const ReactionRecords &src, const ReactionRecords &dst,
-                        cudaStream_t st) {
-  k_rec_permute<<<pgrid(n), kPBlock, 0, st>>>(n, perm, src, dst);
 }
 void launch_particle_momentum(const StepParams &P, const ParticleArrays &pa, double *partial, int nblocks,
                               cudaStream_t st) {

@@ -1050,8 +1050,9 @@ __device__ __forceinline__ void pairs8(const StepParams &P, int p, int k, unsign
 }
 
 // Particle update of slot p: v += F dt / m, x += v dt, periodic wrap kept as (cell,
-// fraction).  Reads src, writes dst (the same arrays for an update in place).
-__device__ __forceinline__ void integrate(const StepParams &P, int p, const ParticleArrays &src,
+// fraction).  Reads src, writes dst (the same arrays for an update in place) and returns the new
+// cell, which is inside the lattice.
+__device__ __forceinline__ int4 integrate(const StepParams &P, int p, const ParticleArrays &src,
                                           const ParticleArrays &dst, const ParticleForces &pf, unsigned *err) {
   int4 c = src.cell[p];
   float4 fr = src.frac[p];
@@ -1073,7 +1074,7 @@ __device__ __forceinline__ void integrate(const StepParams &P, int p, const Part
     dst.cell[p] = c;  // position kept: every index stays inside the lattice
     dst.frac[p] = fr;
     dst.vel[p] = make_float4(0.f, 0.f, 0.f, 0.f);
-    return;
+    return c;
   }
   const float sx = floorf(nx_), sy = floorf(ny_), sz = floorf(nz_);
   nx_ -= sx; ny_ -= sy; nz_ -= sz;
@@ -1087,17 +1088,19 @@ __device__ __forceinline__ void integrate(const StepParams &P, int p, const Part
   dst.cell[p] = c;
   dst.frac[p] = make_float4(nx_, ny_, nz_, fr.w);
   dst.vel[p] = v;
+  return c;
 }
 
 // ------------------------------------------------------------------ row scan
 
-// Exclusive scan of one value per thread over a block of kScanThreads threads (warp shuffles,
+// Exclusive scan of one value per thread over a block of kThreads threads (warp shuffles,
 // then a scan of the warp totals); `total` receives the block's sum.  Every thread of the block
 // must call it.
 constexpr int kScanThreads = 256;
 constexpr int kScanPerThread = 8;
 constexpr int kScanRows = kScanThreads * kScanPerThread;
 
+template <int kThreads = kScanThreads>
 __device__ __forceinline__ int block_exclusive_scan(int v, int *warp_tot, int &total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int x = v;
@@ -1109,16 +1112,16 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *warp_tot, int &t
   if (lane == 31) warp_tot[warp] = x;
   __syncthreads();
   if (warp == 0) {
-    int t = lane < kScanThreads / 32 ? warp_tot[lane] : 0;
+    int t = lane < kThreads / 32 ? warp_tot[lane] : 0;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int y = __shfl_up_sync(0xffffffffu, t, o);
       if (lane >= o) t += y;
     }
-    if (lane < kScanThreads / 32) warp_tot[lane] = t;  // inclusive warp-total prefix
+    if (lane < kThreads / 32) warp_tot[lane] = t;  // inclusive warp-total prefix
   }
   __syncthreads();
-  total = warp_tot[kScanThreads / 32 - 1];
+  total = warp_tot[kThreads / 32 - 1];
   const int before = warp == 0 ? 0 : warp_tot[warp - 1];
   return before + x - v;
 }

@@ -117,6 +117,18 @@ struct ReactionRecords {
   float4 *fric, *psA, *psB;
 };
 
+// Scratch of the particle sort (entries: particles, or reaction records).  row_count and
+// block_count are zero between sorts.
+struct SortScratch {
+  int *row_count;    // [nrows] histogram
+  int *block_count;  // [scan_blocks(nrows)] the histogram summed over the rows of each scan block
+  int *row_of;       // [entries] row
+  int *rank_of;      // [entries] rank of arrival in the row
+  int *perm;         // [entries] the entry scattered to a slot,
+  int *row_at;       // [entries] its row
+  unsigned long long *key;  // [entries] and its sort key
+};
+
 struct CellIndex {
   const int *row_start;  // [nrows + 1] offsets into the sorted particle arrays
 };
@@ -310,20 +322,23 @@ void launch_drift_check(const double *sums, const double *psum, double *ref, dou
                         long long step, double tol, int set_ref, cudaStream_t st);
 
 // particles (lb_particles.cu)
-void launch_bin(const StepParams &P, const ParticleArrays &pa, int *row_of, int *row_count,
-                unsigned *err, cudaStream_t st);
-int scan_blocks(int nrows);  // size of the block-sum scratch is scan_blocks(nrows) + 1
-void launch_scan_rows(int nrows, const int *row_count, int *row_start, int *row_cursor, int *bsum, cudaStream_t st);
-void launch_scatter(int np, const int *row_of, int *row_cursor, int *perm, cudaStream_t st);
-// The particle sort of a small system (nrows and np within one block's shared memory) in one
-// launch: row_start and the sorted copy dst of src, as the chain bin ... permute gives them.
+// The sort of the particles by (row, x cell, id): the bin pass (alone, or with the particle update
+// from src into dst), then launch_place, which leaves src sorted in dst with row_start and
+// slot_of_id.  launch_rec_place is the same for n binned reaction records.
+int scan_blocks(int nrows);
+void launch_bin(const StepParams &P, const ParticleArrays &pa, const SortScratch &S, unsigned *err, cudaStream_t st);
+void launch_integrate_bin(const StepParams &P, const ParticleArrays &src, const ParticleArrays &dst,
+                          const ParticleForces &pf, const SortScratch &S, unsigned *err, cudaStream_t st);
+void launch_place(const StepParams &P, const SortScratch &S, const ParticleArrays &src, const ParticleArrays &dst,
+                  int *row_start, int *slot_of_id, cudaStream_t st);
+void launch_rec_place(const StepParams &P, int n, const SortScratch &S, const ReactionRecords &src,
+                      const ReactionRecords &dst, int *row_start, cudaStream_t st);
+// The same for a small system (nrows and np within one block's shared memory) in one launch: with
+// update_from, the particles are first updated from there into mid; mid is sorted into dst.
 bool sort_fits_one_block(int nrows, int np);
-void launch_sort_small(const StepParams &P, const ParticleArrays &src, const ParticleArrays &dst, int *row_start,
-                       int *slot_of_id, unsigned *err, cudaStream_t st);
-void launch_row_sort(const StepParams &P, const int *row_start, const ParticleArrays &pa, int *perm,
-                     cudaStream_t st);
-void launch_permute(int np, const int *perm, const ParticleArrays &src, const ParticleArrays &dst,
-                    int *slot_of_id, cudaStream_t st);
+void launch_sort_small(const StepParams &P, const ParticleArrays *update_from, const ParticleArrays &mid,
+                       const ParticleForces &pf, const ParticleArrays &dst, int *row_start, int *slot_of_id,
+                       unsigned *err, cudaStream_t st);
 void launch_couple(const StepParams &P, const ParticleArrays &pa, CellIndex ci, const float *rho,
                    const float *jp, const ParticleForces &pf, cudaStream_t st);
 // The same with j' at the corners from jc (8 float4 per particle id, launch_corner_jprime or the
@@ -337,8 +352,6 @@ void launch_corner_jprime(const StepParams &P, const ParticleArrays &pa, int np,
 void launch_pairs(const StepParams &P, const ParticleArrays &pa, CellIndex ci, const int *bond_start,
                   const int *bond_other, const int *slot_of_id, const ParticleForces &pf, unsigned *err,
                   cudaStream_t st);
-void launch_integrate(const StepParams &P, const ParticleArrays &src, const ParticleArrays &dst,
-                      const ParticleForces &pf, unsigned *err, cudaStream_t st);
 // Positions (cell + fraction, in FP64), velocities and the total forces of the last step of n
 // particles into device arrays [n][3] in the caller's particle order; any output may be null.
 // tid_of: the caller's index of each entry of total (the order the particle update wrote them).
@@ -355,7 +368,4 @@ void launch_couple_sub(const StepParams &P, const ParticleArrays &C, const Parti
                        const ReactionRecords &rec, cudaStream_t st);
 void launch_integrate_sub(const StepParams &P, const ParticleArrays &C, const ParticleArrays &S,
                           const ParticleForces &pf, unsigned *err, cudaStream_t st);
-void launch_rec_permute(int n, const int *perm, const ReactionRecords &src, const ReactionRecords &dst,
-                        cudaStream_t st);
-
 }  // namespace lbmd
