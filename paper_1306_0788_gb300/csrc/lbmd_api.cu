@@ -250,20 +250,48 @@ void free_particles(lbmd_ctx *c) {
 }
 
 // One-pass update: BGK, one particle update per lattice step.  Chosen by the lattice size
-// unless set (lbmd_set_lattice_passes): when the blocks of the full persistent grid march at least
-// kOnePassAutoPlanes planes each; smaller lattices (set to one pass) take a grid of stretches of
-// kOnePassMinPlanes planes.
-constexpr int kOnePassMinPlanes = 8;
-constexpr int kOnePassAutoPlanes = 16;
+// unless set (lbmd_set_lattice_passes); see onepass_pays and onepass_chunks.
 constexpr int kOnePassChunkPlanes = 16;
 
 bool onepass_allowed(const lbmd_ctx *c) {
   return c->P.collision == LBMD_COLLISION_BGK && c->P.substeps == 1;
 }
 
-long long onepass_units(const StepParams &P) {
+// Whether one pass is the faster update, from what both took per step without particles (FP32,
+// BGK, microseconds, two passes / one pass): 64^3 16.3 / 21.6, 80^3 33.9 / 38.8, 96^3 64.7 / 54.9,
+// 100^3 75.8 / 74.8, 112^3 102 / 86, 128^3 150 / 119, 144^3 212 / 174, 192^3 476 / 382, 256^3
+// 1124 / 886.  Two passes take about 72 ps per node there (less where the lattice stays in L2), one
+// pass 8 us and 53 ps per lane of its 32 x 8 tiles, idle ones included: it loses where tiles are
+// ragged (100 = 3 x 32 + 4 columns) and where the lattice is small.
+bool onepass_pays(const StepParams &P) {
   const long long ntx = (P.nx + kOnePassCols - 1) / kOnePassCols, nty = (P.ny + kOnePassRows - 1) / kOnePassRows;
-  return ntx * nty * P.nz;
+  const double lanes = (double)(ntx * nty * P.nz) * (kOnePassCols * kOnePassRows);
+  return 53.0 * lanes + 8.0e6 < 72.0 * (double)P.N;
+}
+
+// The z-chunks of the one-pass update, a block for each column tile of a chunk: chunks of 16 planes,
+// unless another count (8 to 32 planes: longer chunks let neighbouring blocks drift apart, and the
+// sectors they share out of L2) fills the waves of the `slots` resident blocks better by 3 % or
+// more, counting the 0.4 planes a block spends on its start and end.  With 16 planes, 128^3 has 512
+// blocks on 456 slots and takes 138 us a step; with 7 chunks, 119 (a coupled step with 2500
+// particles 184 -> 148 us).  Where there are many waves the count hardly matters: 886 to 901 us for 7
+// to 32 chunks at 256^3.
+int onepass_chunks(int tiles, int nz, int slots) {
+  auto score = [&](int n) {
+    const double waves = (double)tiles * n / slots, planes = (double)nz / n;
+    return waves / std::ceil(waves) * planes / (planes + 0.4);
+  };
+  const int usual = std::max(1, (nz + kOnePassChunkPlanes / 2) / kOnePassChunkPlanes);
+  int best = usual;
+  double best_score = score(usual) * 1.03;
+  const int least = (nz + 2 * kOnePassChunkPlanes - 1) / (2 * kOnePassChunkPlanes);
+  const int most = std::min(2 * nz / kOnePassChunkPlanes, 64 * slots / tiles);  // past 64 waves: all alike
+  for (int n = least; n <= most; ++n)
+    if (score(n) > best_score) {
+      best_score = score(n);
+      best = n;
+    }
+  return best;
 }
 
 int onepass_full_grid(const lbmd_ctx *c) {
@@ -301,18 +329,15 @@ int prepare_onepass(lbmd_ctx *c) {
   // set up already (op_grid; the run list may be empty: every node finished from partial sums)
   if (!onepass_allowed(c) || c->passes == 2 || c->op_grid > 0) return LBMD_OK;
   const StepParams &P = c->P;
-  const long long U = onepass_units(P);
-  const int full = onepass_full_grid(c);
-  // automatic: one pass for FP32 storage on lattices large enough (the 16-bit update is bound by
-  // instruction issue, and the one-pass update's extra instructions cost it more than the second
-  // pass over half the bytes)
-  if (c->passes == 0 && (P.storage != LBMD_STORAGE_FP32 || U < (long long)kOnePassAutoPlanes * full))
-    return LBMD_OK;  // two passes
+  // automatic: one pass for FP32 storage where it pays (the 16-bit update is bound by instruction
+  // issue, and the one-pass update's extra instructions cost it more than the second pass over half
+  // the bytes)
+  if (c->passes == 0 && (P.storage != LBMD_STORAGE_FP32 || !onepass_pays(P))) return LBMD_OK;  // two passes
   free_onepass(c);  // what an earlier attempt that failed part-way left
   const int ntx = (P.nx + kOnePassCols - 1) / kOnePassCols, nty = (P.ny + kOnePassRows - 1) / kOnePassRows;
-  // chunks of about kOnePassChunkPlanes planes, one block each, neighbouring column tiles of a
-  // chunk launched together (they march in step, so the sectors they share meet in L2)
-  const int nchunks = std::max(1, (P.nz + kOnePassChunkPlanes / 2) / kOnePassChunkPlanes);
+  // neighbouring column tiles of a chunk are launched together (they march in step, so the sectors
+  // they share meet in L2)
+  const int nchunks = onepass_chunks(ntx * nty, P.nz, onepass_full_grid(c));
   const int grid = ntx * nty * nchunks;
   std::vector<unsigned char> edge((size_t)ntx * nty * P.nz, 0);
   for (int col = 0; col < ntx * nty; ++col)
