@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(kPBlock) k_couple(StepParams P, ParticleArrays
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int p = (int)(t >> 3), k = (int)(t & 7);
   if (p >= P.np) return;
-  site::couple8(P, noise_step(P, P.step), p, k, 0xFFu << (threadIdx.x & 24), pa, pa, ci, rho, jp, pf);
+  site::couple8(P, noise_step(P, P.step), p, k, 0xFFu << (threadIdx.x & 24), pa, ci, rho, jp, pf);
 }
 
 // k_couple with j' at each corner already formed (jc, 8 float4 per particle id).
@@ -233,8 +233,7 @@ __global__ void __launch_bounds__(kPBlock) k_couple_jc(StepParams P, ParticleArr
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int p = (int)(t >> 3), k = (int)(t & 7);
   if (p >= P.np) return;
-  site::couple8(P, noise_step(P, P.step), p, k, 0xFFu << (threadIdx.x & 24), pa, pa, ci, rho, nullptr, pf, true,
-                jc);
+  site::couple8(P, noise_step(P, P.step), p, k, 0xFFu << (threadIdx.x & 24), pa, ci, rho, nullptr, pf, jc);
 }
 
 // j' = sum_z sum_i f_zi c_i of the populations `store` at the 8 corners of every particle's cell,
@@ -265,42 +264,71 @@ __global__ void __launch_bounds__(kPBlock) k_pairs(StepParams P, ParticleArrays 
 
 // ------------------------------------------------------------------ MD sub-stepping
 
-// Coupling forces of substep `sub` at the particles' current positions C (in the order of the
-// step's sorted list S, whose fluid-side solvation force stays frozen), then the substep's
-// reaction record: position, friction and solvation forces over K, and the substep index in
-// the cell's w (the fluid-side solvation force is taken from substep 0's records only).
-__global__ void __launch_bounds__(kPBlock) k_couple_sub(StepParams P, ParticleArrays C, ParticleArrays S,
-                                                        CellIndex ci, const float *__restrict__ rho,
-                                                        const float *__restrict__ jp, ParticleForces pf, int sub,
-                                                        ReactionRecords rec) {
-  // 8 lanes per particle (site::couple8); lane 0, which wrote the forces, writes the records
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int p = (int)(t >> 3), k = (int)(t & 7);
-  if (p >= P.np) return;
-  site::couple8(P, noise_step(P, P.step), p, k, 0xFFu << (threadIdx.x & 24), C, S, ci, rho, jp, pf, sub == 0);
-  if (k != 0) return;
-  const float invK = 1.f / (float)P.substeps;
-  const int r = sub * P.np + p;
-  const int4 c = C.cell[p];
-  rec.cell[r] = make_int4(c.x, c.y, c.z, c.w | (sub << 8));
-  rec.frac[r] = C.frac[p];
-  rec.key[r] = sub * P.np + C.pid[p];
-  const float4 a = pf.fric[p], b = pf.psA[p], d = pf.psB[p];
-  rec.fric[r] = make_float4(a.x * invK, a.y * invK, a.z * invK, 0.f);
-  rec.psA[r] = make_float4(b.x * invK, b.y * invK, b.z * invK, 0.f);
-  rec.psB[r] = make_float4(d.x * invK, d.y * invK, d.z * invK, 0.f);
-}
+// One particle substep: the coupling and the pair forces at the particles' positions C (in the order
+// of the step's sorted list S, whose rows and fluid-side solvation force stay frozen), the substep's
+// reaction record -- position, friction and solvation forces over K, and the substep index in the
+// cell's w (the fluid-side solvation force is taken from substep 0's records only) -- binned for the
+// records' sort, and the update by P.dt = dt / K into D, with the check that each particle is still
+// within one cell of where the step started (the rows of the step rely on it).
+// A block takes 8 particles, 8 lanes each for the coupling (its first two warps) and for the pair
+// forces (the others), which meet in shared memory.  Bound by latency: as three launches on two
+// streams, working in place on a copy of S, a substep of 800 chain beads on 80^3 took 45 us and a
+// lattice step with ten of them 450; this launch takes 18.5 and the step 245.
+constexpr int kSubParticles = 8;
+static_assert(kPBlock == 2 * 8 * kSubParticles, "two groups of 8 lanes per particle");
 
-// Particle update of one substep (P.dt = dt / K), in place, and the check that each particle
-// is still within one cell of where the step started (the cell list of the step relies on it).
-__global__ void k_integrate_sub(StepParams P, ParticleArrays C, ParticleArrays S, ParticleForces pf, unsigned *err) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= P.np) return;
-  site::integrate(P, p, C, C, pf, err);
-  const int4 a = C.cell[p], b = S.cell[p];
-  const int dx = site::min_image_cells(a.x - b.x, P.nx), dy = site::min_image_cells(a.y - b.y, P.ny),
-            dz = site::min_image_cells(a.z - b.z, P.nz);
-  if (dx > 1 || dx < -1 || dy > 1 || dy < -1 || dz > 1 || dz < -1) atomicOr(err, kErrTooFast);
+__global__ void __launch_bounds__(kPBlock) k_substep(StepParams P, ParticleArrays C, ParticleArrays D,
+                                                     ParticleArrays S, CellIndex ci, int pair_reach,
+                                                     const float *__restrict__ rho, const float *__restrict__ jp,
+                                                     const int *__restrict__ bond_start,
+                                                     const int *__restrict__ bond_other,
+                                                     const int *__restrict__ slot_of_id, ParticleForces pf, int sub,
+                                                     ReactionRecords rec, SortScratch rs, unsigned *err) {
+  __shared__ float3 pair[kSubParticles];
+  __shared__ site::CoupleForces coupled[kSubParticles];
+  const int g = (threadIdx.x >> 3) & (kSubParticles - 1), k = threadIdx.x & 7;
+  const int p = blockIdx.x * kSubParticles + g;
+  const unsigned mask = 0xFFu << (threadIdx.x & 24);
+  if (p < P.np) {  // the same for the 8 lanes of a group
+    if (threadIdx.x < 8 * kSubParticles) {
+      const site::CoupleForces F = site::couple_forces(P, noise_step(P, P.step), p, k, mask, C, S, ci, rho, jp, pf,
+                                                       sub == 0, nullptr);
+      if (k == 0) coupled[g] = F;
+    } else {
+      const float3 F = site::pair_forces(P, p, k, mask, C, ci, pair_reach, bond_start, bond_other, slot_of_id, err);
+      if (k == 0) pair[g] = F;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  const int q = blockIdx.x * kSubParticles + threadIdx.x;  // lane t of the first warp finishes particle t
+  const bool valid = threadIdx.x < kSubParticles && q < P.np;
+  int4 c = make_int4(0, 0, 0, 0);
+  const int r = sub * P.np + q;
+  if (valid) {
+    const site::CoupleForces &F = coupled[threadIdx.x];
+    const float invK = 1.f / (float)P.substeps;
+    c = C.cell[q];
+    rec.cell[r] = make_int4(c.x, c.y, c.z, c.w | (sub << 8));
+    rec.frac[r] = C.frac[q];
+    rec.key[r] = sub * P.np + C.pid[q];
+    rec.fric[r] = make_float4(F.fric.x * invK, F.fric.y * invK, F.fric.z * invK, 0.f);
+    rec.psA[r] = make_float4(F.psA.x * invK, F.psA.y * invK, F.psA.z * invK, 0.f);
+    rec.psB[r] = make_float4(F.psB.x * invK, F.psB.y * invK, F.psB.z * invK, 0.f);
+    float4 fsr = F.fsr;
+    if (sub == 0)
+      pf.fsr[q] = fsr;
+    else
+      fsr = pf.fsr[q];
+    const float3 f = pair[threadIdx.x];
+    const float3 total = site::total_force(F.fric, F.psA, F.psB, fsr, make_float4(f.x, f.y, f.z, 0.f));
+    if (sub == P.substeps - 1) pf.total[q] = make_float4(total.x, total.y, total.z, 0.f);
+    const int4 a = site::move_by(P, q, C, D, total, err), b = S.cell[q];
+    const int dx = site::min_image_cells(a.x - b.x, P.nx), dy = site::min_image_cells(a.y - b.y, P.ny),
+              dz = site::min_image_cells(a.z - b.z, P.nz);
+    if (dx > 1 || dx < -1 || dy > 1 || dy < -1 || dz > 1 || dz < -1) atomicOr(err, kErrTooFast);
+  }
+  bin_particle(P, r, valid, c, rs);
 }
 
 __global__ void __launch_bounds__(kPBlock) k_rec_place(int n, SortScratch S, const int *__restrict__ start,
@@ -449,14 +477,12 @@ void launch_pairs(const StepParams &P, const ParticleArrays &pa, CellIndex ci, c
                   cudaStream_t st) {
   k_pairs<<<pgrid(8LL * P.np), kPBlock, 0, st>>>(P, pa, ci, bond_start, bond_other, slot_of_id, pf, err);
 }
-void launch_couple_sub(const StepParams &P, const ParticleArrays &C, const ParticleArrays &S, CellIndex ci,
-                       const float *rho, const float *jp, const ParticleForces &pf, int sub,
-                       const ReactionRecords &rec, cudaStream_t st) {
-  k_couple_sub<<<pgrid(8LL * P.np), kPBlock, 0, st>>>(P, C, S, ci, rho, jp, pf, sub, rec);
-}
-void launch_integrate_sub(const StepParams &P, const ParticleArrays &C, const ParticleArrays &S,
-                          const ParticleForces &pf, unsigned *err, cudaStream_t st) {
-  k_integrate_sub<<<pgrid(P.np), kPBlock, 0, st>>>(P, C, S, pf, err);
+void launch_substep(const StepParams &P, const ParticleArrays &C, const ParticleArrays &D, const ParticleArrays &S,
+                    CellIndex ci, int pair_reach, const float *rho, const float *jp, const int *bond_start,
+                    const int *bond_other, const int *slot_of_id, const ParticleForces &pf, int sub,
+                    const ReactionRecords &rec, const SortScratch &rs, unsigned *err, cudaStream_t st) {
+  k_substep<<<(P.np + kSubParticles - 1) / kSubParticles, kPBlock, 0, st>>>(
+      P, C, D, S, ci, pair_reach, rho, jp, bond_start, bond_other, slot_of_id, pf, sub, rec, rs, err);
 }
 void launch_particle_momentum(const StepParams &P, const ParticleArrays &pa, double *partial, int nblocks,
                               cudaStream_t st) {

@@ -788,19 +788,19 @@ struct NodeState {
   float3 SA, SB;  // sum_i w_i rho_z(r + c_i) c_i
 };
 
-__device__ __forceinline__ NodeState node_state(const StepParams &P, const float *__restrict__ rho, int x, int y,
-                                                int z) {
+__device__ __forceinline__ NodeState node_state(const StepParams &P, const float *__restrict__ rho, const Coord &c) {
   NodeState n;
   const float2 *rho2 = reinterpret_cast<const float2 *>(rho);  // interleaved (rho_A, rho_B)
-  const long long s = site_index(P, x, y, z);
-  n.rA = __ldg(rho2 + s).x;
-  n.rB = __ldg(rho2 + s).y;
+  const NOff o = neighbour_offsets(P, c);
+  const unsigned s32 = (unsigned)site_index(P, c.x, c.y, c.z);
+  const float2 r0 = __ldg(rho2 + s32);
+  n.rA = r0.x;
+  n.rB = r0.y;
   n.SA = make_float3(0.f, 0.f, 0.f);
   n.SB = make_float3(0.f, 0.f, 0.f);
 #pragma unroll
   for (int i = 1; i < kQ; ++i) {
-    const long long nb = site_index(P, wrapi(x + kCx[i], P.nx), wrapi(y + kCy[i], P.ny), wrapi(z + kCz[i], P.nz));
-    const float2 r2 = __ldg(rho2 + nb);
+    const float2 r2 = __ldg(rho2 + (unsigned)((int)s32 + shift(o, kCx[i], kCy[i], kCz[i])));
     const float a = kW[i] * r2.x, b = kW[i] * r2.y;
     n.SA.x += kCx[i] * a; n.SA.y += kCy[i] * a; n.SA.z += kCz[i] * a;
     n.SB.x += kCx[i] * b; n.SB.y += kCy[i] * b; n.SB.z += kCz[i] * b;
@@ -858,19 +858,18 @@ __device__ __forceinline__ void couple_corner(const StepParams &P, int k, int4 c
                                               const float4 *__restrict__ jc = nullptr) {
   const int ox = k & 1, oy = (k >> 1) & 1, oz = (k >> 2) & 1;
   const Coord cc = cell_corner(P, c, k);
-  const int X = cc.x, Y = cc.y, Z = cc.z;
-  const long long s = site_index(P, X, Y, Z);
   float3 j;
   if (jc) {
     const float4 v = __ldg(jc + k);
     j = make_float3(v.x, v.y, v.z);
   } else {
+    const long long s = site_index(P, cc.x, cc.y, cc.z);
     j = make_float3(__ldg(jp + s), __ldg(jp + P.N + s), __ldg(jp + 2 * P.N + s));
   }
-  const NodeState n = node_state(P, rho, X, Y, Z);
+  const NodeState n = node_state(P, rho, cc);
   float3 fA = make_float3(-P.gAB * n.rA * n.SB.x, -P.gAB * n.rA * n.SB.y, -P.gAB * n.rA * n.SB.z);
   float3 fB = make_float3(-P.gBA * n.rB * n.SA.x, -P.gBA * n.rB * n.SA.y, -P.gBA * n.rB * n.SA.z);
-  gather_coupling(P, X, Y, Z, n.rA, n.rB, list, pf, ci, false, fA, fB);
+  if (P.any_lam) gather_coupling(P, cc.x, cc.y, cc.z, n.rA, n.rB, list, pf, ci, false, fA, fB);
   const float rinv = 1.f / (n.rA + n.rB);
   const float w = (ox ? fr.x : 1.f - fr.x) * (oy ? fr.y : 1.f - fr.y) * (oz ? fr.z : 1.f - fr.z);
   S.up.x += w * (j.x + 0.5f * (fA.x + fB.x)) * rinv;
@@ -885,51 +884,76 @@ __device__ __forceinline__ void couple_corner(const StepParams &P, int k, int4 c
   }
 }
 
+// The coupling's forces on one particle.
+struct CoupleForces {
+  float4 fric, psA, psB, fsr;
+};
+
 // Forces from the sums: friction + noise (Eq. NEWTON), solvation (Eq. solvation_kappa), the
 // reaction of the fluid-side solvation force.
-__device__ __forceinline__ void couple_finish(const StepParams &P, unsigned long long step, int p,
-                                              const ParticleArrays &self, const ParticleForces &pf, bool with_fsr,
-                                              const TypeParams &T, float4 v, const CoupleSums &S) {
+__device__ __forceinline__ CoupleForces couple_finish(const StepParams &P, unsigned long long step, int id,
+                                                      const TypeParams &T, float4 v, const CoupleSums &S) {
   float3 R = make_float3(0.f, 0.f, 0.f);
   if (T.noise_amp > 0.f) {
-    const float3 nn = particle_normals(P.seed, step, (unsigned)self.pid[p]);
+    const float3 nn = particle_normals(P.seed, step, (unsigned)id);
     const float amp = T.noise_amp * P.noise_scale;
     R = make_float3(amp * nn.x, amp * nn.y, amp * nn.z);
   }
-  pf.fric[p] = make_float4(-T.gamma * (v.x - S.up.x) + R.x, -T.gamma * (v.y - S.up.y) + R.y,
-                           -T.gamma * (v.z - S.up.z) + R.z, 0.f);
+  CoupleForces F;
+  F.fric = make_float4(-T.gamma * (v.x - S.up.x) + R.x, -T.gamma * (v.y - S.up.y) + R.y,
+                       -T.gamma * (v.z - S.up.z) + R.z, 0.f);
   const float kA = -T.kappa[0] / kCs2, kB = -T.kappa[1] / kCs2;
-  pf.psA[p] = make_float4(kA * S.gA.x, kA * S.gA.y, kA * S.gA.z, 0.f);
-  pf.psB[p] = make_float4(kB * S.gB.x, kB * S.gB.y, kB * S.gB.z, 0.f);
-  if (with_fsr) pf.fsr[p] = make_float4(S.fsr.x, S.fsr.y, S.fsr.z, 0.f);
+  F.psA = make_float4(kA * S.gA.x, kA * S.gA.y, kA * S.gA.z, 0.f);
+  F.psB = make_float4(kB * S.gB.x, kB * S.gB.y, kB * S.gB.z, 0.f);
+  F.fsr = make_float4(S.fsr.x, S.fsr.y, S.fsr.z, 0.f);
+  return F;
 }
 
 // Coupling forces on particle p with 8 lanes per particle: lane k of a group of 8 consecutive
-// lanes takes corner k, the sums are added over the group by shuffles (mask: the group's
-// lanes), and lane 0 writes the forces.  Every lane of the group must call it with the same p.
-// `self` holds the particle's own state; `list` and ci the sorted particles whose fluid-side
-// solvation force enters the coupling velocity (the same arrays, except in the later particle
-// substeps, which keep the list of the step's start).  with_fsr: compute the reaction of the
-// particle's own fluid-side solvation force (else keep the value in pf.fsr).
-__device__ __forceinline__ void couple8(const StepParams &P, unsigned long long step, int p, int k, unsigned mask,
-                                        const ParticleArrays &self, const ParticleArrays &list, CellIndex ci,
-                                        const float *__restrict__ rho, const float *__restrict__ jp,
-                                        const ParticleForces &pf, bool with_fsr = true,
-                                        const float4 *__restrict__ jc = nullptr) {
+// lanes takes corner k and the sums are added over the group by shuffles (mask: the group's
+// lanes); lane 0 of the group returns the forces.  Every lane of the group must call it with the
+// same p.  `self` holds the particle's own state; `list` and ci the sorted particles whose
+// fluid-side solvation force enters the coupling velocity (the same arrays, except in the later
+// particle substeps, which keep the list of the step's start).  with_fsr: compute the reaction of
+// the particle's own fluid-side solvation force (else it is left 0).
+__device__ __forceinline__ CoupleForces couple_forces(const StepParams &P, unsigned long long step, int p, int k,
+                                                      unsigned mask, const ParticleArrays &self,
+                                                      const ParticleArrays &list, CellIndex ci,
+                                                      const float *__restrict__ rho, const float *__restrict__ jp,
+                                                      const ParticleForces &pf, bool with_fsr,
+                                                      const float4 *__restrict__ jc) {
   const int4 c = self.cell[p];
-  const float4 fr = self.frac[p];
+  const float4 fr = self.frac[p], v = self.vel[p];
+  const int id = self.pid[p];
   const TypeParams &Ty = P.types[c.w];
   CoupleSums S{};
-  couple_corner(P, k, c, fr, Ty, list, ci, rho, jp, pf, with_fsr, S, jc ? jc + (long long)self.pid[p] * 8 : nullptr);
+  couple_corner(P, k, c, fr, Ty, list, ci, rho, jp, pf, with_fsr, S, jc ? jc + (long long)id * 8 : nullptr);
   float *x = &S.up.x;  // the 12 sums, contiguous
 #pragma unroll
   for (int off = 4; off > 0; off >>= 1)
 #pragma unroll
     for (int q = 0; q < 12; ++q) x[q] += __shfl_xor_sync(mask, x[q], off);
-  if (k == 0) couple_finish(P, step, p, self, pf, with_fsr, Ty, self.vel[p], S);
+  CoupleForces F{};
+  if (k == 0) F = couple_finish(P, step, id, Ty, v, S);
+  return F;
 }
+
+// couple_forces written to pf by lane 0 of the group.
+__device__ __forceinline__ void couple8(const StepParams &P, unsigned long long step, int p, int k, unsigned mask,
+                                        const ParticleArrays &list, CellIndex ci, const float *__restrict__ rho,
+                                        const float *__restrict__ jp, const ParticleForces &pf,
+                                        const float4 *__restrict__ jc = nullptr) {
+  const CoupleForces F = couple_forces(P, step, p, k, mask, list, list, ci, rho, jp, pf, true, jc);
+  if (k != 0) return;
+  pf.fric[p] = F.fric;
+  pf.psA[p] = F.psA;
+  pf.psB[p] = F.psB;
+  pf.fsr[p] = F.fsr;
+}
+
+// Nearest image of the difference d of two cells of an axis of n (-n < d < n).
 __device__ __forceinline__ int min_image_cells(int d, int n) {
-  d = wrapi(d, n);
+  if (d < 0) d += n;
   return 2 * d > n ? d - n : d;
 }
 
@@ -939,42 +963,35 @@ __device__ __forceinline__ int min_image_cells(int d, int n) {
 // bond_start = no bonds).  Each particle computes its own force (pairs are visited from both
 // ends): no atomics, fixed order.
 //
-// Pair forces on particle p from the particles of one lattice row of the cell index (-dU/dr),
-// accumulated into F.
-__device__ __forceinline__ void pair_row(const StepParams &P, int p, int4 c, float4 fr, int row, bool allx,
-                                         const ParticleArrays &pa, CellIndex ci, float3 &F) {
-  const int m = P.reach;
-  const float Lx = (float)P.nx, Ly = (float)P.ny, Lz = (float)P.nz;
-  const int q0 = ci.row_start[row], q1 = ci.row_start[row + 1];
-  for (int q = q0; q < q1; ++q) {
-    if (q == p) continue;
-    const int4 cq = pa.cell[q];
-    const int dcx = min_image_cells(c.x - cq.x, P.nx);
-    if (!allx && (dcx > m || dcx < -m)) continue;
-    const float4 fq = pa.frac[q];
-    float dx = (float)dcx + (fr.x - fq.x);
-    float dy_ = (float)min_image_cells(c.y - cq.y, P.ny) + (fr.y - fq.y);
-    float dz_ = (float)min_image_cells(c.z - cq.z, P.nz) + (fr.z - fq.z);
-    dx -= Lx * rintf(dx / Lx);
-    dy_ -= Ly * rintf(dy_ / Ly);
-    dz_ -= Lz * rintf(dz_ / Lz);
-    const float r2 = dx * dx + dy_ * dy_ + dz_ * dz_;
-    float fscal = 0.f;  // -dU/dr / r
-    const PairParams &pp = P.pairs[c.w * LBMD_MAX_TYPES + cq.w];
-    if (pp.eps > 0.f && r2 < pp.rc2) {
-      const float sr2 = pp.sigma2 / r2;
-      const float sr6 = sr2 * sr2 * sr2;
-      fscal += 24.f * pp.eps * (2.f * sr6 * sr6 - sr6) / r2;
-    }
-    const float qq = fr.w * fq.w;
-    if (P.dh_lB != 0.f && qq != 0.f && r2 < P.dh_rc2) {
-      const float r = sqrtf(r2);
-      fscal += qq * P.dh_lB * expf(-P.dh_kappa * r) * (1.f / r2 + P.dh_kappa / r) / r;
-    }
-    F.x += fscal * dx;
-    F.y += fscal * dy_;
-    F.z += fscal * dz_;
+// Pair force (-dU/dr) on a particle in cell c at fr from the one in cell cq at fq, added to F (allx:
+// the search covers the whole x axis, else cells further than m away in x are skipped).
+__device__ __forceinline__ void pair_force(const StepParams &P, int m, int4 c, float4 fr, int4 cq, float4 fq,
+                                           bool allx, float3 &F) {
+  const int dcx = min_image_cells(c.x - cq.x, P.nx);
+  if (!allx && (dcx > m || dcx < -m)) return;
+  // the fractions can take a nearest-image pair of cells past half the box: one box back (such a
+  // pair is in range only of lattices a few cells wide)
+  auto nearest = [](float d, float n) { return d > 0.5f * n ? d - n : d < -0.5f * n ? d + n : d; };
+  const float dx = nearest((float)dcx + (fr.x - fq.x), (float)P.nx);
+  const float dy_ = nearest((float)min_image_cells(c.y - cq.y, P.ny) + (fr.y - fq.y), (float)P.ny);
+  const float dz_ = nearest((float)min_image_cells(c.z - cq.z, P.nz) + (fr.z - fq.z), (float)P.nz);
+  const float r2 = dx * dx + dy_ * dy_ + dz_ * dz_;
+  float fscal = 0.f;  // -dU/dr / r
+  const PairParams &pp = P.pairs[c.w * LBMD_MAX_TYPES + cq.w];
+  if (pp.eps > 0.f && r2 < pp.rc2) {
+    const float sr2 = pp.sigma2 / r2;
+    const float sr6 = sr2 * sr2 * sr2;
+    fscal += 24.f * pp.eps * (2.f * sr6 * sr6 - sr6) / r2;
   }
+  const float qq = fr.w * fq.w;
+  if (P.dh_lB != 0.f && qq != 0.f && r2 < P.dh_rc2) {
+    const float r = sqrtf(r2);
+    fscal += qq * P.dh_lB * expf(-P.dh_kappa * r) * (1.f / r2 + P.dh_kappa / r) / r;
+  }
+  if (fscal == 0.f) return;
+  F.x += fscal * dx;
+  F.y += fscal * dy_;
+  F.z += fscal * dz_;
 }
 
 // Bond forces on particle p (FENE or harmonic), accumulated into F; a FENE bond stretched to
@@ -1014,27 +1031,69 @@ __device__ __forceinline__ void bond_forces(const StepParams &P, int p, int4 c, 
 }
 
 // Pair and bonded forces of particle p with 8 lanes per particle: lane k of a group of 8
-// consecutive lanes scans the rows k, k + 8, ... of the (2 reach + 1)^2 rows around the
-// particle (the whole axis where the lattice is narrower), the forces are added over the group
-// by shuffles (mask: the group's lanes), lane 0 adds the bonds and writes.  Every lane of the
-// group must call it with the same p.
-__device__ __forceinline__ void pairs8(const StepParams &P, int p, int k, unsigned mask, const ParticleArrays &pa,
-                                       CellIndex ci, const int *__restrict__ bond_start,
-                                       const int *__restrict__ bond_other, const int *__restrict__ slot_of_id,
-                                       const ParticleForces &pf, unsigned *err) {
+// consecutive lanes scans the rows k, k + 8, ... of the (2 m + 1)^2 rows around the
+// particle (m cells of reach; the whole axis where the lattice is narrower), the forces are added over the group
+// by shuffles (mask: the group's lanes), lane 0 adds the bonds and returns the sum.  Every lane of
+// the group must call it with the same p.
+// Bound by latency: a lane's rows are few and mostly empty, so it looks up the limits of several
+// rows at once, and loads a particle of a row while it works on the one before (64^3 with 1000
+// particles: 8.6 -> 6.3 us, most of it the launch; ten substeps of 800 chain beads with 81 rows
+// each: 34 us before, together with the coupling 26 after).
+constexpr int kPairRows = 6;  // rows a lane looks up at once
+
+__device__ __forceinline__ float3 pair_forces(const StepParams &P, int p, int k, unsigned mask,
+                                              const ParticleArrays &pa, CellIndex ci, int m,
+                                              const int *__restrict__ bond_start,
+                                              const int *__restrict__ bond_other,
+                                              const int *__restrict__ slot_of_id, unsigned *err) {
   const int4 c = pa.cell[p];
   const float4 fr = pa.frac[p];
   float3 F = make_float3(0.f, 0.f, 0.f);
-  const int m = P.reach;
   if (m > 0) {
     const bool allz = 2 * m + 1 >= P.nz, ally = 2 * m + 1 >= P.ny, allx = 2 * m + 1 >= P.nx;
-    const int z0 = allz ? 0 : -m, nzw = allz ? P.nz : 2 * m + 1;
-    const int y0 = ally ? 0 : -m, nyw = ally ? P.ny : 2 * m + 1;
-    for (int w = k; w < nzw * nyw; w += 8) {
-      const int dz = z0 + w / nyw, dy = y0 + w % nyw;
-      const int cz = allz ? dz : wrapi(c.z + dz, P.nz);
-      const int cy = ally ? dy : wrapi(c.y + dy, P.ny);
-      pair_row(P, p, c, fr, cz * P.ny + cy, allx, pa, ci, F);
+    const int z0 = allz ? 0 : c.z - m, nzw = allz ? P.nz : 2 * m + 1;
+    const int y0 = ally ? 0 : c.y - m, nyw = ally ? P.ny : 2 * m + 1;
+    for (int w0 = k; w0 < nzw * nyw; w0 += 8 * kPairRows) {
+      int q0[kPairRows], q1[kPairRows];
+      unsigned some = 0;  // the rows that hold particles
+#pragma unroll
+      for (int j = 0; j < kPairRows; ++j) {
+        const int w = w0 + 8 * j;
+        q0[j] = q1[j] = 0;
+        if (w < nzw * nyw) {
+          const int dz = w / nyw;
+          int z = z0 + dz, y = y0 + (w - dz * nyw);  // less than a lattice outside (2 m + 1 < n there)
+          z += z < 0 ? P.nz : z >= P.nz ? -P.nz : 0;
+          y += y < 0 ? P.ny : y >= P.ny ? -P.ny : 0;
+          const int *start = ci.row_start + (z * P.ny + y);
+          q0[j] = start[0];
+          q1[j] = start[1];
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < kPairRows; ++j) some |= (q0[j] < q1[j] ? 1u : 0u) << j;
+      while (some) {
+        const int row = __ffs(some) - 1;
+        some &= some - 1;
+        int q = 0, e = 0;
+#pragma unroll
+        for (int j = 0; j < kPairRows; ++j)
+          if (j == row) {
+            q = q0[j];
+            e = q1[j];
+          }
+        int4 cn = pa.cell[q];
+        float4 fn = pa.frac[q];
+        for (; q < e; ++q) {
+          const int4 cq = cn;
+          const float4 fq = fn;
+          if (q + 1 < e) {
+            cn = pa.cell[q + 1];
+            fn = pa.frac[q + 1];
+          }
+          if (q != p) pair_force(P, m, c, fr, cq, fq, allx, F);
+        }
+      }
     }
   }
 #pragma unroll
@@ -1043,30 +1102,32 @@ __device__ __forceinline__ void pairs8(const StepParams &P, int p, int k, unsign
     F.y += __shfl_xor_sync(mask, F.y, off);
     F.z += __shfl_xor_sync(mask, F.z, off);
   }
-  if (k == 0) {
-    if (bond_start) bond_forces(P, p, c, fr, pa, bond_start, bond_other, slot_of_id, err, F);
-    pf.pair[p] = make_float4(F.x, F.y, F.z, 0.f);
-  }
+  if (k == 0 && bond_start) bond_forces(P, p, c, fr, pa, bond_start, bond_other, slot_of_id, err, F);
+  return F;
 }
 
-// Particle update of slot p: v += F dt / m, x += v dt, periodic wrap kept as (cell,
+// pair_forces written to pf by lane 0 of the group.
+__device__ __forceinline__ void pairs8(const StepParams &P, int p, int k, unsigned mask, const ParticleArrays &pa,
+                                       CellIndex ci, const int *__restrict__ bond_start,
+                                       const int *__restrict__ bond_other, const int *__restrict__ slot_of_id,
+                                       const ParticleForces &pf, unsigned *err) {
+  const float3 F = pair_forces(P, p, k, mask, pa, ci, P.reach, bond_start, bond_other, slot_of_id, err);
+  if (k == 0) pf.pair[p] = make_float4(F.x, F.y, F.z, 0.f);
+}
+
+// Particle update of slot p by the force F: v += F dt / m, x += v dt, periodic wrap kept as (cell,
 // fraction).  Reads src, writes dst (the same arrays for an update in place) and returns the new
 // cell, which is inside the lattice.
-__device__ __forceinline__ int4 integrate(const StepParams &P, int p, const ParticleArrays &src,
-                                          const ParticleArrays &dst, const ParticleForces &pf, unsigned *err) {
+__device__ __forceinline__ int4 move_by(const StepParams &P, int p, const ParticleArrays &src,
+                                        const ParticleArrays &dst, float3 F, unsigned *err) {
   int4 c = src.cell[p];
   float4 fr = src.frac[p];
   float4 v = src.vel[p];
   if (dst.pid != src.pid) dst.pid[p] = src.pid[p];
   const TypeParams &T = P.types[c.w];
-  const float4 a = pf.fric[p], b = pf.psA[p], d = pf.psB[p], e = pf.fsr[p], g = pf.pair[p];
-  const float Fx = a.x + b.x + d.x + e.x + g.x;
-  const float Fy = a.y + b.y + d.y + e.y + g.y;
-  const float Fz = a.z + b.z + d.z + e.z + g.z;
-  pf.total[p] = make_float4(Fx, Fy, Fz, 0.f);
-  v.x += Fx * P.dt * T.inv_mass;
-  v.y += Fy * P.dt * T.inv_mass;
-  v.z += Fz * P.dt * T.inv_mass;
+  v.x += F.x * P.dt * T.inv_mass;
+  v.y += F.y * P.dt * T.inv_mass;
+  v.z += F.z * P.dt * T.inv_mass;
   float nx_ = fr.x + v.x * P.dt, ny_ = fr.y + v.y * P.dt, nz_ = fr.z + v.z * P.dt;
   const float lim = 1.0e6f;
   if (!(fabsf(nx_) < lim && fabsf(ny_) < lim && fabsf(nz_) < lim)) {
@@ -1089,6 +1150,20 @@ __device__ __forceinline__ int4 integrate(const StepParams &P, int p, const Part
   dst.frac[p] = make_float4(nx_, ny_, nz_, fr.w);
   dst.vel[p] = v;
   return c;
+}
+
+// The total of a particle's forces.
+__device__ __forceinline__ float3 total_force(float4 fric, float4 psA, float4 psB, float4 fsr, float4 pair) {
+  return make_float3(fric.x + psA.x + psB.x + fsr.x + pair.x, fric.y + psA.y + psB.y + fsr.y + pair.y,
+                     fric.z + psA.z + psB.z + fsr.z + pair.z);
+}
+
+// Particle update of slot p by the forces in pf; writes their total there.
+__device__ __forceinline__ int4 integrate(const StepParams &P, int p, const ParticleArrays &src,
+                                          const ParticleArrays &dst, const ParticleForces &pf, unsigned *err) {
+  const float3 F = total_force(pf.fric[p], pf.psA[p], pf.psB[p], pf.fsr[p], pf.pair[p]);
+  pf.total[p] = make_float4(F.x, F.y, F.z, 0.f);
+  return move_by(P, p, src, dst, F, err);
 }
 
 // ------------------------------------------------------------------ row scan

@@ -38,10 +38,10 @@ struct lbmd_ctx {
   // update.  The sort writes the buffers of the step before (pa[1 - pcur], row_start[1 - pcur]),
   // whose last reader, that step's lattice update, the coupling came after.  st waits for the sort
   // (ev_sorted) at the end of a launch sequence or before the next coupling; sort_pending: it has
-  // not yet.  ev_int and ev_pairs order the substeps of MD sub-stepping; the sort of the particles
-  // that took them starts when they and the sort of their records are done (ev_sub).
+  // not yet.  ev_int forks side from st; with MD sub-stepping the substeps run on st, and the sort of
+  // the particles starts when the substeps and the sort of their records are done (ev_sub).
   cudaStream_t side = nullptr;
-  cudaEvent_t ev_int = nullptr, ev_sorted = nullptr, ev_pairs = nullptr, ev_coupled = nullptr, ev_sub = nullptr;
+  cudaEvent_t ev_int = nullptr, ev_sorted = nullptr, ev_coupled = nullptr, ev_sub = nullptr;
   bool sort_pending = false;
   // one pass with particles: ev_integrated (the particle update done, on side) orders the boundary
   // kernel, which forms the next step's corner j' (jc) at the updated positions, after it
@@ -469,11 +469,11 @@ int enqueue_drift(lbmd_ctx *c, int set_ref) {
 namespace {
 
 // MD sub-stepping of one lattice step (K = P.substeps > 1): the sorted particles S of the step's
-// start stay frozen (cell list, fluid-side solvation force); a working copy C takes K substeps
-// of coupling forces (writing one momentum-return record per particle and substep), pair
-// forces over S's rows with one more cell of reach, and updates of dt / K; the records are
-// then sorted by row for the update's node-side gather.  On return C is the particle state and
-// (pa, pf, ci) describe the records.
+// start stay frozen (cell list, fluid-side solvation force); each of the K substeps, one launch,
+// reads the particles' positions from one buffer and writes them to another: coupling forces (one
+// momentum-return record per particle and substep), pair forces over S's rows with one more cell
+// of reach, updates of dt / K.  The records are then sorted by row for the update's node-side
+// gather.  On return pt is the particle state and (pa, pf, ci) describe the records.
 int substep_particles(lbmd_ctx *c, ParticleArrays &pa, ParticleForces &pf, CellIndex &ci) {
   const StepParams &P = c->P;
   const int K = P.substeps, np = P.np;
@@ -482,41 +482,31 @@ int substep_particles(lbmd_ctx *c, ParticleArrays &pa, ParticleForces &pf, CellI
   int r = ensure_records(c, nrec);
   if (r) return r;
   const ParticleArrays &S = c->pa[c->pcur];
-  const ParticleArrays &C = c->pt;
-  CK(cudaMemcpyAsync(C.cell, S.cell, sizeof(int4) * np, cudaMemcpyDeviceToDevice, c->st), "copy particles");
-  CK(cudaMemcpyAsync(C.frac, S.frac, sizeof(float4) * np, cudaMemcpyDeviceToDevice, c->st), "copy particles");
-  CK(cudaMemcpyAsync(C.vel, S.vel, sizeof(float4) * np, cudaMemcpyDeviceToDevice, c->st), "copy particles");
-  CK(cudaMemcpyAsync(C.pid, S.pid, sizeof(int) * np, cudaMemcpyDeviceToDevice, c->st), "copy particles");
+  // the substeps alternate between pt, which takes the last one, and the buffer the particles' sort
+  // overwrites later; the order is S's throughout, and so are the ids until pt gets its own
+  const ParticleArrays &other = c->pa[1 - c->pcur];
+  const ParticleArrays work[2] = {{c->pt.cell, c->pt.frac, c->pt.vel, S.pid},
+                                  {other.cell, other.frac, other.vel, S.pid}};
   const CellIndex rows{c->row_start[c->pcur]};
+  SortScratch rs = c->rec_sort;
+  rs.row_count = c->sort.row_count;
+  rs.block_count = c->sort.block_count;
   for (int sub = 0; sub < K; ++sub) {
     StepParams Q = P;
     Q.step = P.step * (unsigned long long)K + (unsigned long long)sub;
     Q.step_mul = (unsigned long long)K;
     Q.dt = P.dt / (float)K;
-    // the pair forces (side stream) and the coupling read the same positions and write
-    // different forces; the update of the substep waits for both
-    CK(cudaEventRecord(c->ev_int, c->st), "event");
-    CK(cudaStreamWaitEvent(c->side, c->ev_int, 0), "stream wait");
-    StepParams Qp = Q;
-    Qp.reach = P.reach + 1;  // particles may have left their row by one cell
-    launch_pairs(Qp, C, rows, c->nbonds ? c->bond_start : nullptr, c->bond_other, c->slot_of_id, c->pf, c->err,
-                 c->side);
-    CK(cudaEventRecord(c->ev_pairs, c->side), "event");
-    launch_couple_sub(Q, C, S, rows, c->rho_buf[c->cur], c->jp, c->pf, sub, c->rec[0], c->st);
-    CK(cudaStreamWaitEvent(c->st, c->ev_pairs, 0), "stream wait");
-    launch_integrate_sub(Q, C, S, c->pf, c->err, c->st);
-    if ((r = launched(c, "particle substep", 3))) return r;
+    const ParticleArrays &from = sub == 0 ? S : work[(K - sub) & 1];
+    const ParticleArrays &to = sub == K - 1 ? c->pt : work[(K - 1 - sub) & 1];
+    // (pair reach: particles may have left their row by one cell)
+    launch_substep(Q, from, to, S, rows, P.reach > 0 ? P.reach + 1 : 0, c->rho_buf[c->cur], c->jp,
+                   c->nbonds ? c->bond_start : nullptr, c->bond_other, c->slot_of_id, c->pf, sub, c->rec[0], rs,
+                   c->err, c->st);
+    if ((r = launched(c, "particle substep"))) return r;
   }
-  // sort the records by (row, x cell, substep * np + id): the same counting sort as particles
-  StepParams R = P;
-  R.np = (int)nrec;
-  const ParticleArrays view{c->rec[0].cell, c->rec[0].frac, nullptr, c->rec[0].key};
-  SortScratch rs = c->rec_sort;
-  rs.row_count = c->sort.row_count;
-  rs.block_count = c->sort.block_count;
-  launch_bin(R, view, rs, c->err, c->st);
-  launch_rec_place(P, R.np, rs, c->rec[0], c->rec[1], c->rec_row_start, c->st);
-  if ((r = launched(c, "record sort", 4))) return r;
+  // sort the (binned) records by (row, x cell, substep * np + id): the same counting sort as particles
+  launch_rec_place(P, (int)nrec, rs, c->rec[0], c->rec[1], c->rec_row_start, c->st);
+  if ((r = launched(c, "record sort", 3))) return r;
   pa = ParticleArrays{c->rec[1].cell, c->rec[1].frac, nullptr, nullptr};
   pf = c->pf;
   pf.fric = c->rec[1].fric;
@@ -796,7 +786,6 @@ int lbmd_create(const lbmd_params *prm, void *stream, lbmd_ctx **out, unsigned *
   if ((e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&c->ev_int, cudaEventDisableTiming)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&c->ev_sorted, cudaEventDisableTiming)) != cudaSuccess ||
-      (e = cudaEventCreateWithFlags(&c->ev_pairs, cudaEventDisableTiming)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&c->ev_coupled, cudaEventDisableTiming)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&c->ev_sub, cudaEventDisableTiming)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&c->ev_integrated, cudaEventDisableTiming)) != cudaSuccess) {
@@ -829,7 +818,6 @@ void lbmd_destroy(lbmd_ctx *c) {
   }
   if (c->ev_int) cudaEventDestroy(c->ev_int);
   if (c->ev_sorted) cudaEventDestroy(c->ev_sorted);
-  if (c->ev_pairs) cudaEventDestroy(c->ev_pairs);
   if (c->ev_coupled) cudaEventDestroy(c->ev_coupled);
   if (c->ev_sub) cudaEventDestroy(c->ev_sub);
   if (c->ev_integrated) cudaEventDestroy(c->ev_integrated);

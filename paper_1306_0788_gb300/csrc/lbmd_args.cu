@@ -123,6 +123,7 @@ int apply_types(StepParams &P, double kT, double dt, int ntypes, const lbmd_ptyp
   if (ntypes < 1 || ntypes > LBMD_MAX_TYPES || !types || npairs < 0 || (npairs > 0 && !pairs))
     return why = "bad type table", LBMD_E_INVALID_ARG;
   StepParams Q = P;  // applied only if every entry is valid
+  Q.any_lam = false;
   for (int t = 0; t < ntypes; ++t) {
     const lbmd_ptype &T = types[t];
     if (!(T.mass > 0.0) || !(T.gamma >= 0.0)) return why = "mass must be > 0, gamma >= 0", LBMD_E_INVALID_ARG;
@@ -131,6 +132,7 @@ int apply_types(StepParams &P, double kT, double dt, int ntypes, const lbmd_ptyp
     D.kappa[1] = (float)T.kappa_B;
     D.lam[0] = (float)T.lambda_A;
     D.lam[1] = (float)T.lambda_B;
+    Q.any_lam = Q.any_lam || D.lam[0] != 0.f || D.lam[1] != 0.f;
     D.gamma = (float)T.gamma;
     D.inv_mass = (float)(1.0 / T.mass);
     D.mass = (float)T.mass;
