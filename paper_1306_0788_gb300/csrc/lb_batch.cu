@@ -52,7 +52,7 @@ struct RepLayout {   // per slot, written by the host at each repack
   int tile0;         // first tile of the replica in the tile table
   int row0;          // first row of the replica in the shared row space (-1: no particles)
   int p0;            // first slot of the replica in the particle arrays
-  int pad;
+  int bits0;         // first word of the replica in the node bits
 };
 
 struct BatchDev {
@@ -69,6 +69,8 @@ struct BatchDev {
   ParticleArrays S;      // the same particles sorted by (row, x cell, id) during a step
   ParticleForces pf;     // forces, indexed like S (and like U after the update)
   int *row_of, *row_count, *row_start, *row_cursor, *bsum, *perm;
+  unsigned *node_bits;   // [nwords] CellIndex::node_bits of the replicas with particles
+  int nwords;
   double *tile_sums;     // [ntiles][5] FP64 sums of the drift check
   double *drift;         // [max_slots][10]: reference totals [5], last check {step, dA, dB, dP, n}
 };
@@ -90,7 +92,7 @@ struct TileCtx {
   float *rest_out;
   float *rho, *jp;
   unsigned *err;
-  const int *row_start;  // the replica's rows in the shared row space; NULL: no particle coupling
+  CellIndex ci;          // the replica's rows and node bits; row_start NULL: no particle coupling
   long long base;        // first site of the tile
   unsigned long long step;  // the replica's step count (noise counter)
   ParticleArrays pa;     // the sorted particles of the batch
@@ -128,7 +130,7 @@ __device__ __forceinline__ void fill_tile(TileCtx<T> &c, const BatchDev *__restr
     c.rho = R.rho;
     c.jp = R.P.np > 0 ? R.jp : nullptr;
     c.err = &B->state[slot].err;
-    c.row_start = (!tuning && R.P.np > 0) ? B->row_start + L.row0 : nullptr;
+    c.ci = CellIndex{(!tuning && R.P.np > 0) ? B->row_start + L.row0 : nullptr, B->node_bits + L.bits0};
     c.base = (long long)(t - L.tile0) * B->tile_sites;
     c.step = B->state[slot].step;
     c.pa = B->S;
@@ -190,12 +192,12 @@ __global__ void __launch_bounds__(kBThreads, kMinBlocks) kb_collide(const BatchD
     for (int k = threadIdx.x; k < ts; k += kBThreads) {
       const long long s = c.base + k;
       if (s >= c.P.N) break;
-      if (c.row_start)
-        site::collide<T, true, kMRT>(c.P, s, c.step, c.fin, c.fout, c.rho, c.pa, c.pf, CellIndex{c.row_start},
-                                     c.err, c.rest_in, c.rest_out);
+      if (c.ci.row_start)
+        site::collide<T, true, kMRT>(c.P, s, c.step, c.fin, c.fout, c.rho, c.pa, c.pf, c.ci, c.err, c.rest_in,
+                                     c.rest_out);
       else
-        site::collide<T, false, kMRT>(c.P, s, c.step, c.fin, c.fout, c.rho, c.pa, c.pf, CellIndex{nullptr},
-                                      c.err, c.rest_in, c.rest_out);
+        site::collide<T, false, kMRT>(c.P, s, c.step, c.fin, c.fout, c.rho, c.pa, c.pf, c.ci, c.err, c.rest_in,
+                                      c.rest_out);
     }
     __syncthreads();  // the next context is complete; this one is free for the tile after it
     t = tn;
@@ -204,8 +206,11 @@ __global__ void __launch_bounds__(kBThreads, kMinBlocks) kb_collide(const BatchD
 
 // ------------------------------------------------------------------ particle sort
 
+// (also clears the node bits, which kb_permute sets anew)
 __global__ void __launch_bounds__(kBPThreads) kb_bin(const BatchDev *__restrict__ B) {
-  const int np = B->np;
+  const int np = B->np, nwords = B->nwords;
+  unsigned *bits = B->node_bits;
+  for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < nwords; w += gridDim.x * blockDim.x) bits[w] = 0u;
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < np; p += gridDim.x * blockDim.x) {
     const int slot = B->pslot[p];
     const StepParams &P = B->rep[slot].P;
@@ -330,12 +335,15 @@ __global__ void __launch_bounds__(kBPThreads) kb_row_sort(const BatchDev *__rest
 __global__ void __launch_bounds__(kBPThreads) kb_permute(const BatchDev *__restrict__ B) {
   const int np = B->np;
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < np; j += gridDim.x * blockDim.x) {
-    const int p = B->perm[j];
-    B->S.cell[j] = B->U.cell[p];
+    const int p = B->perm[j], slot = B->pslot[j];
+    const int4 c = B->U.cell[p];
+    unsigned *bits = B->node_bits + B->lay[slot].bits0;
+    site::for_corner_bits(B->rep[slot].P, c, [&](long long w, unsigned b) { atomicOr(bits + w, b); });
+    B->S.cell[j] = c;
     B->S.frac[j] = B->U.frac[p];
     B->S.vel[j] = B->U.vel[p];
     B->S.pid[j] = B->U.pid[p];
-    if (B->left[B->pslot[j]] <= 0) B->pf.fric[j] = B->pf.total[p];
+    if (B->left[slot] <= 0) B->pf.fric[j] = B->pf.total[p];
   }
 }
 
@@ -351,7 +359,7 @@ __global__ void __launch_bounds__(kBPThreads) kb_couple(const BatchDev *__restri
     const int slot = B->pslot[p];
     if (B->left[slot] <= 0) continue;
     const RepDev &R = B->rep[slot];
-    const CellIndex ci{B->row_start + B->lay[slot].row0};
+    const CellIndex ci{B->row_start + B->lay[slot].row0, nullptr};
     site::couple8(R.P, B->state[slot].step, p, k, mask, B->S, ci, R.rho, R.jp, B->pf);
   }
 }
@@ -366,7 +374,7 @@ __global__ void __launch_bounds__(kBPThreads) kb_pairs(const BatchDev *__restric
     const int slot = B->pslot[p];
     if (B->left[slot] <= 0) continue;
     const RepDev &R = B->rep[slot];
-    const CellIndex ci{B->row_start + B->lay[slot].row0};
+    const CellIndex ci{B->row_start + B->lay[slot].row0, nullptr};
     site::pairs8(R.P, p, k, mask, B->S, ci, nullptr, nullptr, nullptr, B->pf, &B->state[slot].err);
   }
 }
@@ -606,6 +614,7 @@ struct lbmd_batch {
   int *d_pslot = nullptr;
   int rcap = 0;  // capacity of the row arrays (rows + 1)
   int bcap = 0;  // capacity of the block sums
+  int wcap = 0;  // capacity of the node bits (words)
   double *diag_partial = nullptr, *diag_out = nullptr;
   int diag_cap = 0;
   double *d_drift = nullptr;  // [max_slots][10] (BatchDev::drift)
@@ -847,15 +856,23 @@ int repack(lbmd_batch *b) {
       BK(cudaMemcpyAsync(b->d_pslot, pslot.data(), sizeof(int) * np, cudaMemcpyHostToDevice, b->st), "upload pslot");
   }
   // rows (replicas with particles only)
-  int nrows = 0;
+  int nrows = 0, nwords = 0;
   for (int s : act) {
     Slot &sl = b->slots[s];
     if (sl.np > 0) {
       sl.lay.row0 = nrows;
+      sl.lay.bits0 = nwords;
       nrows += sl.P.nrows;
+      nwords += sl.P.nrows * node_words(sl.P.nx);
     } else {
-      sl.lay.row0 = 0;
+      sl.lay.row0 = sl.lay.bits0 = 0;
     }
+  }
+  if (nwords > b->wcap) {
+    pfree(b, b->hb.node_bits);
+    b->wcap = 0;
+    BK(palloc(b, &b->hb.node_bits, nwords + nwords / 4), "node bits");
+    b->wcap = nwords + nwords / 4;
   }
   const int nbs = site::kScanRows;
   const int nblk = (nrows + nbs - 1) / nbs;
@@ -883,6 +900,7 @@ int repack(lbmd_batch *b) {
   b->hb.nrep = (int)act.size();
   b->hb.np = np;
   b->hb.nrows = nrows;
+  b->hb.nwords = nwords;
   b->hb.pslot = b->d_pslot;
   r = upload_tables(b);
   if (r) return r;
@@ -1021,6 +1039,7 @@ void lbmd_batch_destroy(lbmd_batch *b) {
   free_particle_set(b, b->hb.U); free_particle_set(b, b->hb.S); free_forces(b, b->hb.pf);
   pfree(b, b->hb.row_of); pfree(b, b->hb.perm); pfree(b, b->d_pslot);
   pfree(b, b->hb.row_count); pfree(b, b->hb.row_start); pfree(b, b->hb.row_cursor); pfree(b, b->hb.bsum);
+  pfree(b, b->hb.node_bits);
   pfree(b, b->d_tile_slot);
   cudaStreamSynchronize(b->st);
   if (b->pool) cudaMemPoolDestroy(b->pool);

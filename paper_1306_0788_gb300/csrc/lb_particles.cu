@@ -66,12 +66,22 @@ __global__ void __launch_bounds__(kPBlock) k_bin(StepParams P, ParticleArrays pa
   bin_particle(P, p, valid, c, S);
 }
 
+__device__ __forceinline__ void set_node_bits(const StepParams &P, int4 c, unsigned *node_bits) {
+  site::for_corner_bits(P, c, [&](long long w, unsigned bits) { atomicOr(node_bits + w, bits); });
+}
+__device__ __forceinline__ void clear_node_bits(const StepParams &P, int4 c, unsigned *node_bits) {
+  site::for_corner_bits(P, c, [&](long long w, unsigned) { node_bits[w] = 0u; });
+}
+
 // Particle update (site::integrate) from src into dst, in the same order, and the bin pass of the
-// sort that follows it.
+// sort that follows it.  The nodes of the cells `marked` are cleared in node_bits.
 __global__ void __launch_bounds__(kPBlock) k_integrate_bin(StepParams P, ParticleArrays src, ParticleArrays dst,
-                                                           ParticleForces pf, SortScratch S, unsigned *err) {
+                                                           ParticleForces pf, SortScratch S,
+                                                           const int4 *__restrict__ marked,
+                                                           unsigned *__restrict__ node_bits, unsigned *err) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   const bool valid = p < P.np;
+  if (valid) clear_node_bits(P, marked[p], node_bits);
   bin_particle(P, p, valid, valid ? site::integrate(P, p, src, dst, pf, err) : make_int4(0, 0, 0, 0), S);
 }
 
@@ -125,22 +135,25 @@ __device__ __forceinline__ int placed_slot(int j, const SortScratch &S, const in
   return slot;
 }
 
-__device__ __forceinline__ void move_particle(const ParticleArrays &src, int p, const ParticleArrays &dst, int slot,
-                                              int *__restrict__ slot_of_id) {
+__device__ __forceinline__ void move_particle(const StepParams &P, const ParticleArrays &src, int p,
+                                              const ParticleArrays &dst, int slot, int *__restrict__ slot_of_id,
+                                              unsigned *__restrict__ node_bits) {
   const int id = src.pid[p];
-  dst.cell[slot] = src.cell[p];
+  const int4 c = src.cell[p];
+  if (node_bits) set_node_bits(P, c, node_bits);
+  dst.cell[slot] = c;
   dst.frac[slot] = src.frac[p];
   dst.vel[slot] = src.vel[p];
   dst.pid[slot] = id;
   slot_of_id[id] = slot;
 }
 
-__global__ void __launch_bounds__(kPBlock) k_place(int np, SortScratch S, const int *__restrict__ start,
+__global__ void __launch_bounds__(kPBlock) k_place(StepParams P, SortScratch S, const int *__restrict__ start,
                                                    ParticleArrays src, ParticleArrays dst,
-                                                   int *__restrict__ slot_of_id) {
+                                                   int *__restrict__ slot_of_id, unsigned *__restrict__ node_bits) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= np) return;
-  move_particle(src, S.perm[j], dst, placed_slot(j, S, start), slot_of_id);
+  if (j >= P.np) return;
+  move_particle(P, src, S.perm[j], dst, placed_slot(j, S, start), slot_of_id, node_bits);
 }
 
 // The particle update (kUpdate) and the whole sort of a small system in one block, the counters,
@@ -159,7 +172,7 @@ template <bool kUpdate>
 __global__ void __launch_bounds__(kSmallThreads) k_sort_small(StepParams P, ParticleArrays src, ParticleArrays mid,
                                                               ParticleForces pf, ParticleArrays dst,
                                                               int *__restrict__ start, int *__restrict__ slot_of_id,
-                                                              unsigned *err) {
+                                                              unsigned *__restrict__ node_bits, unsigned *err) {
   extern __shared__ SortKey small_keys[];
   __shared__ int wt[kSmallThreads / 32];
   const int np = P.np, nrows = P.nrows;
@@ -173,6 +186,9 @@ __global__ void __launch_bounds__(kSmallThreads) k_sort_small(StepParams P, Part
   for (int p = threadIdx.x; p < np; p += kSmallThreads) {
     int4 c;
     if (kUpdate) {
+      // dst still holds the particles whose nodes are set; it and the bits are written after the
+      // barriers below
+      clear_node_bits(P, dst.cell[p], node_bits);
       c = site::integrate(P, p, src, mid, pf, err);
     } else {
       c = mid.cell[p];
@@ -211,7 +227,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_sort_small(StepParams P, Part
     const SortKey mine = key[p];
     int slot = b;
     for (int q = b; q < e; ++q) slot += key[list[q]] < mine;
-    move_particle(mid, p, dst, slot, slot_of_id);  // (this thread wrote entry p of mid)
+    move_particle(P, mid, p, dst, slot, slot_of_id, node_bits);  // (this thread wrote entry p of mid)
   }
 }
 
@@ -283,7 +299,13 @@ __global__ void __launch_bounds__(kPBlock) k_substep(StepParams P, ParticleArray
                                                      const int *__restrict__ bond_start,
                                                      const int *__restrict__ bond_other,
                                                      const int *__restrict__ slot_of_id, ParticleForces pf, int sub,
-                                                     ReactionRecords rec, SortScratch rs, unsigned *err) {
+                                                     ReactionRecords rec, SortScratch rs,
+                                                     unsigned *__restrict__ node_bits, unsigned *err) {
+  if (sub == 0) {  // the node bits the last step's records set; the placing of this step's follows
+    const long long n = (long long)P.nrows * node_words(P.nx);
+    for (long long w = (long long)blockIdx.x * kPBlock + threadIdx.x; w < n; w += (long long)gridDim.x * kPBlock)
+      node_bits[w] = 0u;
+  }
   __shared__ float3 pair[kSubParticles];
   __shared__ site::CoupleForces coupled[kSubParticles];
   const int g = (threadIdx.x >> 3) & (kSubParticles - 1), k = threadIdx.x & 7;
@@ -331,14 +353,16 @@ __global__ void __launch_bounds__(kPBlock) k_substep(StepParams P, ParticleArray
   bin_particle(P, r, valid, c, rs);
 }
 
-__global__ void __launch_bounds__(kPBlock) k_rec_place(int n, SortScratch S, const int *__restrict__ start,
-                                                       ReactionRecords src, ReactionRecords dst) {
+__global__ void __launch_bounds__(kPBlock) k_rec_place(StepParams P, int n, SortScratch S,
+                                                       const int *__restrict__ start, ReactionRecords src,
+                                                       ReactionRecords dst, unsigned *__restrict__ node_bits) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
   const int p = S.perm[j];
   const int4 c = src.cell[p];
   const float4 fr = src.frac[p], a = src.fric[p], b = src.psA[p], d = src.psB[p];
   const int slot = placed_slot(j, S, start);
+  set_node_bits(P, c, node_bits);
   dst.cell[slot] = c;
   dst.frac[slot] = fr;
   dst.fric[slot] = a;
@@ -412,8 +436,9 @@ void launch_bin(const StepParams &P, const ParticleArrays &pa, const SortScratch
   k_bin<<<pgrid(P.np), kPBlock, 0, st>>>(P, pa, S, err);
 }
 void launch_integrate_bin(const StepParams &P, const ParticleArrays &src, const ParticleArrays &dst,
-                          const ParticleForces &pf, const SortScratch &S, unsigned *err, cudaStream_t st) {
-  k_integrate_bin<<<pgrid(P.np), kPBlock, 0, st>>>(P, src, dst, pf, S, err);
+                          const ParticleForces &pf, const SortScratch &S, const int4 *marked, unsigned *node_bits,
+                          unsigned *err, cudaStream_t st) {
+  k_integrate_bin<<<pgrid(P.np), kPBlock, 0, st>>>(P, src, dst, pf, S, marked, node_bits, err);
 }
 // The scan and scatter passes of np binned entries.
 static void scan_scatter(const StepParams &P, int np, const SortScratch &S, int *row_start, const int4 *cell,
@@ -423,29 +448,30 @@ static void scan_scatter(const StepParams &P, int np, const SortScratch &S, int 
   k_scatter<<<pgrid(np), kPBlock, 0, st>>>(np, nb, S, row_start, cell, id);
 }
 void launch_place(const StepParams &P, const SortScratch &S, const ParticleArrays &src, const ParticleArrays &dst,
-                  int *row_start, int *slot_of_id, cudaStream_t st) {
+                  int *row_start, int *slot_of_id, unsigned *node_bits, cudaStream_t st) {
   scan_scatter(P, P.np, S, row_start, src.cell, src.pid, st);
-  k_place<<<pgrid(P.np), kPBlock, 0, st>>>(P.np, S, row_start, src, dst, slot_of_id);
+  k_place<<<pgrid(P.np), kPBlock, 0, st>>>(P, S, row_start, src, dst, slot_of_id, node_bits);
 }
 void launch_rec_place(const StepParams &P, int n, const SortScratch &S, const ReactionRecords &src,
-                      const ReactionRecords &dst, int *row_start, cudaStream_t st) {
+                      const ReactionRecords &dst, int *row_start, unsigned *node_bits, cudaStream_t st) {
   scan_scatter(P, n, S, row_start, src.cell, src.key, st);
-  k_rec_place<<<pgrid(n), kPBlock, 0, st>>>(n, S, row_start, src, dst);
+  k_rec_place<<<pgrid(n), kPBlock, 0, st>>>(P, n, S, row_start, src, dst, node_bits);
 }
 
 bool sort_fits_one_block(int nrows, int np) { return nrows <= kSmallRows && np <= kSmallNp; }
 
 void launch_sort_small(const StepParams &P, const ParticleArrays *update_from, const ParticleArrays &mid,
                        const ParticleForces &pf, const ParticleArrays &dst, int *row_start, int *slot_of_id,
-                       unsigned *err, cudaStream_t st) {
+                       unsigned *node_bits, unsigned *err, cudaStream_t st) {
   const size_t smem = small_smem(P.nrows, P.np);
   const int most = (int)small_smem(kSmallRows, kSmallNp);
   if (update_from) {
     cudaFuncSetAttribute(k_sort_small<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    k_sort_small<true><<<1, kSmallThreads, smem, st>>>(P, *update_from, mid, pf, dst, row_start, slot_of_id, err);
+    k_sort_small<true><<<1, kSmallThreads, smem, st>>>(P, *update_from, mid, pf, dst, row_start, slot_of_id, node_bits,
+                                                             err);
   } else {
     cudaFuncSetAttribute(k_sort_small<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    k_sort_small<false><<<1, kSmallThreads, smem, st>>>(P, mid, mid, pf, dst, row_start, slot_of_id, err);
+    k_sort_small<false><<<1, kSmallThreads, smem, st>>>(P, mid, mid, pf, dst, row_start, slot_of_id, node_bits, err);
   }
 }
 
@@ -480,9 +506,10 @@ void launch_pairs(const StepParams &P, const ParticleArrays &pa, CellIndex ci, c
 void launch_substep(const StepParams &P, const ParticleArrays &C, const ParticleArrays &D, const ParticleArrays &S,
                     CellIndex ci, int pair_reach, const float *rho, const float *jp, const int *bond_start,
                     const int *bond_other, const int *slot_of_id, const ParticleForces &pf, int sub,
-                    const ReactionRecords &rec, const SortScratch &rs, unsigned *err, cudaStream_t st) {
+                    const ReactionRecords &rec, const SortScratch &rs, unsigned *node_bits, unsigned *err,
+                    cudaStream_t st) {
   k_substep<<<(P.np + kSubParticles - 1) / kSubParticles, kPBlock, 0, st>>>(
-      P, C, D, S, ci, pair_reach, rho, jp, bond_start, bond_other, slot_of_id, pf, sub, rec, rs, err);
+      P, C, D, S, ci, pair_reach, rho, jp, bond_start, bond_other, slot_of_id, pf, sub, rec, rs, node_bits, err);
 }
 void launch_particle_momentum(const StepParams &P, const ParticleArrays &pa, double *partial, int nblocks,
                               cudaStream_t st) {

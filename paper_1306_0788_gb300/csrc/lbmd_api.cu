@@ -83,6 +83,9 @@ struct lbmd_ctx {
   ParticleForces pf{};
   int *slot_of_id = nullptr;
   int *row_start[2] = {nullptr, nullptr};
+  // CellIndex::node_bits: [b] those of pa[b] (with MD sub-stepping [0] those of the records, formed
+  // anew each step)
+  unsigned *node_bits[2] = {nullptr, nullptr};
   SortScratch sort{};
   int *bond_start = nullptr, *bond_other = nullptr;
   int nbonds = 0, bond_np = 0;  // bonds index particles 0..bond_np-1
@@ -421,18 +424,19 @@ int sort_particles(lbmd_ctx *c, bool update, cudaStream_t st) {
   const StepParams &P = c->P;
   const ParticleArrays &from = c->pa[c->pcur], &to = c->pa[1 - c->pcur];
   int *start = c->row_start[1 - c->pcur];
+  unsigned *bits = P.substeps > 1 ? nullptr : c->node_bits[1 - c->pcur];
   c->pcur = 1 - c->pcur;
   if (sort_fits_one_block(P.nrows, P.np)) {
-    launch_sort_small(P, update ? &from : nullptr, c->pt, c->pf, to, start, c->slot_of_id, c->err, st);
+    launch_sort_small(P, update ? &from : nullptr, c->pt, c->pf, to, start, c->slot_of_id, bits, c->err, st);
     if (update) CK(cudaEventRecord(c->ev_integrated, st), "event");
     return launched(c, "particle sort");
   }
   if (update)
-    launch_integrate_bin(P, from, c->pt, c->pf, c->sort, c->err, st);
+    launch_integrate_bin(P, from, c->pt, c->pf, c->sort, to.cell, bits, c->err, st);
   else
     launch_bin(P, c->pt, c->sort, c->err, st);
   if (update) CK(cudaEventRecord(c->ev_integrated, st), "event");
-  launch_place(P, c->sort, c->pt, to, start, c->slot_of_id, st);
+  launch_place(P, c->sort, c->pt, to, start, c->slot_of_id, bits, st);
   return launched(c, "particle sort", 4);  // bin, scan, scatter, place
 }
 
@@ -487,7 +491,7 @@ int substep_particles(lbmd_ctx *c, ParticleArrays &pa, ParticleForces &pf, CellI
   const ParticleArrays &other = c->pa[1 - c->pcur];
   const ParticleArrays work[2] = {{c->pt.cell, c->pt.frac, c->pt.vel, S.pid},
                                   {other.cell, other.frac, other.vel, S.pid}};
-  const CellIndex rows{c->row_start[c->pcur]};
+  const CellIndex rows{c->row_start[c->pcur], nullptr};
   SortScratch rs = c->rec_sort;
   rs.row_count = c->sort.row_count;
   rs.block_count = c->sort.block_count;
@@ -501,18 +505,18 @@ int substep_particles(lbmd_ctx *c, ParticleArrays &pa, ParticleForces &pf, CellI
     // (pair reach: particles may have left their row by one cell)
     launch_substep(Q, from, to, S, rows, P.reach > 0 ? P.reach + 1 : 0, c->rho_buf[c->cur], c->jp,
                    c->nbonds ? c->bond_start : nullptr, c->bond_other, c->slot_of_id, c->pf, sub, c->rec[0], rs,
-                   c->err, c->st);
+                   c->node_bits[0], c->err, c->st);
     if ((r = launched(c, "particle substep"))) return r;
   }
   // sort the (binned) records by (row, x cell, substep * np + id): the same counting sort as particles
-  launch_rec_place(P, (int)nrec, rs, c->rec[0], c->rec[1], c->rec_row_start, c->st);
+  launch_rec_place(P, (int)nrec, rs, c->rec[0], c->rec[1], c->rec_row_start, c->node_bits[0], c->st);
   if ((r = launched(c, "record sort", 3))) return r;
   pa = ParticleArrays{c->rec[1].cell, c->rec[1].frac, nullptr, nullptr};
   pf = c->pf;
   pf.fric = c->rec[1].fric;
   pf.psA = c->rec[1].psA;
   pf.psB = c->rec[1].psB;
-  ci = CellIndex{c->rec_row_start};
+  ci = CellIndex{c->rec_row_start, c->node_bits[0]};
   return LBMD_OK;
 }
 
@@ -538,7 +542,7 @@ int reserve_events(lbmd_ctx *c, size_t n) {
 int one_step(lbmd_ctx *c, unsigned long long step, cudaEvent_t t0, cudaEvent_t t1, unsigned flags, bool join) {
   StepParams &P = c->P;
   P.step = step;
-  const CellIndex ci{c->row_start[c->pcur]};
+  const CellIndex ci{c->row_start[c->pcur], c->node_bits[c->pcur]};
   const void *fin = c->pop[c->cur];
   void *fout = c->pop[1 - c->cur];
   float *rho = c->rho_buf[c->cur];
@@ -835,6 +839,7 @@ void lbmd_destroy(lbmd_ctx *c) {
   free_particles(c);
   free_records(c);
   dfree(c->sort.row_count); dfree(c->sort.block_count); dfree(c->row_start[0]); dfree(c->row_start[1]);
+  dfree(c->node_bits[0]); dfree(c->node_bits[1]);
   dfree(c->bond_start); dfree(c->bond_other);
   for (cudaEvent_t ev : c->ev) cudaEventDestroy(ev);
   delete c;
@@ -968,6 +973,8 @@ int lbmd_set_particles(lbmd_ctx *c, int n, const double *x, const double *v, con
     const size_t nb = (size_t)scan_blocks(P.nrows);
     for (int *&start : c->row_start)
       if (!start) CK(dalloc(&start, (size_t)P.nrows + 1), "alloc rows");
+    for (unsigned *&bits : c->node_bits)
+      if (!bits) CK(dalloc(&bits, node_words(P.nx) * (size_t)P.nrows), "alloc rows");
     if (!c->sort.block_count) CK(dalloc(&c->sort.block_count, nb), "alloc rows");
     CK(cudaMemsetAsync(c->sort.block_count, 0, sizeof(int) * nb, c->st), "clear rows");
     CK(dalloc(&c->sort.row_count, (size_t)P.nrows), "alloc rows");
@@ -982,7 +989,11 @@ int lbmd_set_particles(lbmd_ctx *c, int n, const double *x, const double *v, con
     CK(cudaMemcpyAsync(c->pt.frac, hf.data(), sizeof(float4) * n, cudaMemcpyHostToDevice, c->st), "upload");
     CK(cudaMemcpyAsync(c->pt.vel, hv.data(), sizeof(float4) * n, cudaMemcpyHostToDevice, c->st), "upload");
     CK(cudaMemcpyAsync(c->pt.pid, hid.data(), sizeof(int) * n, cudaMemcpyHostToDevice, c->st), "upload");
-    // the order of the (zero) total forces, as after a step: that of the buffer the sort leaves
+    // as after a step, the buffer the sort does not take holds the order of the (zero) total forces
+    // and, its nodes cleared below, cells of the lattice
+    for (unsigned *bits : c->node_bits)
+      CK(cudaMemsetAsync(bits, 0, sizeof(unsigned) * node_words(P.nx) * (size_t)P.nrows, c->st), "clear nodes");
+    CK(cudaMemcpyAsync(c->pa[0].cell, hc.data(), sizeof(int4) * n, cudaMemcpyHostToDevice, c->st), "upload");
     CK(cudaMemcpyAsync(c->pa[0].pid, hid.data(), sizeof(int) * n, cudaMemcpyHostToDevice, c->st), "upload");
     CK(cudaMemsetAsync(c->pf.total, 0, sizeof(float4) * n, c->st), "memset");
     int r = sort_particles(c, false, c->st);

@@ -132,7 +132,11 @@ struct SortScratch {
 
 struct CellIndex {
   const int *row_start;  // [nrows + 1] offsets into the sorted particle arrays
+  // the lattice update only: a bit per node, set where one of the node's 8 cells holds a particle
+  // (or reaction record) -- nodes elsewhere have nothing to gather.  Rows of node_words(nx) words.
+  const unsigned *node_bits;
 };
+__host__ __device__ __forceinline__ int node_words(int nx) { return (nx + 31) / 32; }
 
 // The one-pass lattice update: a block's warps own 8 consecutive rows (y) of a column tile of 32
 // x nodes (one per lane) and the block marches along z through one chunk of planes of that tile;
@@ -325,17 +329,21 @@ void launch_drift_check(const double *sums, const double *psum, double *ref, dou
 int scan_blocks(int nrows);
 void launch_bin(const StepParams &P, const ParticleArrays &pa, const SortScratch &S, unsigned *err, cudaStream_t st);
 void launch_integrate_bin(const StepParams &P, const ParticleArrays &src, const ParticleArrays &dst,
-                          const ParticleForces &pf, const SortScratch &S, unsigned *err, cudaStream_t st);
+                          const ParticleForces &pf, const SortScratch &S, const int4 *marked, unsigned *node_bits,
+                          unsigned *err, cudaStream_t st);
 void launch_place(const StepParams &P, const SortScratch &S, const ParticleArrays &src, const ParticleArrays &dst,
-                  int *row_start, int *slot_of_id, cudaStream_t st);
+                  int *row_start, int *slot_of_id, unsigned *node_bits, cudaStream_t st);
 void launch_rec_place(const StepParams &P, int n, const SortScratch &S, const ReactionRecords &src,
-                      const ReactionRecords &dst, int *row_start, cudaStream_t st);
+                      const ReactionRecords &dst, int *row_start, unsigned *node_bits, cudaStream_t st);
 // The same for a small system (nrows and np within one block's shared memory) in one launch: with
 // update_from, the particles are first updated from there into mid; mid is sorted into dst.
+// node_bits (or null): CellIndex::node_bits of the sorted particles.  The update clears the nodes of
+// the cells `marked` (those of dst before the sort overwrites it, whose nodes are the set ones), the
+// placing sets the new ones.
 bool sort_fits_one_block(int nrows, int np);
 void launch_sort_small(const StepParams &P, const ParticleArrays *update_from, const ParticleArrays &mid,
                        const ParticleForces &pf, const ParticleArrays &dst, int *row_start, int *slot_of_id,
-                       unsigned *err, cudaStream_t st);
+                       unsigned *node_bits, unsigned *err, cudaStream_t st);
 void launch_couple(const StepParams &P, const ParticleArrays &pa, CellIndex ci, const float *rho,
                    const float *jp, const ParticleForces &pf, cudaStream_t st);
 // The same with j' at the corners from jc (8 float4 per particle id, launch_corner_jprime or the
@@ -361,9 +369,11 @@ void launch_particle_momentum(const StepParams &P, const ParticleArrays &pa, dou
                               cudaStream_t st);
 // MD sub-stepping: one particle substep (coupling and pair forces at C, the substep's reaction
 // records, binned in rs for their sort, and the update into D); S, ci: the step's sorted particles.
+// The first substep clears node_bits, which launch_rec_place sets.
 void launch_substep(const StepParams &P, const ParticleArrays &C, const ParticleArrays &D, const ParticleArrays &S,
                     CellIndex ci, int pair_reach, const float *rho, const float *jp, const int *bond_start,
                     const int *bond_other, const int *slot_of_id, const ParticleForces &pf, int sub,
-                    const ReactionRecords &rec, const SortScratch &rs, unsigned *err, cudaStream_t st);
+                    const ReactionRecords &rec, const SortScratch &rs, unsigned *node_bits, unsigned *err,
+                    cudaStream_t st);
 
 }  // namespace lbmd
