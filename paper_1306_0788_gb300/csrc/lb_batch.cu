@@ -440,24 +440,14 @@ __global__ void __launch_bounds__(kBThreads) kb_drift_sums(const BatchDev *__res
     const StepParams &P = R.P;
     const T *f = static_cast<const T *>(R.pop[S.cur]);
     const long long base = (long long)(t - B->lay[slot].tile0) * ts;
-    double acc[5] = {0, 0, 0, 0, 0};
+    site::TotalSums sums;
     for (int k = threadIdx.x; k < ts; k += kBThreads) {
       const long long s = base + k;
       if (s >= P.N) break;
-      site::FloatPair m[5];  // the node's sums without rounding error; FP64 over nodes
-#pragma unroll
-      for (int i = 0; i < kQ; ++i) {
-        const float a = site::pop_read(P, f, R.rest, 0, i, s);
-        const float b = site::pop_read(P, f, R.rest, 1, i, s);
-        m[0].add(a);
-        m[1].add(b);
-        if (kCx[i]) { m[2].add(kCx[i] > 0 ? a : -a); m[2].add(kCx[i] > 0 ? b : -b); }
-        if (kCy[i]) { m[3].add(kCy[i] > 0 ? a : -a); m[3].add(kCy[i] > 0 ? b : -b); }
-        if (kCz[i]) { m[4].add(kCz[i] > 0 ? a : -a); m[4].add(kCz[i] > 0 ? b : -b); }
-      }
-#pragma unroll
-      for (int q = 0; q < 5; ++q) acc[q] += m[q].value();
+      sums.add([&](int i) { return site::pop_pair<T>(P, f, R.rest, i, (unsigned)s); });
     }
+    sums.flush();
+    const double *acc = sums.acc;
     __syncthreads();  // sh is free (previous tile)
 #pragma unroll
     for (int k = 0; k < 5; ++k) sh[k][threadIdx.x] = acc[k];
@@ -1378,7 +1368,7 @@ int lbmd_batch_get_fields(lbmd_batch *b, int slot, float *rhoA, float *rhoB, flo
   const long long N = sl.P.N;
   float *stage = reinterpret_cast<float *>(sl.pop[1 - cur]);
   launch_moments(sl.P, sl.pop[cur], sl.rest, sl.rho, nullptr, b->st);
-  launch_fields(sl.P, sl.pop[cur], sl.rest, sl.rho, stage, stage + N, stage + 2 * N, b->st);
+  launch_fields(sl.P, sl.pop[cur], sl.rest, sl.rho, stage, stage + N, u ? stage + 2 * N : nullptr, b->st);
   BK(cudaGetLastError(), "fields");
   const size_t bytes = sizeof(float) * (size_t)N;
   if (rhoA) BK(cudaMemcpyAsync(rhoA, stage, bytes, cudaMemcpyDeviceToHost, b->st), "download");

@@ -19,6 +19,19 @@ constexpr int kBlock = 256;
 
 using namespace site;
 
+// 8- and 4-byte asynchronous copies global -> shared (cp.async), their commit and wait.
+__device__ __forceinline__ void cp_async8(void *smem, const void *gmem) {
+  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async4(void *smem, const void *gmem) {
+  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all_but_one() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
+
 template <class T>
 __global__ void __launch_bounds__(kBlock) k_init_equilibrium(StepParams P, const float *__restrict__ rhoA,
                                                              const float *__restrict__ rhoB,
@@ -123,14 +136,6 @@ static_assert(kOnePassCols == 32 && kRhoCols - 32 <= 32, "a warp stages a ring r
 static_assert(kOnePassRows - 1 <= 15, "pair barriers 1 .. kOnePassRows - 1");
 
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-
-// 8-byte asynchronous copy global -> shared (cp.async), its commit and wait.
-__device__ __forceinline__ void cp_async8(void *smem, const void *gmem) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
 // Named barrier `id` (1 .. 15; 0 is __syncthreads) for `n` threads of the block, all of whose
 // warps take it convergently.
@@ -528,7 +533,10 @@ __global__ void __launch_bounds__(kBlock) k_boundary_densities(StepParams P, One
   rho2[node] = add2(rho2[node], zo[(long long)q * plane + (long long)y * P.nx + x]);
 }
 
-// rho_A, rho_B and u = (j' + g^SC/2)/rho at the current step (for readback).
+// rho_A, rho_B and u = (j' + g^SC/2)/rho at the current step (for readback; any output may be null:
+// without u the populations are not read).  Bound by HBM: 152 B of populations, 8 of densities and 20
+// of results per node in FP32: 467 us at 256^3, 6.5 TB/s (578 with a load for each component and 64-bit
+// neighbour addresses).
 template <class T>
 __global__ void __launch_bounds__(kBlock) k_fields(StepParams P, const T *__restrict__ store,
                                                    const float *__restrict__ rest,
@@ -536,23 +544,29 @@ __global__ void __launch_bounds__(kBlock) k_fields(StepParams P, const T *__rest
                                                    float *__restrict__ oB, float *__restrict__ ou) {
   const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= P.N) return;
-  const Coord c = site_coord(P, s);
-  int xs[3], ys[3], zs[3];
-  neighbours(P, c, xs, ys, zs);
+  const unsigned s32 = (unsigned)s;
+  const float2 *rho2 = reinterpret_cast<const float2 *>(rho);
+  const float2 r0 = __ldg(rho2 + s32);
+  if (oA) oA[s] = r0.x;
+  if (oB) oB[s] = r0.y;
+  if (!ou) return;
+  const NOff o = neighbour_offsets(P, site_coord(P, s));
+  float2 f[kQ];
+#pragma unroll
+  for (int i = 1; i < kQ; ++i)  // (the rest populations carry no momentum)
+    f[i] = pop_pair<T>(P, store, rest, i, (unsigned)((int)s32 + shift(o, -kCx[i], -kCy[i], -kCz[i])));
   float jx = 0.f, jy = 0.f, jz = 0.f;
 #pragma unroll
-  for (int i = 0; i < kQ; ++i) {
-    const long long src = pull_source(P, i, xs, ys, zs);
-    const float a = pop_read(P, store, rest, 0, i, src) + pop_read(P, store, rest, 1, i, src);
+  for (int i = 1; i < kQ; ++i) {
+    const float a = f[i].x + f[i].y;
     jx += kCx[i] * a; jy += kCy[i] * a; jz += kCz[i] * a;
   }
-  const float2 *rho2 = reinterpret_cast<const float2 *>(rho);
-  const float rA = rho2[s].x, rB = rho2[s].y;
+  const float rA = r0.x, rB = r0.y;
   float SAx = 0.f, SAy = 0.f, SAz = 0.f, SBx = 0.f, SBy = 0.f, SBz = 0.f;
 #pragma unroll
   for (int i = 1; i < kQ; ++i) {
-    const long long nb = ((long long)zs[1 + kCz[i]] * P.ny + ys[1 + kCy[i]]) * P.nx + xs[1 + kCx[i]];
-    const float a = kW[i] * rho2[nb].x, b = kW[i] * rho2[nb].y;
+    const float2 r = __ldg(rho2 + (unsigned)((int)s32 + shift(o, kCx[i], kCy[i], kCz[i])));
+    const float a = kW[i] * r.x, b = kW[i] * r.y;
     SAx += kCx[i] * a; SAy += kCy[i] * a; SAz += kCz[i] * a;
     SBx += kCx[i] * b; SBy += kCy[i] * b; SBz += kCz[i] * b;
   }
@@ -560,40 +574,63 @@ __global__ void __launch_bounds__(kBlock) k_fields(StepParams P, const T *__rest
   const float gy = -P.gAB * rA * SBy - P.gBA * rB * SAy;
   const float gz = -P.gAB * rA * SBz - P.gBA * rB * SAz;
   const float rinv = 1.f / (rA + rB);
-  if (oA) oA[s] = rA;
-  if (oB) oB[s] = rB;
-  if (ou) {
-    ou[3 * s] = (jx + 0.5f * gx) * rinv;
-    ou[3 * s + 1] = (jy + 0.5f * gy) * rinv;
-    ou[3 * s + 2] = (jz + 0.5f * gz) * rinv;
-  }
+  ou[3 * s] = (jx + 0.5f * gx) * rinv;
+  ou[3 * s + 1] = (jy + 0.5f * gy) * rinv;
+  ou[3 * s + 2] = (jz + 0.5f * gz) * rinv;
 }
 
-// FP64 block partial sums of [M_A, M_B, Px, Py, Pz] over the stored buffer (streaming
-// permutes populations, so sums over stored and post-streaming values agree), each node's sums
-// formed as FloatPair (lb_site.cuh): five FP64 additions per node instead of about ninety.
-constexpr int kSumBlock = 256;
+// FP64 block partial sums of [M_A, M_B, Px, Py, Pz] over the stored buffer (site::TotalSums).
+// Bound by HBM once enough loads are in flight: with loads into registers the compiler kept a few
+// per thread at a time (2 TB/s, 1008 us at 256^3, whatever the arithmetic).  Each thread copies its
+// next node's values into a slot of its own in shared memory (cp.async, no barriers) while it adds
+// the present one's: 497 us, 5.1 TB/s.  Five blocks fit an SM.
+constexpr int kSumBlock = 128;
+constexpr int kSumGrid = 5 * 152;
 template <class T>
 __global__ void __launch_bounds__(kSumBlock) k_fluid_sums(StepParams P, const T *__restrict__ store,
                                                           const float *__restrict__ rest,
                                                           double *__restrict__ partial) {
-  double acc[5] = {0, 0, 0, 0, 0};
-  for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < P.N;
-       s += (long long)gridDim.x * blockDim.x) {
-    FloatPair m[5];
+  // FP32: the (A, B) pair of each direction; 16-bit: its word, the rest pair in two more
+  using Word = std::conditional_t<kSplitRest<T>, unsigned, float2>;
+  constexpr int kWords = kSplitRest<T> ? kQ + 1 : kQ;
+  __shared__ Word stage[2][kWords][kSumBlock];
+  const unsigned N32 = (unsigned)P.N, stride = gridDim.x * kSumBlock;
+  auto fetch = [&](int k, unsigned s) {
+    const Word *src = reinterpret_cast<const Word *>(store) + s;
+    if constexpr (kSplitRest<T>) {
 #pragma unroll
-    for (int i = 0; i < kQ; ++i) {
-      const float a = pop_read(P, store, rest, 0, i, s);
-      const float b = pop_read(P, store, rest, 1, i, s);
-      m[0].add(a);
-      m[1].add(b);
-      if (kCx[i]) { m[2].add(kCx[i] > 0 ? a : -a); m[2].add(kCx[i] > 0 ? b : -b); }
-      if (kCy[i]) { m[3].add(kCy[i] > 0 ? a : -a); m[3].add(kCy[i] > 0 ? b : -b); }
-      if (kCz[i]) { m[4].add(kCz[i] > 0 ? a : -a); m[4].add(kCz[i] > 0 ? b : -b); }
+      for (int i = 1; i < kQ; ++i) cp_async4(&stage[k][i][threadIdx.x], src + (size_t)i * N32);
+      cp_async4(&stage[k][0][threadIdx.x], rest + s);
+      cp_async4(&stage[k][kQ][threadIdx.x], rest + N32 + s);
+    } else {
+#pragma unroll
+      for (int i = 0; i < kQ; ++i) cp_async8(&stage[k][i][threadIdx.x], src + (size_t)i * N32);
     }
-#pragma unroll
-    for (int k = 0; k < 5; ++k) acc[k] += m[k].value();
+  };
+  TotalSums sums;
+  unsigned s = blockIdx.x * kSumBlock + threadIdx.x;
+  if (s < N32) fetch(0, s);
+  cp_async_commit();
+  for (int k = 0; s < N32; k ^= 1) {
+    const unsigned next = s + stride;  // N + stride < 2^32: 19 N is
+    if (next < N32) fetch(k ^ 1, next);
+    cp_async_commit();
+    cp_async_wait_all_but_one();
+    sums.add([&](int i) {
+      if constexpr (kSplitRest<T>) {
+        if (i == 0)
+          return make_float2(__uint_as_float(stage[k][0][threadIdx.x]), __uint_as_float(stage[k][kQ][threadIdx.x]));
+        const float2 v = Pair16<T>::dec(stage[k][i][threadIdx.x]);
+        return make_float2(v.x + pop_shift(P, 0, i), v.y + pop_shift(P, 1, i));
+      } else {
+        return stage[k][i][threadIdx.x];
+      }
+    });
+    s = next;
   }
+  cp_async_wait_all();
+  sums.flush();
+  const double *acc = sums.acc;
   __shared__ double sh[5][kSumBlock];
 #pragma unroll
   for (int k = 0; k < 5; ++k) sh[k][threadIdx.x] = acc[k];
@@ -798,8 +835,8 @@ void launch_fields(const StepParams &P, const void *store, const float *rest, co
   });
 }
 int fluid_sum_blocks(const StepParams &P) {
-  long long b = (P.N + kSumBlock - 1) / kSumBlock;
-  return (int)(b < 1024 ? b : 1024);
+  const long long b = (P.N + kSumBlock - 1) / kSumBlock;
+  return (int)(b < kSumGrid ? b : kSumGrid);
 }
 void launch_fluid_sums(const StepParams &P, const void *store, const float *rest, double *partial, int nblocks,
                        cudaStream_t st) {

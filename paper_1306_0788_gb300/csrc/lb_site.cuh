@@ -91,24 +91,6 @@ struct Pair16<__nv_bfloat16> {
 
 __device__ __forceinline__ float pop_shift(const StepParams &P, int comp, int i) { return kW[i] * P.rho0[comp]; }
 
-// A sum of FP32 values without rounding error: kept as an unevaluated pair (hi, lo) of FP32
-// numbers, each addition split by Knuth's error-free two-sum (s + e == hi + x exactly; plain FP32
-// additions, nothing the compiler may contract).  FP64 arithmetic is slow on this GPU, so the FP64
-// reductions form each node's sums this way and add only the node totals, hi + lo, in FP64.  The
-// pair holds about 48 significant bits: a node total of a few dozen values carries a relative error
-// of ~2^-47 at most.
-struct FloatPair {
-  float hi = 0.f, lo = 0.f;
-  __device__ __forceinline__ void add(float x) {
-    const float s = hi + x;
-    const float bp = s - hi;
-    const float e = (hi - (s - bp)) + (x - bp);
-    hi = s;
-    lo += e;
-  }
-  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
-
 // Element index of direction i of component c at site s: [19][N][2], the (A, B) pair of a
 // direction at a node side by side (one 8-byte word in FP32, one 4-byte word in 16 bits).
 template <class T>
@@ -137,6 +119,77 @@ __device__ __forceinline__ void pop_write(const StepParams &P, T *buf, float *re
   else
     Pop<T>::st(buf + pop_elem<T>(P, c, i, s), v, kW[i] * P.rho0[c]);
 }
+
+// The (A, B) pair of direction i at site s, as pop_read of both components.
+template <class T>
+__device__ __forceinline__ float2 pop_pair(const StepParams &P, const T *buf, const float *rest, int i, unsigned s) {
+  const unsigned N32 = (unsigned)P.N;
+  if constexpr (kSplitRest<T>) {
+    if (i == 0 && rest) return make_float2(__ldg(rest + s), __ldg(rest + N32 + s));
+    const float2 v = Pair16<T>::dec(__ldg(reinterpret_cast<const unsigned *>(buf) + i * N32 + s));
+    return make_float2(v.x + pop_shift(P, 0, i), v.y + pop_shift(P, 1, i));
+  } else {
+    return __ldg(reinterpret_cast<const float2 *>(buf) + i * N32 + s);
+  }
+}
+
+// Sums of (A, B) pairs of FP32 values almost without rounding error: each lane is kept as an
+// unevaluated pair (hi, lo) of FP32 numbers, each addition split by Knuth's error-free two-sum
+// (s + e == hi + x exactly; plain FP32 additions, nothing the compiler may contract), on both lanes at
+// once with the packed instructions.  The pair holds about 48 significant bits; FP64 arithmetic is
+// slow on this GPU (a converted addition costs about a hundred FP32 ones), so the FP64 reductions add
+// only the sums of a few nodes, hi + lo, in FP64.
+struct FloatPair2 {
+  float2 hi{0.f, 0.f}, lo{0.f, 0.f};
+  // adds x, or (kMinus) subtracts it
+  template <bool kMinus = false>
+  __device__ __forceinline__ void add(float2 x) {
+    const float2 minus = make_float2(-1.f, -1.f);
+    const float2 s = kMinus ? __ffma2_rn(minus, x, hi) : __fadd2_rn(hi, x);
+    const float2 part = __ffma2_rn(minus, hi, s);  // of x, what reached s
+    const float2 e = __ffma2_rn(minus, __ffma2_rn(minus, part, s), hi);
+    lo = __fadd2_rn(lo, kMinus ? __ffma2_rn(minus, __fadd2_rn(x, part), e)
+                               : __fadd2_rn(e, __ffma2_rn(minus, part, x)));
+    hi = s;
+  }
+  __device__ __forceinline__ double a() const { return (double)hi.x + (double)lo.x; }
+  __device__ __forceinline__ double b() const { return (double)hi.y + (double)lo.y; }
+};
+
+// The conserved sums [M_A, M_B, Px, Py, Pz] of the nodes a thread visits (over stored values:
+// streaming permutes populations, so they sum alike), in FP64 over groups of kNodes nodes: 340 packed
+// FP32 instructions and 8 FP64 ones per node.
+struct TotalSums {
+  static constexpr int kNodes = 4;
+  double acc[5] = {0, 0, 0, 0, 0};
+  FloatPair2 m, px, py, pz;
+  int n = 0;
+  // adds a node whose (A, B) pair of direction i is value(i)
+  template <class F>
+  __device__ __forceinline__ void add(F value) {
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) {
+      const float2 v = value(i);
+      m.add(v);
+      if (kCx[i] > 0) px.add(v);
+      if (kCx[i] < 0) px.add<true>(v);
+      if (kCy[i] > 0) py.add(v);
+      if (kCy[i] < 0) py.add<true>(v);
+      if (kCz[i] > 0) pz.add(v);
+      if (kCz[i] < 0) pz.add<true>(v);
+    }
+    if (++n == kNodes) flush();
+  }
+  __device__ __forceinline__ void flush() {
+    acc[0] += m.a();
+    acc[1] += m.b();
+    acc[2] += px.a() + px.b();
+    acc[3] += py.a() + py.b();
+    acc[4] += pz.a() + pz.b();
+    m = px = py = pz = FloatPair2{};
+    n = 0;
+  }
+};
 
 struct Coord {
   int x, y, z;

@@ -1143,7 +1143,7 @@ int lbmd_get_fields(lbmd_ctx *c, float *rhoA, float *rhoB, float *u) {
   float *stage = reinterpret_cast<float *>(c->pop[1 - c->cur]);
   int r = ensure_densities(c);
   if (r) return r;
-  launch_fields(c->P, c->pop[c->cur], c->rest, c->rho_buf[c->cur], stage, stage + N, stage + 2 * N, c->st);
+  launch_fields(c->P, c->pop[c->cur], c->rest, c->rho_buf[c->cur], stage, stage + N, u ? stage + 2 * N : nullptr, c->st);
   if ((r = launched(c, "fields"))) return r;
   const size_t bytes = sizeof(float) * (size_t)N;
   if (rhoA) CK(cudaMemcpyAsync(rhoA, stage, bytes, cudaMemcpyDeviceToHost, c->st), "download");
@@ -1230,11 +1230,8 @@ int lbmd_get_fields_dev(lbmd_ctx *c, float *rhoA, float *rhoB, float *u, void *s
   if (!rhoA && !rhoB && !u) return LBMD_OK;
   const cudaStream_t caller = static_cast<cudaStream_t>(stream);
   if ((r = dev_getter_begin(c, caller))) return r;
-  // outputs the caller does not want go to the spare population buffer, as in lbmd_get_fields
-  float *stage = reinterpret_cast<float *>(c->pop[1 - c->cur]);
   if ((r = ensure_densities(c))) return r;
-  launch_fields(c->P, c->pop[c->cur], c->rest, c->rho_buf[c->cur], rhoA ? rhoA : stage, rhoB ? rhoB : stage + N,
-                u ? u : stage + 2 * N, c->st);
+  launch_fields(c->P, c->pop[c->cur], c->rest, c->rho_buf[c->cur], rhoA, rhoB, u, c->st);
   if ((r = launched(c, "fields"))) return r;
   return dev_getter_end(c, caller);
 }
