@@ -12,19 +12,30 @@
 using namespace lbmd;
 
 namespace {
-constexpr int kGraphSteps = 2;  // steps per replayed graph: both buffer pairs return to their start
+// Replayed graphs hold an even number of steps (both buffer pairs return to their start), of three
+// lengths.  A replay costs about 5 us between one graph and the next: of 50 steps of 32^3 with 64
+// particles 702 us with graphs of two steps, 579 of ten, 556 of fifty; of 45x37x29 fluid only 468,
+// 356, 337; of 64^3 with 1000 particles 1273, 1122, 1092.  Recording takes 6 us per step of fluid
+// alone and about 35 with particles (0.2 and 1.3 ms for 32 steps), so the longer graphs are recorded
+// once a context has replayed as many steps as make up for it.
+constexpr int kGraphLevels = 3;
+constexpr int kGraphSteps[kGraphLevels] = {2, 8, 32};
+constexpr int64_t kGraphAfter[kGraphLevels] = {0, 128, 4096};  // steps replayed since the last setter
+constexpr int kShortGraph = kGraphSteps[0];
 
-// A recorded sequence of kGraphSteps coupled steps (lbmd_set_graphs).
+// A recorded sequence of coupled steps (lbmd_set_graphs).
 struct StepGraph {
   cudaGraph_t graph = nullptr;  // kept for the event nodes' handles
   cudaGraphExec_t exec = nullptr;
   int64_t launches = 0;                            // kernels per replay
-  cudaGraphNode_t ev_node[2 * kGraphSteps] = {};  // k_collide timing events, retargeted per replay
+  cudaGraphNode_t ev_node[2 * kShortGraph] = {};  // k_collide timing events, retargeted per replay
   // the noisy MRT update of each step: its node and the counter offset it was recorded with
   // (its counter is patched per replay; see is_noisy_update)
-  cudaGraphNode_t upd_node[kGraphSteps] = {};
-  unsigned long long upd_off[kGraphSteps] = {};
-  int n_upd = 0;
+  struct Update {
+    cudaGraphNode_t node;
+    unsigned long long off;
+  };
+  std::vector<Update> updates;
 };
 constexpr int kGraphUnavailable = 1;  // record_steps: take the steps one by one instead
 }  // namespace
@@ -110,15 +121,16 @@ struct lbmd_ctx {
   double prof_ms = 0.0;
   int64_t prof_launches = 0;
   // replayed step graphs: recorded on gst (never on the caller's stream, which may carry other
-  // work), one per parity of (cur, pcur) at the replay's start, launched into st; the kernels
+  // work), one per length and parity of (cur, pcur) at the replay's start, launched into st; the kernels
   // read their noise counter's base from step_base, which holds dev_step once the work
   // enqueued so far has run (-1: not known)
   bool graphs = true;
   cudaStream_t gst = nullptr;
-  StepGraph graph[2][2];
+  StepGraph graph[kGraphLevels][2][2];
+  int64_t replayed = 0;  // steps replayed since the graphs were dropped
   unsigned long long *step_base = nullptr;
   int64_t dev_step = -1;
-  cudaEvent_t ph[2 * kGraphSteps] = {};  // stand-ins for the timing events while recording
+  cudaEvent_t ph[2 * kShortGraph] = {};  // stand-ins for the timing events while recording
 };
 
 namespace {
@@ -622,18 +634,21 @@ int one_step(lbmd_ctx *c, unsigned long long step, cudaEvent_t t0, cudaEvent_t t
 }
 
 void drop_graphs(lbmd_ctx *c) {
-  for (auto &row : c->graph)
-    for (StepGraph &g : row) {
-      if (g.exec) cudaGraphExecDestroy(g.exec);  // a launch in flight completes first
-      if (g.graph) cudaGraphDestroy(g.graph);
-      g = StepGraph{};
-    }
+  for (auto &level : c->graph)
+    for (auto &row : level)
+      for (StepGraph &g : row) {
+        if (g.exec) cudaGraphExecDestroy(g.exec);  // a launch in flight completes first
+        if (g.graph) cudaGraphDestroy(g.graph);
+        g = StepGraph{};
+      }
+  c->replayed = 0;
 }
 
-// Records kGraphSteps steps from the current buffers into g: on the private stream gst, with
+// Records nsteps steps from the current buffers into g: on the private stream gst, with
 // the noise counters relative to the device-resident step base, the base advanced at the end.
-// Nothing runs; the context's host state is left as it was.
-int record_steps(lbmd_ctx *c, StepGraph &g) {
+// Nothing runs; the context's host state is left as it was.  (Profiled steps are recorded kShortGraph
+// at a time.)
+int record_steps(lbmd_ctx *c, StepGraph &g, int nsteps) {
   const StepParams &P = c->P;
   int r;
   if (P.np > 0 && P.substeps > 1 && (r = ensure_records(c, (long long)P.substeps * P.np)))
@@ -652,11 +667,11 @@ int record_steps(lbmd_ctx *c, StepGraph &g) {
   c->st = c->gst;
   c->P.step_base = c->step_base;
   r = LBMD_OK;
-  for (int j = 0; j < kGraphSteps && !r; ++j)
+  for (int j = 0; j < nsteps && !r; ++j)
     r = one_step(c, (unsigned long long)j, c->prof ? c->ph[2 * j] : nullptr, c->prof ? c->ph[2 * j + 1] : nullptr,
-                 cudaEventRecordExternal, j == kGraphSteps - 1);
+                 cudaEventRecordExternal, j == nsteps - 1);
   if (!r) {
-    launch_advance_step(c->step_base, kGraphSteps, c->gst);
+    launch_advance_step(c->step_base, nsteps, c->gst);
     r = launched(c, "step counter");
   }
   cudaGraph_t graph = nullptr;
@@ -693,19 +708,18 @@ int record_steps(lbmd_ctx *c, StepGraph &g) {
       if (t == cudaGraphNodeTypeEventRecord) {
         cudaEvent_t ev = nullptr;
         if ((ei = cudaGraphEventRecordNodeGetEvent(nodes[k], &ev)) != cudaSuccess) break;
-        for (int q = 0; q < 2 * kGraphSteps; ++q)
+        for (int q = 0; q < 2 * kShortGraph; ++q)
           if (ev == c->ph[q]) g.ev_node[q] = nodes[k];
       } else if (t == cudaGraphNodeTypeKernel && noisy) {
         cudaKernelNodeParams kp;
         if ((ei = cudaGraphKernelNodeGetParams(nodes[k], &kp)) != cudaSuccess) break;
-        if (!is_noisy_update(kp.func) || !kp.kernelParams || g.n_upd == kGraphSteps) continue;
+        if (!is_noisy_update(kp.func) || !kp.kernelParams) continue;
         StepParams Q;
         std::memcpy(&Q, kp.kernelParams[0], sizeof(Q));
-        g.upd_node[g.n_upd] = nodes[k];
-        g.upd_off[g.n_upd++] = Q.step;
+        g.updates.push_back({nodes[k], Q.step});
       }
     }
-    for (int q = 0; q < 2 * kGraphSteps && ei == cudaSuccess && c->prof; ++q)
+    for (int q = 0; q < 2 * kShortGraph && ei == cudaSuccess && c->prof; ++q)
       if (!g.ev_node[q]) ei = cudaErrorInvalidValue;
   }
   if (ei != cudaSuccess) {
@@ -713,7 +727,7 @@ int record_steps(lbmd_ctx *c, StepGraph &g) {
     cudaGetLastError();
     return cuda_fail(c, ei, "graph instantiation");
   }
-  if (noisy && g.n_upd != kGraphSteps) {  // the update's nodes were not recognised
+  if (noisy && g.updates.size() != (size_t)nsteps) {  // the update's nodes were not recognised
     drop_graphs(c);
     c->graphs = false;
     return kGraphUnavailable;
@@ -721,29 +735,39 @@ int record_steps(lbmd_ctx *c, StepGraph &g) {
   return LBMD_OK;
 }
 
-// kGraphSteps steps by one launch of the graph recorded for the current buffers.
-int replay_steps(lbmd_ctx *c) {
-  StepGraph &g = c->graph[c->cur][c->pcur];
+// The graph length for the next of n steps: the longest that fits and is recorded, or due for it.
+int graph_level(const lbmd_ctx *c, int n) {
+  int level = 0;
+  for (int k = 1; k < kGraphLevels && !c->prof; ++k)
+    if (kGraphSteps[k] <= n && c->replayed >= kGraphAfter[k]) level = k;
+  return level;
+}
+
+// kGraphSteps[level] steps by one launch of the graph recorded for the current buffers.
+int replay_steps(lbmd_ctx *c, int level) {
+  StepGraph &g = c->graph[level][c->cur][c->pcur];
+  const int nsteps = kGraphSteps[level];
   int r;
   if ((r = prepare_onepass(c))) return r;
   if (uses_onepass(c) && ((r = ensure_densities(c)) || (r = ensure_corner_j(c))))
     return r;  // before recording: not in the graph
-  if (!g.exec && (r = record_steps(c, g))) return r;
+  if (!g.exec && (r = record_steps(c, g, nsteps))) return r;
   if (c->dev_step != c->steps) {  // steps were taken without the graph since it last ran
     launch_set_step(c->step_base, (unsigned long long)c->steps, c->st);
     if ((r = launched(c, "step counter"))) return r;
   }
   if (c->prof) {
-    if ((r = reserve_events(c, 2 * kGraphSteps))) return r;
-    for (int q = 0; q < 2 * kGraphSteps; ++q)
+    if ((r = reserve_events(c, 2 * kShortGraph))) return r;
+    for (int q = 0; q < 2 * kShortGraph; ++q)
       CK(cudaGraphExecEventRecordNodeSetEvent(g.exec, g.ev_node[q], c->ev[c->ev_used + q]), "timing event");
   }
-  for (int q = 0; q < g.n_upd; ++q)
-    CK(set_update_step(g.exec, g.upd_node[q], (unsigned long long)c->steps + g.upd_off[q]), "update counter");
+  for (const StepGraph::Update &u : g.updates)
+    CK(set_update_step(g.exec, u.node, (unsigned long long)c->steps + u.off), "update counter");
   CK(cudaGraphLaunch(g.exec, c->st), "graph launch");
-  if (c->prof) c->ev_used += 2 * kGraphSteps;
+  if (c->prof) c->ev_used += 2 * kShortGraph;
   c->launches += g.launches;
-  c->steps += kGraphSteps;
+  c->steps += nsteps;
+  c->replayed += nsteps;
   c->dev_step = c->steps;
   c->rho_valid = uses_onepass(c);
   c->jc_valid = c->rho_valid && c->np > 0 && c->P.substeps == 1;
@@ -1064,11 +1088,14 @@ int lbmd_step(lbmd_ctx *c, int nsteps) {
     left -= n;
     int s = 0;
     if (c->graphs)
-      for (; s + kGraphSteps <= n; s += kGraphSteps)
-        if ((r = replay_steps(c))) {
+      while (s + kShortGraph <= n) {
+        const int level = graph_level(c, n - s);
+        if ((r = replay_steps(c, level))) {
           if (r != kGraphUnavailable) return r;
           break;
         }
+        s += kGraphSteps[level];
+      }
     if (s < n) {
       if ((r = prepare_onepass(c))) return r;
       if (uses_onepass(c) && ((r = ensure_densities(c)) || (r = ensure_corner_j(c)))) return r;
