@@ -224,7 +224,8 @@ int lbmd_set_graphs(lbmd_ctx *ctx, int on);
  * reads the populations once per step instead of twice.  passes = 0 (the default) takes one
  * pass with FP32 storage on lattices large enough (about 96^3 and up, a little larger where the
  * tiles of 32 x 8 columns are ragged), two passes otherwise (with 16-bit storage the update is
- * bound by instruction issue, not by the bytes the second pass reads).  Both give the
+ * bound by instruction issue, not by the bytes the second pass reads); without particles, lattices
+ * of up to 65536 nodes take the two passes in one launch (the same bits).  Both give the
  * same step up to FP32 rounding order (the densities are sums in another order).  One pass
  * needs the BGK collision and md_substeps = 1 (else LBMD_E_INVALID_ARG for passes = 1).  Drops
  * the recorded graphs.  lbmd_get_lattice_passes returns the update the next step takes (1 or 2;

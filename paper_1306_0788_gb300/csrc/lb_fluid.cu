@@ -106,6 +106,65 @@ __global__ void __launch_bounds__(kBlock, 3) k_collide(StepParams P, const T *__
   collide<T, kParticles, kMRT, kBisect>(P, s, P.step, fin, fout, rho, pa, pf, ci, err, rest_in, rest_out);
 }
 
+// ------------------------------------------------------------------ small lattices
+//
+// Density pass and update of a lattice without particles in one launch: a block forms the densities
+// of its tile of 16 x 4 x 4 nodes and of the nodes around it (up to 648 for 256: the populations are
+// read 2.5 times more than by a density pass, from L2 and L1, where a small lattice lives) in shared
+// memory, then updates its nodes.  What bounds a small lattice is the chain of dependent launches; this
+// halves it.  The same sums in the same order as the two kernels, so the same bits.  A step in two
+// launches / one, us: 32^3 5.64 / 4.87, 45x37x29 6.92 / 6.42, 40^3 6.67 / 6.16, 48^3 8.06 / 9.48; 32^3 in
+// FP16 5.03 / 4.62, with the fluctuating MRT collision 7.70 / 7.00.  (With particles the chain of
+// coupling, particle update and sort bounds the step, and this form gains nothing.)
+constexpr int kTileX = 16, kTileY = 4, kTileZ = 4;
+static_assert(kTileX * kTileY * kTileZ == kBlock, "a thread per node of the tile");
+
+struct TileRho {
+  static constexpr bool kStaged = true;
+  const float2 (*rho)[kTileY + 2][kTileX + 2];
+  int x, y, z;  // this node in the tile, counted from the layer around it
+  __device__ float2 operator()(int cx, int cy, int cz) const { return rho[z + cz][y + cy][x + cx]; }
+};
+
+// (the parameters of k_collide; rho, pa, pf and ci are not used)
+template <class T, bool kMRT>
+__global__ void __launch_bounds__(kBlock, 2) k_step_small(StepParams P, const T *__restrict__ fin,
+                                                          T *__restrict__ fout, const float *__restrict__,
+                                                          ParticleArrays pa, ParticleForces pf, CellIndex ci,
+                                                          unsigned *err, const float *__restrict__ rest_in,
+                                                          float *__restrict__ rest_out) {
+  __shared__ float2 rho[kTileZ + 2][kTileY + 2][kTileX + 2];
+  const int ntx = (P.nx + kTileX - 1) / kTileX, nty = (P.ny + kTileY - 1) / kTileY;
+  const int tz = blockIdx.x / (ntx * nty), txy = blockIdx.x - tz * (ntx * nty), ty = txy / ntx;
+  const int x0 = (txy - ty * ntx) * kTileX, y0 = ty * kTileY, z0 = tz * kTileZ;
+  const int vx = min(kTileX, P.nx - x0), vy = min(kTileY, P.ny - y0), vz = min(kTileZ, P.nz - z0);
+  constexpr int kAround = (kTileX + 2) * (kTileY + 2) * (kTileZ + 2);
+#pragma unroll
+  for (int r = 0; r < (kAround + kBlock - 1) / kBlock; ++r) {
+    const int e = r * kBlock + threadIdx.x;
+    const int hz = e / ((kTileX + 2) * (kTileY + 2)), hxy = e - hz * ((kTileX + 2) * (kTileY + 2));
+    const int hy = hxy / (kTileX + 2), hx = hxy - hy * (kTileX + 2);
+    if (hx > vx + 1 || hy > vy + 1 || hz > vz + 1) continue;
+    const bool in_x = hx != 0 && hx != vx + 1, in_y = hy != 0 && hy != vy + 1, in_z = hz != 0 && hz != vz + 1;
+    if (!in_x && !in_y && !in_z) continue;  // no neighbour of a node of the tile
+    Coord c{x0 + hx - 1, y0 + hy - 1, z0 + hz - 1};
+    c.x += c.x < 0 ? P.nx : c.x >= P.nx ? -P.nx : 0;
+    c.y += c.y < 0 ? P.ny : c.y >= P.ny ? -P.ny : 0;
+    c.z += c.z < 0 ? P.nz : c.z >= P.nz ? -P.nz : 0;
+    const NodeMoments n = node_moments(P, c, (unsigned)site_index(P, c.x, c.y, c.z), fin, rest_in);
+    rho[hz][hy][hx] = make_float2(n.rA, n.rB);
+  }
+  __syncthreads();
+  const int x = threadIdx.x % kTileX, y = threadIdx.x / kTileX % kTileY, z = threadIdx.x / (kTileX * kTileY);
+  if (x >= vx || y >= vy || z >= vz) return;
+  const Coord c{x0 + x, y0 + y, z0 + z};
+  const long long s = site_index(P, c.x, c.y, c.z);
+  float fA[kQ], fB[kQ], rA, rB;
+  collide_core_at<T, false, kMRT, false, TileRho>(P, c, s, P.step, fin, nullptr, pa, pf, ci, err, rest_in, fA, fB, rA,
+                                                  rB, TileRho{rho, x + 1, y + 1, z + 1});
+  store_node<T, kMRT>(P, (unsigned)s, fout, rest_out, fA, fB, rA, rB);
+}
+
 // ------------------------------------------------------------------ one-pass update
 //
 // Streaming carries f*_i(r) to r + c_i, so the next density of a node is the sum of the
@@ -724,8 +783,20 @@ void launch_moments(const StepParams &P, const void *store, const float *rest, f
     k_moments<T><<<grid_for(P.N), kBlock, 0, st>>>(P, static_cast<const T *>(store), rest, rho, jp);
   });
 }
-void launch_collide(const StepParams &P, const void *fin, void *fout, float *rest, const float *rho,
-                    const ParticleArrays &pa, const ParticleForces &pf, CellIndex ci, unsigned *err,
+void launch_step_small(const StepParams &P, const void *fin, void *fout, const float *rest_in, float *rest_out,
+                       unsigned *err, cudaStream_t st) {
+  auto tiles = [](int n, int edge) { return (unsigned)((n + edge - 1) / edge); };
+  const unsigned grid = tiles(P.nx, kTileX) * tiles(P.ny, kTileY) * tiles(P.nz, kTileZ);
+  with_storage(P, [&](auto t) {
+    using T = std::remove_pointer_t<decltype(t)>;
+    auto *kernel = P.collision == LBMD_COLLISION_MRT ? k_step_small<T, true> : k_step_small<T, false>;
+    kernel<<<grid, kBlock, 0, st>>>(P, static_cast<const T *>(fin), static_cast<T *>(fout), nullptr, ParticleArrays{},
+                                    ParticleForces{}, CellIndex{}, err, rest_in, rest_out);
+  });
+}
+
+void launch_collide(const StepParams &P, const void *fin, void *fout, const float *rest_in, float *rest_out,
+                    const float *rho, const ParticleArrays &pa, const ParticleForces &pf, CellIndex ci, unsigned *err,
                     cudaStream_t st) {
   with_storage(P, [&](auto t) {
     using T = std::remove_pointer_t<decltype(t)>;
@@ -734,33 +805,33 @@ void launch_collide(const StepParams &P, const void *fin, void *fout, float *res
     const bool mrt = P.collision == LBMD_COLLISION_MRT;
     const bool records = P.np > 0 && P.substeps > 1;
     if (records && mrt)
-      k_collide<T, true, true, true><<<grid_for(P.N), kBlock, 0, st>>>(P, a, b, rho, pa, pf, ci, err, rest, rest);
+      k_collide<T, true, true, true><<<grid_for(P.N), kBlock, 0, st>>>(P, a, b, rho, pa, pf, ci, err, rest_in, rest_out);
     else if (records)
-      k_collide<T, true, false, true><<<grid_for(P.N), kBlock, 0, st>>>(P, a, b, rho, pa, pf, ci, err, rest, rest);
+      k_collide<T, true, false, true><<<grid_for(P.N), kBlock, 0, st>>>(P, a, b, rho, pa, pf, ci, err, rest_in, rest_out);
     else if (P.np > 0 && mrt)
-      k_collide<T, true, true><<<grid_for(P.N), kBlock, 0, st>>>(P, a, b, rho, pa, pf, ci, err, rest, rest);
+      k_collide<T, true, true><<<grid_for(P.N), kBlock, 0, st>>>(P, a, b, rho, pa, pf, ci, err, rest_in, rest_out);
     else if (P.np > 0)
-      k_collide<T, true, false><<<grid_for(P.N), kBlock, 0, st>>>(P, a, b, rho, pa, pf, ci, err, rest, rest);
+      k_collide<T, true, false><<<grid_for(P.N), kBlock, 0, st>>>(P, a, b, rho, pa, pf, ci, err, rest_in, rest_out);
     else if (mrt)
-      k_collide<T, false, true><<<grid_for(P.N), kBlock, 0, st>>>(P, a, b, rho, pa, pf, ci, err, rest, rest);
+      k_collide<T, false, true><<<grid_for(P.N), kBlock, 0, st>>>(P, a, b, rho, pa, pf, ci, err, rest_in, rest_out);
     else
-      k_collide<T, false, false><<<grid_for(P.N), kBlock, 0, st>>>(P, a, b, rho, pa, pf, ci, err, rest, rest);
+      k_collide<T, false, false><<<grid_for(P.N), kBlock, 0, st>>>(P, a, b, rho, pa, pf, ci, err, rest_in, rest_out);
   });
 }
 
-void launch_collide_onepass(const StepParams &P, const void *fin, void *fout, float *rest, const float *rho,
-                            float *rho_next, OnePassOut out, const ParticleArrays &pa, const ParticleForces &pf,
+void launch_collide_onepass(const StepParams &P, const void *fin, void *fout, const float *rest_in, float *rest_out,
+                            const float *rho, float *rho_next, OnePassOut out, const ParticleArrays &pa, const ParticleForces &pf,
                             CellIndex ci, unsigned *err, OnePassGeom G, int grid, cudaStream_t st) {
   with_storage(P, [&](auto t) {
     using T = std::remove_pointer_t<decltype(t)>;
     const T *a = static_cast<const T *>(fin);
     T *b = static_cast<T *>(fout);
     if (P.np > 0)
-      k_collide_onepass<T, true><<<grid, kOPThreads, 0, st>>>(P, a, b, rho, rho_next, out, pa, pf, ci, err, rest,
-                                                              rest, G);
+      k_collide_onepass<T, true><<<grid, kOPThreads, 0, st>>>(P, a, b, rho, rho_next, out, pa, pf, ci, err, rest_in,
+                                                              rest_out, G);
     else
-      k_collide_onepass<T, false><<<grid, kOPThreads, 0, st>>>(P, a, b, rho, rho_next, out, pa, pf, ci, err, rest,
-                                                               rest, G);
+      k_collide_onepass<T, false><<<grid, kOPThreads, 0, st>>>(P, a, b, rho, rho_next, out, pa, pf, ci, err, rest_in,
+                                                               rest_out, G);
   });
 }
 
@@ -798,7 +869,8 @@ template <class T>
 bool is_noisy_update_of(const void *fn) {
   return fn == reinterpret_cast<const void *>(&k_collide<T, true, true, true>) ||
          fn == reinterpret_cast<const void *>(&k_collide<T, true, true>) ||
-         fn == reinterpret_cast<const void *>(&k_collide<T, false, true>);
+         fn == reinterpret_cast<const void *>(&k_collide<T, false, true>) ||
+         fn == reinterpret_cast<const void *>(&k_step_small<T, true>);
 }
 
 bool is_noisy_update(const void *fn) {
@@ -812,6 +884,7 @@ constexpr int arity(void (*)(A...)) {
 
 cudaError_t set_update_step(cudaGraphExec_t exec, cudaGraphNode_t node, unsigned long long step) {
   constexpr int kArgs = arity(&k_collide<float, false, true>);
+  static_assert(kArgs == arity(&k_step_small<float, true>), "the noisy updates take the same parameters");
   cudaKernelNodeParams kp;
   cudaError_t e = cudaGraphKernelNodeGetParams(node, &kp);
   if (e != cudaSuccess) return e;

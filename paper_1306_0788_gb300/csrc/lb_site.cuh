@@ -251,15 +251,17 @@ __device__ __forceinline__ int shift(const NOff &o, int cx, int cy, int cz) {
          (cz < 0 ? o.m[2] : cz > 0 ? o.p[2] : 0);
 }
 
-// Densities rho_z = sum_i f_zi (appendix, zeroth mode) of site s, stored interleaved
-// (rho_A, rho_B), and j' = sum_z sum_i f_zi c_i (written when jp is not NULL).
+// Densities rho_z = sum_i f_zi (appendix, zeroth mode) of the node c at site s32, and j' = sum_z sum_i
+// f_zi c_i.
+struct NodeMoments {
+  float rA, rB, jx, jy, jz;
+};
+
 template <class T>
-__device__ __forceinline__ void moments(const StepParams &P, long long s, const T *__restrict__ fin,
-                                        const float *__restrict__ rest, float *__restrict__ rho,
-                                        float *__restrict__ jp) {
-  const Coord c = site_coord(P, s);
+__device__ __forceinline__ NodeMoments node_moments(const StepParams &P, const Coord &c, unsigned s32,
+                                                    const T *__restrict__ fin, const float *__restrict__ rest) {
   const NOff o = neighbour_offsets(P, c);
-  const unsigned N32 = (unsigned)P.N, s32 = (unsigned)s;
+  const unsigned N32 = (unsigned)P.N;
   // 16-bit storage: the moving populations are summed as stored (shifted) and the shifts added
   // once; the shifts cancel in j' (sum_i w_i c_i = 0)
   constexpr bool kShifted = kSplitRest<T>;
@@ -299,11 +301,20 @@ __device__ __forceinline__ void moments(const StepParams &P, long long s, const 
     rA += shift_sum(P, 0);
     rB += shift_sum(P, 1);
   }
-  reinterpret_cast<float2 *>(rho)[s] = make_float2(rA, rB);
+  return NodeMoments{rA, rB, jx, jy, jz};
+}
+
+// node_moments of site s, the densities stored interleaved (rho_A, rho_B), j' when jp is not NULL.
+template <class T>
+__device__ __forceinline__ void moments(const StepParams &P, long long s, const T *__restrict__ fin,
+                                        const float *__restrict__ rest, float *__restrict__ rho,
+                                        float *__restrict__ jp) {
+  const NodeMoments n = node_moments(P, site_coord(P, s), (unsigned)s, fin, rest);
+  reinterpret_cast<float2 *>(rho)[s] = make_float2(n.rA, n.rB);
   if (jp) {
-    jp[s] = jx;
-    jp[P.N + s] = jy;
-    jp[2 * P.N + s] = jz;
+    jp[s] = n.jx;
+    jp[P.N + s] = n.jy;
+    jp[2 * P.N + s] = n.jz;
   }
 }
 

@@ -64,7 +64,9 @@ struct lbmd_ctx {
   StepParams P{};
   unsigned char *pop[2] = {nullptr, nullptr};  // population buffers, element type P.storage
   size_t pop_elem = 4;
-  float *rest = nullptr;  // 16-bit storage: FP32 rest populations [2][N] (not double-buffered: local)
+  // 16-bit storage: FP32 rest populations [2][N], those of pop[cur] in rest[cur]; the same array twice
+  // (they are local to a node) except on small lattices, whose update may read its neighbours' too
+  float *rest[2] = {nullptr, nullptr};
   int cur = 0;
   // [N][2] interleaved rho_A, rho_B: rho_buf[cur] holds the densities of pop[cur] while
   // rho_valid (after init_fluid, set_populations and one-pass steps; the two-pass update
@@ -324,6 +326,16 @@ bool uses_onepass(const lbmd_ctx *c) {
   return c->op_grid > 0;  // auto: prepare_onepass decided from the size
 }
 
+// Lattices without particles of up to kSmallNodes nodes take density pass and update in one launch
+// (k_step_small has the figures on both sides of the line), unless two passes are set.
+constexpr long long kSmallNodes = 65536;
+
+bool small_lattice(const StepParams &P) { return P.N <= kSmallNodes; }
+
+bool uses_one_launch(const lbmd_ctx *c) {
+  return small_lattice(c->P) && c->np == 0 && c->passes == 0 && !uses_onepass(c);
+}
+
 // Frees what prepare_onepass set up.
 void free_onepass(lbmd_ctx *c) {
   dfree(c->op_runs);
@@ -409,7 +421,7 @@ int prepare_onepass(lbmd_ctx *c) {
 // The densities of the current state into rho_buf[cur] (a density pass), if not there already.
 int ensure_densities(lbmd_ctx *c) {
   if (c->rho_valid) return LBMD_OK;
-  launch_moments(c->P, c->pop[c->cur], c->rest, c->rho_buf[c->cur], nullptr, c->st);
+  launch_moments(c->P, c->pop[c->cur], c->rest[c->cur], c->rho_buf[c->cur], nullptr, c->st);
   const int r = launched(c, "moments");
   if (!r) c->rho_valid = true;
   return r;
@@ -455,7 +467,7 @@ int sort_particles(lbmd_ctx *c, bool update, cudaStream_t st) {
 // FP64 totals of the current state into diag_out: [M_A, M_B, Px, Py, Pz] of the fluid and,
 // with particles, [5..7] = sum m v (K9 of the step; appendix and Sec. 2 for what they conserve).
 int enqueue_totals(lbmd_ctx *c) {
-  launch_fluid_sums(c->P, c->pop[c->cur], c->rest, c->diag_partial, c->diag_blocks, c->st);
+  launch_fluid_sums(c->P, c->pop[c->cur], c->rest[c->cur], c->diag_partial, c->diag_blocks, c->st);
   launch_finish_sums(c->diag_partial, c->diag_blocks, 5, c->diag_out, c->st);
   int r = launched(c, "fluid sums", 2);
   if (r || c->np == 0) return r;
@@ -560,7 +572,9 @@ int one_step(lbmd_ctx *c, unsigned long long step, cudaEvent_t t0, cudaEvent_t t
   float *rho = c->rho_buf[c->cur];
   int r;
   const bool sub = P.np > 0 && P.substeps > 1;
-  const bool onepass = uses_onepass(c);
+  const bool onepass = uses_onepass(c), small = uses_one_launch(c);
+  const float *rest_in = c->rest[c->cur];
+  float *rest_out = c->rest[1 - c->cur];
   if (P.np > 0 && !sub && !c->sort_pending) {
     // fork the side stream from the step's start (while st records a graph, this is also what
     // makes the side stream's work part of the graph); after a sort still pending there, the side
@@ -570,9 +584,9 @@ int one_step(lbmd_ctx *c, unsigned long long step, cudaEvent_t t0, cudaEvent_t t
   }
   if (onepass) {
     if (!c->rho_valid) return fail(c, LBMD_E_STATE, "one-pass update without the densities of the current state");
-  } else {
+  } else if (!small) {
     // densities (and j' for the particle coupling) of this step's populations
-    launch_moments(P, fin, c->rest, rho, P.np > 0 ? c->jp : nullptr, c->st);
+    launch_moments(P, fin, rest_in, rho, P.np > 0 ? c->jp : nullptr, c->st);
     if ((r = launched(c, "moments"))) return r;
   }
   if (P.np > 0 && c->sort_pending) {  // the previous step's sort of these particles
@@ -607,17 +621,19 @@ int one_step(lbmd_ctx *c, unsigned long long step, cudaEvent_t t0, cudaEvent_t t
   }
   if (t0) CK(cudaEventRecordWithFlags(t0, c->st, flags), "event");
   if (onepass)
-    launch_collide_onepass(P, fin, fout, c->rest, rho, c->rho_buf[1 - c->cur],
+    launch_collide_onepass(P, fin, fout, rest_in, rest_out, rho, c->rho_buf[1 - c->cur],
                            c->op_out, gpa, gpf, gci, c->err, c->op_geom,
                            c->op_grid, c->st);
+  else if (small)
+    launch_step_small(P, fin, fout, rest_in, rest_out, c->err, c->st);
   else
-    launch_collide(P, fin, fout, c->rest, rho, gpa, gpf, gci, c->err, c->st);
+    launch_collide(P, fin, fout, rest_in, rest_out, rho, gpa, gpf, gci, c->err, c->st);
   if ((r = launched(c, "collide"))) return r;
   if (t1) CK(cudaEventRecordWithFlags(t1, c->st, flags), "event");
   const bool corner_j = onepass && P.np > 0 && !sub;  // the boundary kernel forms the next step's jc
   if (onepass) {
     if (corner_j) CK(cudaStreamWaitEvent(c->st, c->ev_integrated, 0), "stream wait");
-    launch_boundary_densities(P, c->op_geom, fout, c->rest, c->rho_buf[1 - c->cur], c->op_runs, c->op_nruns,
+    launch_boundary_densities(P, c->op_geom, fout, rest_out, c->rho_buf[1 - c->cur], c->op_runs, c->op_nruns,
                               c->op_out, c->op_zslot, c->pt, corner_j ? P.np : 0,
                               corner_j ? c->jc : nullptr, c->st);
     if ((r = launched(c, "boundary densities"))) return r;
@@ -805,7 +821,8 @@ int lbmd_create(const lbmd_params *prm, void *stream, lbmd_ctx **out, unsigned *
       (e = dalloc(&c->rho_buf[0], (size_t)2 * P.N)) != cudaSuccess ||
       (e = dalloc(&c->rho_buf[1], (size_t)2 * P.N)) != cudaSuccess || (e = dalloc(&c->jp, (size_t)3 * P.N)) != cudaSuccess ||
       (e = dalloc(&c->err, 1)) != cudaSuccess ||
-      (c->pop_elem == 2 && (e = dalloc(&c->rest, (size_t)2 * P.N)) != cudaSuccess)) {
+      (c->pop_elem == 2 && (e = dalloc(&c->rest[0], (size_t)2 * P.N)) != cudaSuccess) ||
+      (c->pop_elem == 2 && small_lattice(P) && (e = dalloc(&c->rest[1], (size_t)2 * P.N)) != cudaSuccess)) {
     cudaGetLastError();
     lbmd_destroy(c);
     return fail(nullptr, e == cudaErrorMemoryAllocation ? LBMD_E_NOMEM : LBMD_E_CUDA,
@@ -821,6 +838,7 @@ int lbmd_create(const lbmd_params *prm, void *stream, lbmd_ctx **out, unsigned *
     lbmd_destroy(c);
     return fail(nullptr, LBMD_E_CUDA, std::string("stream / event creation: ") + cudaGetErrorString(e));
   }
+  if (!c->rest[1]) c->rest[1] = c->rest[0];
   c->diag_blocks = fluid_sum_blocks(P);
   if ((e = dalloc(&c->diag_partial, (size_t)5 * c->diag_blocks)) != cudaSuccess ||
       (e = dalloc(&c->diag_out, 8)) != cudaSuccess || (e = dalloc(&c->drift, 10)) != cudaSuccess ||
@@ -857,7 +875,8 @@ void lbmd_destroy(lbmd_ctx *c) {
     if (e) cudaEventDestroy(e);
   dfree(c->step_base);
   dfree(c->pop[0]); dfree(c->pop[1]); dfree(c->rho_buf[0]); dfree(c->rho_buf[1]); dfree(c->jp); dfree(c->err);
-  dfree(c->rest);
+  if (c->rest[1] == c->rest[0]) c->rest[1] = nullptr;
+  dfree(c->rest[0]); dfree(c->rest[1]);
   free_onepass(c);
   dfree(c->diag_partial); dfree(c->diag_out); dfree(c->drift);
   free_particles(c);
@@ -908,7 +927,7 @@ int lbmd_init_fluid(lbmd_ctx *c, const float *rhoA, const float *rhoB, const flo
     CK(cudaMemcpyAsync(stage + 2 * N, u, 3 * bytes, cudaMemcpyHostToDevice, c->st), "upload u");
     du = stage + 2 * N;
   }
-  launch_init_equilibrium(c->P, stage, stage + N, du, c->pop[c->cur], c->rest, c->st);
+  launch_init_equilibrium(c->P, stage, stage + N, du, c->pop[c->cur], c->rest[c->cur], c->st);
   int r = launched(c, "init_equilibrium");
   if (r) return r;
   c->steps = 0;
@@ -928,7 +947,7 @@ int lbmd_set_populations(lbmd_ctx *c, int comp, const float *f) {
   drop_graphs(c);
   float *stage = reinterpret_cast<float *>(c->pop[1 - c->cur]);
   CK(cudaMemcpyAsync(stage, f, sizeof(float) * kQ * (size_t)c->P.N, cudaMemcpyHostToDevice, c->st), "upload f");
-  launch_restream(c->P, stage, comp, c->pop[c->cur], c->rest, c->st);
+  launch_restream(c->P, stage, comp, c->pop[c->cur], c->rest[c->cur], c->st);
   int r = launched(c, "restream");
   if (r) return r;
   c->rho_valid = false;
@@ -944,7 +963,7 @@ int lbmd_get_populations(lbmd_ctx *c, int comp, float *f) {
   if (!c->fluid_ready) return fail(c, LBMD_E_STATE, "fluid not initialised");
   cudaSetDevice(c->dev);
   float *stage = reinterpret_cast<float *>(c->pop[1 - c->cur]);
-  launch_unstream(c->P, c->pop[c->cur], c->rest, comp, stage, c->st);
+  launch_unstream(c->P, c->pop[c->cur], c->rest[c->cur], comp, stage, c->st);
   int r = launched(c, "unstream");
   if (r) return r;
   CK(cudaMemcpyAsync(f, stage, sizeof(float) * kQ * (size_t)c->P.N, cudaMemcpyDeviceToHost, c->st), "download f");
@@ -1170,7 +1189,7 @@ int lbmd_get_fields(lbmd_ctx *c, float *rhoA, float *rhoB, float *u) {
   float *stage = reinterpret_cast<float *>(c->pop[1 - c->cur]);
   int r = ensure_densities(c);
   if (r) return r;
-  launch_fields(c->P, c->pop[c->cur], c->rest, c->rho_buf[c->cur], stage, stage + N, u ? stage + 2 * N : nullptr, c->st);
+  launch_fields(c->P, c->pop[c->cur], c->rest[c->cur], c->rho_buf[c->cur], stage, stage + N, u ? stage + 2 * N : nullptr, c->st);
   if ((r = launched(c, "fields"))) return r;
   const size_t bytes = sizeof(float) * (size_t)N;
   if (rhoA) CK(cudaMemcpyAsync(rhoA, stage, bytes, cudaMemcpyDeviceToHost, c->st), "download");
@@ -1258,7 +1277,7 @@ int lbmd_get_fields_dev(lbmd_ctx *c, float *rhoA, float *rhoB, float *u, void *s
   const cudaStream_t caller = static_cast<cudaStream_t>(stream);
   if ((r = dev_getter_begin(c, caller))) return r;
   if ((r = ensure_densities(c))) return r;
-  launch_fields(c->P, c->pop[c->cur], c->rest, c->rho_buf[c->cur], rhoA, rhoB, u, c->st);
+  launch_fields(c->P, c->pop[c->cur], c->rest[c->cur], c->rho_buf[c->cur], rhoA, rhoB, u, c->st);
   if ((r = launched(c, "fields"))) return r;
   return dev_getter_end(c, caller);
 }
@@ -1271,7 +1290,7 @@ int lbmd_get_populations_dev(lbmd_ctx *c, int comp, float *f, void *stream) {
   if ((r = dev_buffers_ok(c, "f_dev", f, sizeof(float) * kQ * (size_t)c->P.N))) return r;
   const cudaStream_t caller = static_cast<cudaStream_t>(stream);
   if ((r = dev_getter_begin(c, caller))) return r;
-  launch_unstream(c->P, c->pop[c->cur], c->rest, comp, f, c->st);
+  launch_unstream(c->P, c->pop[c->cur], c->rest[c->cur], comp, f, c->st);
   if ((r = launched(c, "unstream"))) return r;
   return dev_getter_end(c, caller);
 }

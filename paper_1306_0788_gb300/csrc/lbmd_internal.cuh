@@ -280,14 +280,18 @@ void launch_unstream(const StepParams &P, const void *store, const float *rest, 
                      cudaStream_t st);
 void launch_moments(const StepParams &P, const void *store, const float *rest, float *rho, float *jp,
                     cudaStream_t st);
-void launch_collide(const StepParams &P, const void *fin, void *fout, float *rest, const float *rho,
-                    const ParticleArrays &pa, const ParticleForces &pf, CellIndex ci, unsigned *err,
+void launch_collide(const StepParams &P, const void *fin, void *fout, const float *rest_in, float *rest_out,
+                    const float *rho, const ParticleArrays &pa, const ParticleForces &pf, CellIndex ci, unsigned *err,
                     cudaStream_t st);
+// Density pass and update of a small lattice without particles in one launch.  rest_in and rest_out must
+// not be the same buffer: blocks read the rest populations of nodes that others update.
+void launch_step_small(const StepParams &P, const void *fin, void *fout, const float *rest_in, float *rest_out,
+                       unsigned *err, cudaStream_t st);
 // One-pass update (BGK, md_substeps = 1): writes the populations of the next step, the densities
 // rho_next of the nodes whose sources are all in one block, and the partial sums of `out` for the
 // others; launch_boundary_densities then finishes those.
-void launch_collide_onepass(const StepParams &P, const void *fin, void *fout, float *rest, const float *rho,
-                            float *rho_next, OnePassOut out, const ParticleArrays &pa, const ParticleForces &pf,
+void launch_collide_onepass(const StepParams &P, const void *fin, void *fout, const float *rest_in, float *rest_out,
+                            const float *rho, float *rho_next, OnePassOut out, const ParticleArrays &pa, const ParticleForces &pf,
                             CellIndex ci, unsigned *err, OnePassGeom G, int grid, cudaStream_t st);
 // Adds the partial sums of `out` where they belong and pulls the densities of the listed boundary
 // runs from the new populations, in one launch.  zslot[z]: -1 where z is neither the first nor the
