@@ -16,6 +16,20 @@ namespace lbmd {
 namespace {
 
 constexpr int kBlock = 256;
+// Blocks of the density pass and of the two-pass update, which wait for nothing within a block: small
+// ones on large lattices, whose warps' slots are free again sooner (with 256 threads the slots of an
+// update block stayed taken until its last warp was done: 17.7 of 24 warps active at 160^3).  Ten steps
+// at 256^3 with the update in blocks of 256 / 128 / 64 / 32 threads: FP16 9.29 / 8.70 / 8.61 / 8.68 ms,
+// fluctuating MRT 15.37 / 15.07 / 15.01 / 15.39; twenty of 100x90x110 MRT 2133 / 2101 / 2095 / 2155 us;
+// 64 threads and the density pass in 256 / 128 / 64: FP16 8.61 / 8.58 / 8.58 ms.  A small lattice is
+// launched in few waves, and starting more blocks costs it more: fifty steps of 64^3 1120 / 1111 / 1123 us,
+// of 32^3 573 in 256 and 603 in 64; with the update of reaction records, whose blocks share the rows they
+// search, ten steps of 80^3 take 14 % longer in 64 than in 256.  (More than 24 update warps an SM leave
+// too few registers: 26 take 8.78 and 15.29 ms.)
+constexpr long long kSmallBlocksFrom = 1 << 19;  // nodes
+constexpr int kMomentsBlock = 128;
+constexpr int kCollideBlock = 64;
+constexpr int kUpdateThreads = 768;  // threads of the update per SM, 80 registers each
 
 using namespace site;
 
@@ -92,11 +106,11 @@ __global__ void __launch_bounds__(kBlock) k_moments(StepParams P, const T *__res
 }
 
 // The lattice update of one step at every site (site::collide; with kMRT the fluctuating MRT
-// collision, whose mode transforms spill a few registers at this budget of three blocks per SM
-// but run faster than without spills at two; with kBisect the gather over the sub-stepping
+// collision, whose mode transforms spill a few registers at this budget of 24 warps per SM
+// but run faster than without spills at 16; with kBisect the gather over the sub-stepping
 // reaction records).
-template <class T, bool kParticles, bool kMRT, bool kBisect = false>
-__global__ void __launch_bounds__(kBlock, 3) k_collide(StepParams P, const T *__restrict__ fin,
+template <class T, bool kParticles, bool kMRT, bool kBisect = false, int kThreads = kBlock>
+__global__ void __launch_bounds__(kThreads, kUpdateThreads / kThreads) k_collide(StepParams P, const T *__restrict__ fin,
                                                                   T *__restrict__ fout, const float *__restrict__ rho,
                                                                   ParticleArrays pa, ParticleForces pf, CellIndex ci,
                                                                   unsigned *err, const float *__restrict__ rest_in,
@@ -742,7 +756,7 @@ __global__ void k_drift_check(const double *__restrict__ sums, const double *__r
   if (!(dA <= tol) || !(dB <= tol) || !(dP <= tol)) atomicOr(err, kErrDrift);
 }
 
-inline unsigned grid_for(long long n) { return (unsigned)((n + kBlock - 1) / kBlock); }
+inline unsigned grid_for(long long n, int block = kBlock) { return (unsigned)((n + block - 1) / block); }
 
 }  // namespace
 
@@ -780,7 +794,8 @@ void launch_moments(const StepParams &P, const void *store, const float *rest, f
                     cudaStream_t st) {
   with_storage(P, [&](auto t) {
     using T = std::remove_pointer_t<decltype(t)>;
-    k_moments<T><<<grid_for(P.N), kBlock, 0, st>>>(P, static_cast<const T *>(store), rest, rho, jp);
+    const int block = P.N >= kSmallBlocksFrom ? kMomentsBlock : kBlock;
+    k_moments<T><<<grid_for(P.N, block), block, 0, st>>>(P, static_cast<const T *>(store), rest, rho, jp);
   });
 }
 void launch_step_small(const StepParams &P, const void *fin, void *fout, const float *rest_in, float *rest_out,
@@ -803,19 +818,16 @@ void launch_collide(const StepParams &P, const void *fin, void *fout, const floa
     const T *a = static_cast<const T *>(fin);
     T *b = static_cast<T *>(fout);
     const bool mrt = P.collision == LBMD_COLLISION_MRT;
-    const bool records = P.np > 0 && P.substeps > 1;
-    if (records && mrt)
-      k_collide<T, true, true, true><<<grid_for(P.N), kBlock, 0, st>>>(P, a, b, rho, pa, pf, ci, err, rest_in, rest_out);
-    else if (records)
-      k_collide<T, true, false, true><<<grid_for(P.N), kBlock, 0, st>>>(P, a, b, rho, pa, pf, ci, err, rest_in, rest_out);
-    else if (P.np > 0 && mrt)
-      k_collide<T, true, true><<<grid_for(P.N), kBlock, 0, st>>>(P, a, b, rho, pa, pf, ci, err, rest_in, rest_out);
-    else if (P.np > 0)
-      k_collide<T, true, false><<<grid_for(P.N), kBlock, 0, st>>>(P, a, b, rho, pa, pf, ci, err, rest_in, rest_out);
-    else if (mrt)
-      k_collide<T, false, true><<<grid_for(P.N), kBlock, 0, st>>>(P, a, b, rho, pa, pf, ci, err, rest_in, rest_out);
-    else
-      k_collide<T, false, false><<<grid_for(P.N), kBlock, 0, st>>>(P, a, b, rho, pa, pf, ci, err, rest_in, rest_out);
+    const bool records = P.np > 0 && P.substeps > 1, parts = P.np > 0;
+    constexpr int kC = kCollideBlock;
+    const bool large = P.N >= kSmallBlocksFrom && !records;
+    const int block = large ? kC : kBlock;
+    auto *kernel = records ? (mrt ? k_collide<T, true, true, true> : k_collide<T, true, false, true>)
+                   : large ? (parts ? (mrt ? k_collide<T, true, true, false, kC> : k_collide<T, true, false, false, kC>)
+                                    : (mrt ? k_collide<T, false, true, false, kC> : k_collide<T, false, false, false, kC>))
+                           : (parts ? (mrt ? k_collide<T, true, true> : k_collide<T, true, false>)
+                                    : (mrt ? k_collide<T, false, true> : k_collide<T, false, false>));
+    kernel<<<grid_for(P.N, block), block, 0, st>>>(P, a, b, rho, pa, pf, ci, err, rest_in, rest_out);
   });
 }
 
@@ -867,10 +879,10 @@ int onepass_blocks_per_sm() {
 
 template <class T>
 bool is_noisy_update_of(const void *fn) {
-  return fn == reinterpret_cast<const void *>(&k_collide<T, true, true, true>) ||
-         fn == reinterpret_cast<const void *>(&k_collide<T, true, true>) ||
-         fn == reinterpret_cast<const void *>(&k_collide<T, false, true>) ||
-         fn == reinterpret_cast<const void *>(&k_step_small<T, true>);
+  auto is = [fn](auto *kernel) { return fn == reinterpret_cast<const void *>(kernel); };
+  return is(&k_collide<T, true, true, true>) || is(&k_collide<T, true, true>) || is(&k_collide<T, false, true>) ||
+         is(&k_collide<T, true, true, false, kCollideBlock>) || is(&k_collide<T, false, true, false, kCollideBlock>) ||
+         is(&k_step_small<T, true>);
 }
 
 bool is_noisy_update(const void *fn) {

@@ -10,8 +10,7 @@ from paper_1306_0788_gb300 import inputs
 pytestmark = pytest.mark.gpu
 
 
-def _case(particles, **more):
-    dims = (16, 14, 18)
+def _case(particles, dims=(16, 14, 18), **more):
     rA, rB = inputs.flat_slab(dims, 1.8586, 0.1414)  # coexistence at g rho = 1.5
     x = inputs.spaced_particles(particles, dims, 2.5, seed=4)
     c = Case(dims=dims, g=1.5, kT=1e-4, seed=9, rhoA=rA, rhoB=rB, x=x, v=np.zeros_like(x),
@@ -43,5 +42,15 @@ def _run(c, graphs, schedule):
 def test_long_graphs_are_bit_identical(c, schedule):
     a, b = _run(c, True, schedule), _run(c, False, schedule)
     assert a[1] == b[1] == sum(schedule)
+    for x, y in zip(a, b):
+        assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("nz,storage,collision", [(64, 0, 1), (63, 0, 1), (64, 1, 0)])
+def test_large_and_small_update_blocks(nz, storage, collision):
+    """From 2^19 nodes (128 x 64 x 64) the update runs in blocks of 64 threads: its noise counter is
+    patched in the graphs as that of the 256-thread one below."""
+    c = _case(300, dims=(128, 64, nz), storage=storage, collision=collision, rho0=(1.0, 1.0))
+    a, b = _run(c, True, (3, 4)), _run(c, False, (3, 4))
     for x, y in zip(a, b):
         assert np.array_equal(x, y)
