@@ -1367,7 +1367,7 @@ int lbmd_batch_get_fields(lbmd_batch *b, int slot, float *rhoA, float *rhoB, flo
   const int cur = sl.mirror.cur;
   const long long N = sl.P.N;
   float *stage = reinterpret_cast<float *>(sl.pop[1 - cur]);
-  launch_moments(sl.P, sl.pop[cur], sl.rest, sl.rho, nullptr, b->st);
+  launch_moments(sl.P, sl.pop[cur], sl.rest, sl.rho, nullptr, nullptr, b->st);
   launch_fields(sl.P, sl.pop[cur], sl.rest, sl.rho, stage, stage + N, u ? stage + 2 * N : nullptr, b->st);
   BK(cudaGetLastError(), "fields");
   const size_t bytes = sizeof(float) * (size_t)N;

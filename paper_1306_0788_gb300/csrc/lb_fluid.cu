@@ -99,10 +99,10 @@ __global__ void __launch_bounds__(kBlock) k_unstream(StepParams P, const T *__re
 template <class T>
 __global__ void __launch_bounds__(kBlock) k_moments(StepParams P, const T *__restrict__ fin,
                                                     const float *__restrict__ rest, float *__restrict__ rho,
-                                                    float *__restrict__ jp) {
+                                                    float *__restrict__ jp, const unsigned *__restrict__ node_bits) {
   const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= P.N) return;
-  moments(P, s, fin, rest, rho, jp);
+  moments(P, s, fin, rest, rho, jp, node_bits);
 }
 
 // The lattice update of one step at every site (site::collide; with kMRT the fluctuating MRT
@@ -791,11 +791,11 @@ void launch_unstream(const StepParams &P, const void *store, const float *rest, 
   });
 }
 void launch_moments(const StepParams &P, const void *store, const float *rest, float *rho, float *jp,
-                    cudaStream_t st) {
+                    const unsigned *node_bits, cudaStream_t st) {
   with_storage(P, [&](auto t) {
     using T = std::remove_pointer_t<decltype(t)>;
     const int block = P.N >= kSmallBlocksFrom ? kMomentsBlock : kBlock;
-    k_moments<T><<<grid_for(P.N, block), block, 0, st>>>(P, static_cast<const T *>(store), rest, rho, jp);
+    k_moments<T><<<grid_for(P.N, block), block, 0, st>>>(P, static_cast<const T *>(store), rest, rho, jp, node_bits);
   });
 }
 void launch_step_small(const StepParams &P, const void *fin, void *fout, const float *rest_in, float *rest_out,

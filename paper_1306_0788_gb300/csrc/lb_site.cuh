@@ -304,14 +304,24 @@ __device__ __forceinline__ NodeMoments node_moments(const StepParams &P, const C
   return NodeMoments{rA, rB, jx, jy, jz};
 }
 
-// node_moments of site s, the densities stored interleaved (rho_A, rho_B), j' when jp is not NULL.
+// Whether a particle's cell has the node c as a corner (CellIndex::node_bits).
+__device__ __forceinline__ bool node_touched(const StepParams &P, const Coord &c, const unsigned *node_bits) {
+  return __ldg(node_bits + (c.z * P.ny + c.y) * node_words(P.nx) + (c.x >> 5)) >> (c.x & 31) & 1u;
+}
+
+// node_moments of site s, the densities stored interleaved (rho_A, rho_B), j' when jp is not NULL: at
+// every node, or with node_bits at those that a particle's coupling reads (at 256^3 with 20,000 particles
+// the 12 bytes per node take 7 of 235 us in FP16, 16 of 392 in FP32).  The bit is looked up first: after
+// the sums, its latency came on top of theirs (24 us more instead of 16 less).
 template <class T>
 __device__ __forceinline__ void moments(const StepParams &P, long long s, const T *__restrict__ fin,
                                         const float *__restrict__ rest, float *__restrict__ rho,
-                                        float *__restrict__ jp) {
-  const NodeMoments n = node_moments(P, site_coord(P, s), (unsigned)s, fin, rest);
+                                        float *__restrict__ jp, const unsigned *__restrict__ node_bits = nullptr) {
+  const Coord c = site_coord(P, s);
+  const bool want = jp && (!node_bits || node_touched(P, c, node_bits));
+  const NodeMoments n = node_moments(P, c, (unsigned)s, fin, rest);
   reinterpret_cast<float2 *>(rho)[s] = make_float2(n.rA, n.rB);
-  if (jp) {
+  if (want) {
     jp[s] = n.jx;
     jp[P.N + s] = n.jy;
     jp[2 * P.N + s] = n.jz;
@@ -698,7 +708,7 @@ __device__ __forceinline__ void collide_core_at(const StepParams &P, const Coord
   // four rows of every node instead cost the update at 256^3 with 20,000 particles 50 of 1056 us
   // (fluctuating MRT, bound by instruction issue), 9 of 878 (one pass, FP32), 4 of 580 (FP16), and
   // the batched update of 24 replicas about 30 of 800.
-  if (kParticles && (__ldg(ci.node_bits + (c.z * P.ny + c.y) * node_words(P.nx) + (c.x >> 5)) >> (c.x & 31) & 1u))
+  if (kParticles && node_touched(P, c, ci.node_bits))
     gather_coupling<kBisect>(P, c.x, c.y, c.z, rA, rB, pa, pf, ci, true, gA, gB);
   const float r = rA + rB;
   if (!(rA > 0.f) || !(rB > 0.f) || !isfinite(r)) atomicOr(err, isfinite(r) ? kErrNegDensity : kErrNonFinite);

@@ -421,7 +421,7 @@ int prepare_onepass(lbmd_ctx *c) {
 // The densities of the current state into rho_buf[cur] (a density pass), if not there already.
 int ensure_densities(lbmd_ctx *c) {
   if (c->rho_valid) return LBMD_OK;
-  launch_moments(c->P, c->pop[c->cur], c->rest[c->cur], c->rho_buf[c->cur], nullptr, c->st);
+  launch_moments(c->P, c->pop[c->cur], c->rest[c->cur], c->rho_buf[c->cur], nullptr, nullptr, c->st);
   const int r = launched(c, "moments");
   if (!r) c->rho_valid = true;
   return r;
@@ -554,6 +554,19 @@ int reserve_events(lbmd_ctx *c, size_t n) {
   return LBMD_OK;
 }
 
+// st waits for a sort still pending on side.
+int join_sort(lbmd_ctx *c) {
+  if (!c->sort_pending) return LBMD_OK;
+  CK(cudaStreamWaitEvent(c->st, c->ev_sorted, 0), "stream wait");
+  c->sort_pending = false;
+  return LBMD_OK;
+}
+
+// From this size on j' is stored at the marked nodes only, which needs the sort of the particles before
+// the density pass.  Ten steps at 256^3: FP16 8575 -> 8529 us, fluctuating MRT 15000 -> 14857; twenty of
+// 100x90x110, whose update is too short to hide the sort, 2087 -> 2153.
+constexpr long long kMarkedFrom = 1 << 22;  // nodes
+
 // One coupled step on st and side.  `step` is the noise counter the kernels get: the lattice
 // step, or, while a graph is recorded, the step's offset in it (the kernels add the base).
 // t0, t1 (or null): events recorded around the lattice update, with `flags`.
@@ -585,14 +598,15 @@ int one_step(lbmd_ctx *c, unsigned long long step, cudaEvent_t t0, cudaEvent_t t
   if (onepass) {
     if (!c->rho_valid) return fail(c, LBMD_E_STATE, "one-pass update without the densities of the current state");
   } else if (!small) {
-    // densities (and j' for the particle coupling) of this step's populations
-    launch_moments(P, fin, rest_in, rho, P.np > 0 ? c->jp : nullptr, c->st);
+    // densities (and j' for the particle coupling) of this step's populations; on large lattices j'
+    // only at the nodes the sorted particles mark, whose sort the lattice update before has hidden
+    // (with MD sub-stepping at every node: the particles move on within the step)
+    const bool marked = P.np > 0 && !sub && P.N >= kMarkedFrom;
+    if (marked && (r = join_sort(c))) return r;
+    launch_moments(P, fin, rest_in, rho, P.np > 0 ? c->jp : nullptr, marked ? ci.node_bits : nullptr, c->st);
     if ((r = launched(c, "moments"))) return r;
   }
-  if (P.np > 0 && c->sort_pending) {  // the previous step's sort of these particles
-    CK(cudaStreamWaitEvent(c->st, c->ev_sorted, 0), "stream wait");
-    c->sort_pending = false;
-  }
+  if ((r = join_sort(c))) return r;
   ParticleArrays gpa = c->pa[c->pcur];  // what the update gathers the momentum return from
   ParticleForces gpf = c->pf;
   CellIndex gci = ci;
@@ -638,10 +652,7 @@ int one_step(lbmd_ctx *c, unsigned long long step, cudaEvent_t t0, cudaEvent_t t
                               corner_j ? c->jc : nullptr, c->st);
     if ((r = launched(c, "boundary densities"))) return r;
   }
-  if (P.np > 0 && join) {
-    CK(cudaStreamWaitEvent(c->st, c->ev_sorted, 0), "stream wait");
-    c->sort_pending = false;
-  }
+  if (join && (r = join_sort(c))) return r;
   c->cur = 1 - c->cur;
   c->steps++;
   c->rho_valid = onepass;  // the two-pass update leaves the new state's densities to its next step

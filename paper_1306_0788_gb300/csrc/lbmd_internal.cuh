@@ -278,8 +278,9 @@ void launch_init_equilibrium(const StepParams &P, const float *rhoA, const float
 void launch_restream(const StepParams &P, const float *post, int comp, void *store, float *rest, cudaStream_t st);
 void launch_unstream(const StepParams &P, const void *store, const float *rest, int comp, float *post,
                      cudaStream_t st);
+// jp (or null): j', at every node or (node_bits not null) at the nodes whose bit is set.
 void launch_moments(const StepParams &P, const void *store, const float *rest, float *rho, float *jp,
-                    cudaStream_t st);
+                    const unsigned *node_bits, cudaStream_t st);
 void launch_collide(const StepParams &P, const void *fin, void *fout, const float *rest_in, float *rest_out,
                     const float *rho, const ParticleArrays &pa, const ParticleForces &pf, CellIndex ci, unsigned *err,
                     cudaStream_t st);
