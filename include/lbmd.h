@@ -422,14 +422,15 @@ int lbmd_batch_get_drift(lbmd_batch *batch, int slot, double out[5]);
  * [256, 65536]), the persistent grid of the density pass and of the update (in [1, 64 x SM
  * count]), and the register budget of the update, collide_blocks = 3 (80 registers, three
  * blocks of 256 threads per SM) or 2 (up to 128 registers).  cfg[5] = {tile_sites,
- * grid_moments, grid_collide, collide_blocks, grid_particles}.  Results do not depend on it. */
+ * grid_moments, grid_collide, collide_blocks, grid_particles}.  Results do not depend on it.  Until it is
+ * set or tuned, the tile size follows the number of sites whenever replicas join or leave. */
 int lbmd_batch_set_config(lbmd_batch *batch, int tile_sites, int grid_moments, int grid_collide,
                           int collide_blocks);
 int lbmd_batch_get_config(const lbmd_batch *batch, int cfg[5]);
 
 /* Autotuner: times the lattice kernels over the current replicas for tiles of 256, 1024 and
  * 4096 sites, density-pass grids of 2/3/4 blocks per SM and update variants (register budget
- * of 3 blocks per SM with grids of 1/2/3 blocks per SM, of 2 blocks per SM with 1/2), keeps
+ * of 3 blocks per SM with grids of 1/2/3 blocks per SM, of 2 blocks per SM with 1/2/8), keeps
  * the fastest, and returns it in cfg[5] and the two kernel times in ms[2] (either may be
  * NULL).  The state of the replicas is unchanged.  Needs at least one initialised replica. */
 int lbmd_batch_tune(lbmd_batch *batch, int cfg[5], double ms[2]);

@@ -69,7 +69,11 @@ struct BatchDev {
   ParticleArrays S;      // the same particles sorted by (row, x cell, id) during a step
   ParticleForces pf;     // forces, indexed like S (and like U after the update)
   int *row_of, *row_count, *row_start, *row_cursor, *bsum, *perm;
-  unsigned *node_bits;   // [nwords] CellIndex::node_bits of the replicas with particles
+  // CellIndex::node_bits of the replicas with particles, [nwords] for the present step at
+  // node_bits[*parity] (set from the particles' positions by the step before, or by a repack); the
+  // other half is cleared and takes the next step's
+  unsigned *node_bits[2];
+  int *parity;
   int nwords;
   double *tile_sums;     // [ntiles][5] FP64 sums of the drift check
   double *drift;         // [max_slots][10]: reference totals [5], last check {step, dA, dB, dP, n}
@@ -130,7 +134,8 @@ __device__ __forceinline__ void fill_tile(TileCtx<T> &c, const BatchDev *__restr
     c.rho = R.rho;
     c.jp = R.P.np > 0 ? R.jp : nullptr;
     c.err = &B->state[slot].err;
-    c.ci = CellIndex{(!tuning && R.P.np > 0) ? B->row_start + L.row0 : nullptr, B->node_bits + L.bits0};
+    c.ci = CellIndex{(!tuning && R.P.np > 0) ? B->row_start + L.row0 : nullptr,
+                     B->node_bits[*B->parity] + L.bits0};
     c.base = (long long)(t - L.tile0) * B->tile_sites;
     c.step = B->state[slot].step;
     c.pa = B->S;
@@ -163,7 +168,7 @@ __global__ void __launch_bounds__(kBThreads, 4) kb_moments(const BatchDev *__res
     for (int k = threadIdx.x; k < ts; k += kBThreads) {
       const long long s = c.base + k;
       if (s >= c.P.N) break;
-      site::moments<T>(c.P, s, c.fin, c.rest_in, c.rho, c.jp);
+      site::moments<T>(c.P, s, c.fin, c.rest_in, c.rho, c.jp, c.ci.node_bits);
     }
     __syncthreads();  // the next context is complete; this one is free for the tile after it
     t = tn;
@@ -206,10 +211,23 @@ __global__ void __launch_bounds__(kBThreads, kMinBlocks) kb_collide(const BatchD
 
 // ------------------------------------------------------------------ particle sort
 
-// (also clears the node bits, which kb_permute sets anew)
+// Sets the node bits of the particle of `slot` in cell c.
+__device__ __forceinline__ void mark_nodes(const BatchDev *__restrict__ B, int slot, int4 c, unsigned *node_bits) {
+  unsigned *bits = node_bits + B->lay[slot].bits0;
+  site::for_corner_bits(B->rep[slot].P, c, [&](long long w, unsigned b) { atomicOr(bits + w, b); });
+}
+
+// After a repack: the node bits of the present positions.
+__global__ void __launch_bounds__(kBPThreads) kb_mark(const BatchDev *__restrict__ B) {
+  unsigned *bits = B->node_bits[*B->parity];
+  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < B->np; p += gridDim.x * blockDim.x)
+    mark_nodes(B, B->pslot[p], B->U.cell[p], bits);
+}
+
+// (also clears the next step's node bits, which kb_integrate sets)
 __global__ void __launch_bounds__(kBPThreads) kb_bin(const BatchDev *__restrict__ B) {
   const int np = B->np, nwords = B->nwords;
-  unsigned *bits = B->node_bits;
+  unsigned *bits = B->node_bits[*B->parity ^ 1];
   for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < nwords; w += gridDim.x * blockDim.x) bits[w] = 0u;
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < np; p += gridDim.x * blockDim.x) {
     const int slot = B->pslot[p];
@@ -335,15 +353,12 @@ __global__ void __launch_bounds__(kBPThreads) kb_row_sort(const BatchDev *__rest
 __global__ void __launch_bounds__(kBPThreads) kb_permute(const BatchDev *__restrict__ B) {
   const int np = B->np;
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < np; j += gridDim.x * blockDim.x) {
-    const int p = B->perm[j], slot = B->pslot[j];
-    const int4 c = B->U.cell[p];
-    unsigned *bits = B->node_bits + B->lay[slot].bits0;
-    site::for_corner_bits(B->rep[slot].P, c, [&](long long w, unsigned b) { atomicOr(bits + w, b); });
-    B->S.cell[j] = c;
+    const int p = B->perm[j];
+    B->S.cell[j] = B->U.cell[p];
     B->S.frac[j] = B->U.frac[p];
     B->S.vel[j] = B->U.vel[p];
     B->S.pid[j] = B->U.pid[p];
-    if (B->left[slot] <= 0) B->pf.fric[j] = B->pf.total[p];
+    if (B->left[B->pslot[j]] <= 0) B->pf.fric[j] = B->pf.total[p];
   }
 }
 
@@ -382,23 +397,27 @@ __global__ void __launch_bounds__(kBPThreads) kb_pairs(const BatchDev *__restric
 // S -> U: the update for replicas still stepping, a plain copy for frozen ones.
 __global__ void __launch_bounds__(kBPThreads) kb_integrate(const BatchDev *__restrict__ B) {
   const int np = B->np;
+  unsigned *bits = B->node_bits[*B->parity ^ 1];  // the next step's
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < np; p += gridDim.x * blockDim.x) {
     const int slot = B->pslot[p];
     if (B->left[slot] <= 0) {
-      B->U.cell[p] = B->S.cell[p];
+      const int4 c = B->S.cell[p];
+      mark_nodes(B, slot, c, bits);
+      B->U.cell[p] = c;
       B->U.frac[p] = B->S.frac[p];
       B->U.vel[p] = B->S.vel[p];
       B->U.pid[p] = B->S.pid[p];
       B->pf.total[p] = B->pf.fric[p];
       continue;
     }
-    site::integrate(B->rep[slot].P, p, B->S, B->U, B->pf, &B->state[slot].err);
+    mark_nodes(B, slot, site::integrate(B->rep[slot].P, p, B->S, B->U, B->pf, &B->state[slot].err), bits);
   }
 }
 
 // End of a step: replicas that stepped swap buffers and count the step; a replica with a device
 // error stops (its remaining steps are dropped).
 __global__ void kb_advance(const BatchDev *__restrict__ B) {
+  if (threadIdx.x == 0) *B->parity ^= 1;
   for (int r = threadIdx.x; r < B->nrep; r += blockDim.x) {
     const int slot = B->rep_slot[r];
     if (B->left[slot] <= 0) continue;
@@ -583,7 +602,7 @@ struct lbmd_batch {
   // the particle sort and the pair forces run on a side stream beside the density pass (joined
   // into st within every captured step; see enqueue_step)
   cudaStream_t side = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_sorted = nullptr, ev_pairs = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_sorted = nullptr, ev_coupled = nullptr, ev_moved = nullptr;
   bool own_stream = false;
   size_t budget = 0, used = 0;
   int storage = 0;
@@ -610,9 +629,10 @@ struct lbmd_batch {
   double *d_drift = nullptr;  // [max_slots][10] (BatchDev::drift)
   double *d_tile_sums = nullptr;  // [tile_cap][5] (BatchDev::tile_sums)
   bool dirty = true;
-  // launch shape (autotuned)
+  // launch shape; until it is set or tuned, each repack chooses the tile size (default_tile)
+  bool shaped = false;
   int tile_sites = 1024, grid_moments = 0, grid_collide = 0, grid_particles = 0;
-  int collide_blocks = 3;  // register budget of the update kernel: blocks per SM
+  int collide_blocks = 2;  // register budget of the update kernel: blocks per SM
   // collisions among the replicas of the tables: bit 0 BGK, bit 1 MRT (the update launches only
   // the variants in use)
   int mix = 0;
@@ -765,6 +785,20 @@ std::vector<int> active_slots(const lbmd_batch *b) {
   return act;
 }
 
+// The tile size without tuning: the largest that leaves the update's blocks two tiles each.  24 replicas
+// of 18^3 to 125^3 (13.1 M sites, 42,000 particles), ms per step: tiles of 512 / 1024 / 2048 / 4096 sites
+// at 8 blocks of 128 registers per SM queued 1.157 / 1.114 / 1.116 / 1.091; at 2 per SM 1.149 / 1.127 / 1.121 /
+// 1.100; at 3 blocks of 80 registers 1.194 / 1.168 / 1.171 / 1.188 (1024 was the default).
+int default_tile(const lbmd_batch *b, const std::vector<int> &act) {
+  int ts = 4096;
+  for (; ts > kBThreads; ts /= 2) {
+    long long tiles = 0;
+    for (int s : act) tiles += (b->slots[s].P.N + ts - 1) / ts;
+    if (tiles >= 2LL * b->grid_collide) break;
+  }
+  return ts;
+}
+
 // Lay the tables out again after replicas joined or left or changed their particles: particle
 // ranges (moving the particles that stay, uploading new ones), row ranges, tiles.
 int repack(lbmd_batch *b) {
@@ -859,11 +893,14 @@ int repack(lbmd_batch *b) {
     }
   }
   if (nwords > b->wcap) {
-    pfree(b, b->hb.node_bits);
+    pfree(b, b->hb.node_bits[0]); pfree(b, b->hb.node_bits[1]);
     b->wcap = 0;
-    BK(palloc(b, &b->hb.node_bits, nwords + nwords / 4), "node bits");
+    BK(palloc(b, &b->hb.node_bits[0], nwords + nwords / 4), "node bits");
+    BK(palloc(b, &b->hb.node_bits[1], nwords + nwords / 4), "node bits");
     b->wcap = nwords + nwords / 4;
   }
+  if (nwords > 0) BK(cudaMemsetAsync(b->hb.node_bits[0], 0, sizeof(unsigned) * nwords, b->st), "clear nodes");
+  BK(cudaMemsetAsync(b->hb.parity, 0, sizeof(int), b->st), "clear nodes");
   const int nbs = site::kScanRows;
   const int nblk = (nrows + nbs - 1) / nbs;
   if (nrows + 1 > b->rcap || nblk + 1 > b->bcap) {
@@ -883,6 +920,7 @@ int repack(lbmd_batch *b) {
   if (!rep_slot.empty())
     BK(cudaMemcpyAsync(b->d_rep_slot, rep_slot.data(), sizeof(int) * rep_slot.size(), cudaMemcpyHostToDevice, b->st),
        "upload replicas");
+  if (!b->shaped) b->tile_sites = default_tile(b, act);
   int r = build_tiles(b, act);
   if (r) return r;
   b->mix = 0;
@@ -894,6 +932,11 @@ int repack(lbmd_batch *b) {
   b->hb.pslot = b->d_pslot;
   r = upload_tables(b);
   if (r) return r;
+  if (np > 0) {
+    kb_mark<<<std::max(1, std::min(b->grid_particles, (np + kBPThreads - 1) / kBPThreads)), kBPThreads, 0, b->st>>>(b->d_batch);
+    BK(cudaGetLastError(), "mark nodes");
+    b->launches++;
+  }
   b->dirty = false;
   return LBMD_OK;
 }
@@ -948,7 +991,8 @@ void launch_drift(lbmd_batch *b) {
 // Enqueues one step; returns the number of kernel launches.
 // The particle sort and the pair forces depend on the particles only: they run on the side
 // stream beside the density pass, forked from st at the start of the step and joined before the
-// coupling (sorted rows) and before the particle update (pair forces).
+// coupling (sorted rows); the particle update follows there once the coupling is done, beside the
+// lattice update, and is joined before the end of the step.
 int enqueue_step(lbmd_batch *b) {
   const BatchDev *B = b->d_batch;
   const int gp = b->grid_particles;
@@ -969,11 +1013,14 @@ int enqueue_step(lbmd_batch *b) {
   // kPairGrid times the particle grid (blocks beyond the resident ones queue) leaves each of their
   // threads about one particle instead of a few in a row
   kb_couple<<<kPairGrid * gp, kBPThreads, 0, b->st>>>(B);
+  cudaEventRecord(b->ev_coupled, b->st);
   kb_pairs<<<kPairGrid * gp, kBPThreads, 0, sd>>>(B);
-  cudaEventRecord(b->ev_pairs, sd);
+  // the particle update beside the lattice update, which reads the sorted copy
+  cudaStreamWaitEvent(sd, b->ev_coupled, 0);
+  kb_integrate<<<gp, kBPThreads, 0, sd>>>(B);
+  cudaEventRecord(b->ev_moved, sd);
   const int nc = launch_batched_collide(b, b->grid_collide, b->collide_blocks, 0);
-  cudaStreamWaitEvent(b->st, b->ev_pairs, 0);
-  kb_integrate<<<gp, kBPThreads, 0, b->st>>>(B);
+  cudaStreamWaitEvent(b->st, b->ev_moved, 0);
   kb_advance<<<1, 256, 0, b->st>>>(B);
   launch_drift(b);
   return 14 + nc;
@@ -1029,19 +1076,21 @@ void lbmd_batch_destroy(lbmd_batch *b) {
   free_particle_set(b, b->hb.U); free_particle_set(b, b->hb.S); free_forces(b, b->hb.pf);
   pfree(b, b->hb.row_of); pfree(b, b->hb.perm); pfree(b, b->d_pslot);
   pfree(b, b->hb.row_count); pfree(b, b->hb.row_start); pfree(b, b->hb.row_cursor); pfree(b, b->hb.bsum);
-  pfree(b, b->hb.node_bits);
+  pfree(b, b->hb.node_bits[0]); pfree(b, b->hb.node_bits[1]);
   pfree(b, b->d_tile_slot);
   cudaStreamSynchronize(b->st);
   if (b->pool) cudaMemPoolDestroy(b->pool);
   cudaFree(b->d_rep); cudaFree(b->d_state); cudaFree(b->d_lay); cudaFree(b->d_left); cudaFree(b->d_rep_slot);
   pfree(b, b->d_tile_sums);
   cudaStreamSynchronize(b->st);
+  cudaFree(b->hb.parity);
   cudaFree(b->d_batch); cudaFree(b->diag_partial); cudaFree(b->diag_out); cudaFree(b->d_drift);
   if (b->own_stream) cudaStreamDestroy(b->st);
   if (b->side) cudaStreamDestroy(b->side);
   if (b->ev_fork) cudaEventDestroy(b->ev_fork);
   if (b->ev_sorted) cudaEventDestroy(b->ev_sorted);
-  if (b->ev_pairs) cudaEventDestroy(b->ev_pairs);
+  if (b->ev_coupled) cudaEventDestroy(b->ev_coupled);
+  if (b->ev_moved) cudaEventDestroy(b->ev_moved);
   delete b;
 }
 
@@ -1064,7 +1113,8 @@ int lbmd_batch_create(size_t mem_budget, int storage, int max_slots, void *strea
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_sorted, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_pairs, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_coupled, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_moved, cudaEventDisableTiming);
   size_t free_b = 0, total_b = 0;
   if (e == cudaSuccess) e = cudaMemGetInfo(&free_b, &total_b);
   if (e == cudaSuccess) {
@@ -1085,6 +1135,9 @@ int lbmd_batch_create(size_t mem_budget, int storage, int max_slots, void *strea
   if (e == cudaSuccess) e = cudaMalloc(&b->d_left, sizeof(int) * max_slots);
   if (e == cudaSuccess) e = cudaMalloc(&b->d_rep_slot, sizeof(int) * max_slots);
   if (e == cudaSuccess) e = cudaMalloc(&b->d_batch, sizeof(BatchDev));
+  int *parity = nullptr;
+  if (e == cudaSuccess) e = cudaMalloc(&parity, sizeof(int));
+  b->hb.parity = parity;
   if (e == cudaSuccess) e = cudaMalloc(&b->diag_partial, sizeof(double) * 8 * 1024);
   if (e == cudaSuccess) e = cudaMalloc(&b->d_drift, sizeof(double) * 10 * max_slots);
   if (e == cudaSuccess) e = cudaMalloc(&b->diag_out, sizeof(double) * 8);
@@ -1103,9 +1156,8 @@ int lbmd_batch_create(size_t mem_budget, int storage, int max_slots, void *strea
   b->max_slots = max_slots;
   b->slots.resize(max_slots);
   b->grid_moments = 4 * b->sms;
-  b->grid_collide = 3 * b->sms;
+  b->grid_collide = 8 * b->sms;
   b->grid_particles = 8 * b->sms;
-  b->hb = BatchDev{};
   b->hb.rep = b->d_rep;
   b->hb.state = b->d_state;
   b->hb.lay = b->d_lay;
@@ -1473,6 +1525,7 @@ int lbmd_batch_set_config(lbmd_batch *b, int tile_sites, int grid_moments, int g
     return bfail(b, LBMD_E_INVALID_ARG, "grid sizes must be in [1, 64 x SM count]");
   cudaSetDevice(b->dev);
   if (tile_sites != b->tile_sites) b->dirty = true;
+  b->shaped = true;
   b->tile_sites = tile_sites;
   b->grid_moments = grid_moments;
   b->grid_collide = grid_collide;
@@ -1518,8 +1571,8 @@ int lbmd_batch_tune(lbmd_batch *b, int cfg[5], double ms[2]) {
   };
   const int tiles[] = {256, 1024, 4096};
   const int gms[] = {2, 3, 4};
-  static const int gcs_v[][2] = {{3, 1}, {3, 2}, {3, 3}, {2, 1}, {2, 2}};  // (blocks per SM budget, grid / SMs)
-  const int *gcs[] = {gcs_v[0], gcs_v[1], gcs_v[2], gcs_v[3], gcs_v[4]};
+  static const int gcs_v[][2] = {{3, 1}, {3, 2}, {3, 3}, {2, 1}, {2, 2}, {2, 8}};  // (blocks per SM budget, grid / SMs)
+  const int *gcs[] = {gcs_v[0], gcs_v[1], gcs_v[2], gcs_v[3], gcs_v[4], gcs_v[5]};
   float best = 1e30f, best_m = 0.f, best_c = 0.f;
   int bt = b->tile_sites, bm = b->grid_moments, bc = b->grid_collide, bb = b->collide_blocks;
   const int saved_tile = b->tile_sites;
@@ -1557,6 +1610,7 @@ int lbmd_batch_tune(lbmd_batch *b, int cfg[5], double ms[2]) {
     b->dirty = true;
     return r ? r : bcuda(b, e, "tuning launches");
   }
+  b->shaped = true;
   b->tile_sites = bt;
   b->grid_moments = bm;
   b->grid_collide = bc;
