@@ -460,8 +460,7 @@ __global__ void __launch_bounds__(kOPThreads, 3)
   cp_async_wait_all();  // no copy outlives the block
 }
 
-// The nodes the one-pass update leaves unfinished, in one launch of five block ranges (range 5
-// first):
+// The nodes the one-pass update leaves unfinished, in one launch of four block ranges:
 //  1. the boundary runs, a warp per run: their densities from the new populations, as the density
 //     pass computes them (without y partials the first and last row of each tile; without z
 //     partials the first and last plane of each chunk);
@@ -472,138 +471,171 @@ __global__ void __launch_bounds__(kOPThreads, 3)
 //     above (for the top row) sends across, and at the two corners also the x-neighbour's edge-row
 //     sums and the value the diagonal neighbour sends, in that order;
 //  4. with z partials, the other nodes of the chunk-edge planes: own partial plus the lower
-//     chunk's;
-//  5. with particles, j' of the new populations at the 8 corners of each particle's cell, for the
-//     next step's coupling (jc, by particle id; pn: the particles as the next step starts).
+//     chunk's.
 // In ranges 2 and 3 a chunk-edge plane's node adds the lower chunk's part after each term.  The
 // sets of nodes are disjoint, and every node's sum has a fixed order.
-template <class T>
-__global__ void __launch_bounds__(kBlock) k_boundary_densities(StepParams P, OnePassGeom G, const T *__restrict__ store,
+// Bound by latency and by its scattered sectors: ranges 3 and 4 take kVec neighbouring nodes a thread (2
+// where rows start on 16 bytes, nx even), indices by multiplication.  At 256^3: 45 us, with a node a thread and
+// divisions 66; the next step's corner j' (33 us) runs on the side stream beside it, with it in one launch the two
+// took 95.
+template <int kVec>
+struct NodeRun {
+  float2 v[kVec];
+  __device__ __forceinline__ void load(const float2 *p) {
+    if constexpr (kVec == 2) {
+      const float4 w = *reinterpret_cast<const float4 *>(p);
+      v[0] = make_float2(w.x, w.y);
+      v[1] = make_float2(w.z, w.w);
+    } else {
+      v[0] = *p;
+    }
+  }
+  __device__ __forceinline__ void store(float2 *p) const {
+    if constexpr (kVec == 2)
+      *reinterpret_cast<float4 *>(p) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+    else
+      *p = v[0];
+  }
+  __device__ __forceinline__ void add(const NodeRun &o) {
+#pragma unroll
+    for (int k = 0; k < kVec; ++k) v[k] = add2(v[k], o.v[k]);
+  }
+};
+
+struct BoundaryBlocks {
+  unsigned runs, edge, row;  // blocks of the ranges 1, 2 and 3 (the rest: 4)
+  FastDiv by_ntx, by_nty, by_run;  // by the column tiles along x and y, and by nx / kVec
+};
+
+template <class T, int kVec>
+__global__ void __launch_bounds__(kBlock) k_boundary_densities(StepParams P, OnePassGeom G, BoundaryBlocks D,
+                                                               const T *__restrict__ store,
                                                                const float *__restrict__ rest,
                                                                float *__restrict__ rho_next,
                                                                const BoundaryRun *__restrict__ runs, int nruns,
-                                                               int corner_blocks, int run_blocks, int edge_blocks,
-                                                               int row_blocks, OnePassOut out,
-                                                               const int *__restrict__ zslot, ParticleArrays pn,
-                                                               int np, float4 *__restrict__ jc) {
-  // the latency-bound corner j' blocks first, so that they run beside the others
-  if ((int)blockIdx.x < corner_blocks) {
-    // 5: corner j' (a thread per particle and corner)
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= 8LL * np) return;
-    const int p = (int)(t >> 3), k = (int)(t & 7);
-    const Coord cc = cell_corner(P, __ldg(pn.cell + p), k);
-    const float3 j = jprime_at<T>(P, store, cc.x, cc.y, cc.z);
-    jc[(long long)__ldg(pn.pid + p) * 8 + k] = make_float4(j.x, j.y, j.z, 0.f);
-    return;
-  }
-  const int bid = (int)blockIdx.x - corner_blocks;
-  if (bid < run_blocks) {
-    const int r = bid * (kBlock / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+                                                               OnePassOut out, const int *__restrict__ zslot) {
+  unsigned bid = blockIdx.x;
+  if (bid < D.runs) {
+    const int r = (int)bid * (kBlock / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (r >= nruns) return;
     const BoundaryRun b = runs[r];
     if (lane >= b.n) return;
     moments(P, (long long)b.row * P.nx + b.x0 + lane, store, rest, rho_next, nullptr);
     return;
   }
+  bid -= D.runs;
   const float2 *e2 = reinterpret_cast<const float2 *>(out.edge);
   const float2 *zo = reinterpret_cast<const float2 *>(out.zown);
   const float2 *ze2 = reinterpret_cast<const float2 *>(out.zedge);
   float2 *rho2 = reinterpret_cast<float2 *>(rho_next);
-  const long long plane = (long long)P.ny * P.nx;
-  if (bid < run_blocks + edge_blocks) {
-    // 32-bit index arithmetic: nz ny ntx < N < 2^32 / 19
-    const unsigned t = (unsigned)(bid - run_blocks) * blockDim.x + threadIdx.x;
-    const unsigned n = (unsigned)P.nz * P.ny * G.ntx;
-    if (t >= n) return;
-    const unsigned r = t / G.ntx;  // z * ny + y
-    const int tx = (int)(t - r * G.ntx);
-    const int z = (int)(r / P.ny), y = (int)(r - (unsigned)z * P.ny);
-    const int w = y % kOnePassRows, y0 = y - w, rows = min(kOnePassRows, P.ny - y0);
+  const unsigned nx = (unsigned)P.nx, ny = (unsigned)P.ny, ntx = (unsigned)G.ntx, nty = (unsigned)G.nty;
+  // 32-bit index arithmetic: nodes and partial sums are fewer than 2^32 / 19
+  if (bid < D.edge) {
+    const unsigned t = bid * kBlock + threadIdx.x;
+    if (t >= (unsigned)P.nz * ny * ntx) return;
+    const unsigned r = fast_div(t, D.by_ntx), tx = t - r * ntx;  // r = z * ny + y
+    const unsigned z = fast_div(r, P.divy), y = r - z * ny;
+    const int w = (int)(y % kOnePassRows), rows = min(kOnePassRows, P.ny - (int)(y - w));
     if (w < 1 || w > rows - 2) return;  // tile edge rows: runs, or range 3
     const int q = zslot[z];             // chunk-edge plane: its slot in the z arrays
     if (q >= 0 && !G.zpart) return;     // runs
-    const int x0 = tx * kOnePassCols, nown = min(kOnePassCols, P.nx - x0);
-    const int txl = tx == 0 ? G.ntx - 1 : tx - 1, txr = tx == G.ntx - 1 ? 0 : tx + 1;
-    const long long base = (long long)r * P.nx;
-    const long long zb = ((long long)q * P.ny + y) * P.nx;  // this row in the z arrays (q >= 0)
-    const long long zr = (long long)q * P.ny + y;
-    float2 v = rho2[base + x0];
+    const unsigned x0 = tx * kOnePassCols, nown = min((unsigned)kOnePassCols, nx - x0);
+    const unsigned txl = tx == 0 ? ntx - 1 : tx - 1, txr = tx == ntx - 1 ? 0 : tx + 1;
+    const unsigned base = r * nx;
+    const unsigned zr = (unsigned)q * ny + y, zb = zr * nx;  // this row in the z arrays (q >= 0)
+    const unsigned xr = x0 + nown - 1;
+    float2 v = rho2[base + x0], vr = rho2[base + xr];
+    const float2 el = e2[(r * ntx + txl) * 2 + 1];  // from the left tile's last lane
+    const float2 er = e2[(r * ntx + txr) * 2 + 0];  // and from the right tile's lane 0
     if (q >= 0) v = add2(v, zo[zb + x0]);
-    v = add2(v, e2[((long long)r * G.ntx + txl) * 2 + 1]);  // from the left tile's last lane
-    if (q >= 0) v = add2(v, ze2[(zr * G.ntx + txl) * 2 + 1]);
-    if (nown == 1) {  // and from the right tile's lane 0
-      v = add2(v, e2[((long long)r * G.ntx + txr) * 2 + 0]);
-      if (q >= 0) v = add2(v, ze2[(zr * G.ntx + txr) * 2 + 0]);
-      rho2[base + x0] = v;
-      return;
-    }
-    rho2[base + x0] = v;
-    const int xr = x0 + nown - 1;
-    v = rho2[base + xr];
-    if (q >= 0) v = add2(v, zo[zb + xr]);
-    v = add2(v, e2[((long long)r * G.ntx + txr) * 2 + 0]);
-    if (q >= 0) v = add2(v, ze2[(zr * G.ntx + txr) * 2 + 0]);
-    rho2[base + xr] = v;
+    v = add2(v, el);
+    if (q >= 0) v = add2(v, ze2[(zr * ntx + txl) * 2 + 1]);
+    if (nown == 1)
+      vr = v;
+    else if (q >= 0)
+      vr = add2(vr, zo[zb + xr]);
+    vr = add2(vr, er);
+    if (q >= 0) vr = add2(vr, ze2[(zr * ntx + txr) * 2 + 0]);
+    if (nown > 1) rho2[base + x0] = v;
+    rho2[base + xr] = vr;
     return;
   }
-  if (bid < run_blocks + edge_blocks + row_blocks) {
-    // 3: edge rows (y partials): thread per (z, tile row, bottom / top, x)
-    const unsigned t = (unsigned)(bid - run_blocks - edge_blocks) * blockDim.x + threadIdx.x;
-    const unsigned n = (unsigned)P.nz * G.nty * 2 * P.nx;
-    if (t >= n) return;
-    const unsigned qq = t / P.nx;
-    const int x = (int)(t - qq * P.nx);
-    const int sy = (int)(qq & 1u);
-    const unsigned zt = qq >> 1;
-    const int z = (int)(zt / G.nty), ty = (int)(zt - (unsigned)z * G.nty);
+  bid -= D.edge;
+  const unsigned run = nx / kVec;  // threads per row
+  if (bid < D.row) {
+    // 3: edge rows (y partials): thread per (z, tile row, bottom / top, kVec nodes)
+    const unsigned t = bid * kBlock + threadIdx.x;
+    if (t >= (unsigned)P.nz * nty * 2 * run) return;
+    const unsigned qq = fast_div(t, D.by_run), x = (t - qq * run) * kVec, sy = qq & 1u;
+    const unsigned zt = qq >> 1, z = fast_div(zt, D.by_nty), ty = zt - z * nty;
     const int q = zslot[z];
     if (q >= 0 && !G.zpart) return;  // runs
-    const int y0 = ty * kOnePassRows, rows = min(kOnePassRows, P.ny - y0), y = sy ? y0 + rows - 1 : y0;
-    const int tx = x / kOnePassCols, x0 = tx * kOnePassCols, nown = min(kOnePassCols, P.nx - x0);
-    const int txl = tx == 0 ? G.ntx - 1 : tx - 1, txr = tx == G.ntx - 1 ? 0 : tx + 1;
-    const int tyn = sy ? (ty == G.nty - 1 ? 0 : ty + 1) : (ty == 0 ? G.nty - 1 : ty - 1);  // the tile sending across
+    const unsigned y0 = ty * kOnePassRows, rows = min((unsigned)kOnePassRows, ny - y0), y = sy ? y0 + rows - 1 : y0;
+    const unsigned tx = x / kOnePassCols, x0 = tx * kOnePassCols, nown = min((unsigned)kOnePassCols, nx - x0);
+    const unsigned txl = tx == 0 ? ntx - 1 : tx - 1, txr = tx == ntx - 1 ? 0 : tx + 1;
+    const unsigned tyn = sy ? (ty == nty - 1 ? 0 : ty + 1) : (ty == 0 ? nty - 1 : ty - 1);  // the tile sending across
     const float2 *y2 = reinterpret_cast<const float2 *>(out.yedge);
     const float2 *zy = reinterpret_cast<const float2 *>(out.zyedge);
     const float2 *d2 = reinterpret_cast<const float2 *>(out.diag);
-    const long long node = ((long long)z * P.ny + y) * P.nx + x;
-    const long long ystride = (long long)G.ntx * kOnePassCols;
-    float2 v = rho2[node];
-    if (q >= 0) v = add2(v, zo[(long long)q * plane + (long long)y * P.nx + x]);
+    const unsigned er = z * ny + y, zr = (unsigned)q * ny + y, node = er * nx + x;
+    const unsigned ystride = ntx * kOnePassCols;
+    NodeRun<kVec> v, part;
+    v.load(rho2 + node);
     // the bottom row gets what the tile below sends up (its side 1), the top row what the tile
     // above sends down (its side 0)
-    v = add2(v, y2[(((long long)(1 - sy) * P.nz + z) * G.nty + tyn) * ystride + x]);
-    if (q >= 0) v = add2(v, zy[(((long long)(1 - sy) * 2 * G.nchunks + q) * G.nty + tyn) * ystride + x]);
-    const long long er = (long long)z * P.ny + y, zr = (long long)q * P.ny + y;
+    part.load(y2 + (((1 - sy) * (unsigned)P.nz + z) * nty + tyn) * ystride + x);
+    if (q >= 0) {
+      NodeRun<kVec> below;
+      below.load(zo + zr * nx + x);
+      v.add(below);
+    }
+    v.add(part);
+    if (q >= 0) {
+      part.load(zy + (((1 - sy) * 2 * (unsigned)G.nchunks + (unsigned)q) * nty + tyn) * ystride + x);
+      v.add(part);
+    }
     if (x == x0) {  // corner: the left tile's side-1 sums of this row, the diagonal value
-      v = add2(v, e2[(er * G.ntx + txl) * 2 + 1]);
-      if (q >= 0) v = add2(v, ze2[(zr * G.ntx + txl) * 2 + 1]);
-      v = add2(v, d2[(((long long)z * G.nty + tyn) * G.ntx + txl) * 4 + (sy ? 1 : 3)]);
+      float2 &c = v.v[0];
+      c = add2(c, e2[(er * ntx + txl) * 2 + 1]);
+      if (q >= 0) c = add2(c, ze2[(zr * ntx + txl) * 2 + 1]);
+      c = add2(c, d2[((z * nty + tyn) * ntx + txl) * 4 + (sy ? 1 : 3)]);
     }
-    if (x == x0 + nown - 1) {  // corner: the right tile's side-0 sums of this row, the diagonal value
-      v = add2(v, e2[(er * G.ntx + txr) * 2 + 0]);
-      if (q >= 0) v = add2(v, ze2[(zr * G.ntx + txr) * 2 + 0]);
-      v = add2(v, d2[(((long long)z * G.nty + tyn) * G.ntx + txr) * 4 + (sy ? 0 : 2)]);
+    if (x + kVec - 1 == x0 + nown - 1) {  // corner: the right tile's side-0 sums of this row, the diagonal value
+      float2 &c = v.v[kVec - 1];
+      c = add2(c, e2[(er * ntx + txr) * 2 + 0]);
+      if (q >= 0) c = add2(c, ze2[(zr * ntx + txr) * 2 + 0]);
+      c = add2(c, d2[((z * nty + tyn) * ntx + txr) * 4 + (sy ? 0 : 2)]);
     }
-    rho2[node] = v;
+    v.store(rho2 + node);
     return;
   }
-  // 4: the other nodes of the chunk-edge planes (z partials): thread per (slot, y, x)
-  const unsigned t = (unsigned)(bid - run_blocks - edge_blocks - row_blocks) * blockDim.x + threadIdx.x;
-  const unsigned n = (unsigned)(2 * G.nchunks) * P.ny * P.nx;
-  if (t >= n) return;
-  const unsigned qy = t / P.nx;
-  const int x = (int)(t - qy * P.nx);
-  const int q = (int)(qy / P.ny), y = (int)(qy - (unsigned)q * P.ny);
-  const int w = y % kOnePassRows, rows = min(kOnePassRows, P.ny - (y - w));
+  bid -= D.row;
+  // 4: the other nodes of the chunk-edge planes (z partials): thread per (slot, y, kVec nodes)
+  const unsigned t = bid * kBlock + threadIdx.x;
+  if (t >= 2u * (unsigned)G.nchunks * ny * run) return;
+  const unsigned qy = fast_div(t, D.by_run), x = (t - qy * run) * kVec;
+  const unsigned q = fast_div(qy, P.divy), y = qy - q * ny;
+  const int w = (int)(y % kOnePassRows), rows = min(kOnePassRows, P.ny - (int)(y - w));
   if (w < 1 || w > rows - 2) return;  // tile edge rows: runs, or range 3
-  const int xt = x % kOnePassCols, nown = min(kOnePassCols, P.nx - (x - xt));
-  if (xt == 0 || xt == nown - 1) return;  // x edges: range 2
+  const unsigned xt = x % kOnePassCols, nown = min((unsigned)kOnePassCols, nx - (x - xt));
+  // x edges: range 2 (which stores them; they are not written here)
+  const bool first = xt != 0, last = xt + kVec - 1 != nown - 1;
+  if (kVec == 1 && (!first || !last)) return;
   // the plane of slot q: zs - 1 (q even) or zs (q odd) of chunk q / 2
-  const int zs = (int)((long long)(q >> 1) * P.nz / G.nchunks);
-  const int z = (q & 1) ? zs : (zs == 0 ? P.nz - 1 : zs - 1);
-  const long long node = (long long)z * plane + (long long)y * P.nx + x;
-  rho2[node] = add2(rho2[node], zo[(long long)q * plane + (long long)y * P.nx + x]);
+  const unsigned zs = (unsigned)((unsigned long long)(q >> 1) * P.nz / G.nchunks);
+  const unsigned z = (q & 1) ? zs : (zs == 0 ? P.nz - 1 : zs - 1);
+  const unsigned at = y * nx + x, node = z * ny * nx + at;
+  if (first && last) {
+    NodeRun<kVec> v, part;
+    v.load(rho2 + node);
+    part.load(zo + q * ny * nx + at);
+    v.add(part);
+    v.store(rho2 + node);
+  } else if (kVec == 2 && first) {
+    rho2[node] = add2(rho2[node], zo[q * ny * nx + at]);
+  } else if (kVec == 2 && last) {
+    rho2[node + 1] = add2(rho2[node + 1], zo[q * ny * nx + at + 1]);
+  }
 }
 
 // rho_A, rho_B and u = (j' + g^SC/2)/rho at the current step (for readback; any output may be null:
@@ -849,20 +881,22 @@ void launch_collide_onepass(const StepParams &P, const void *fin, void *fout, co
 
 void launch_boundary_densities(const StepParams &P, OnePassGeom G, const void *store, const float *rest,
                                float *rho_next, const BoundaryRun *runs, int nruns, OnePassOut out,
-                               const int *zslot, const ParticleArrays &pn, int np, float4 *jc, cudaStream_t st) {
-  const long long run_blocks = (nruns + kBlock / 32 - 1) / (kBlock / 32);
-  const long long edge_blocks = ((long long)P.nz * P.ny * G.ntx + kBlock - 1) / kBlock;
-  const long long row_blocks = G.ypart ? ((long long)P.nz * G.nty * 2 * P.nx + kBlock - 1) / kBlock : 0;
-  const long long zplane_blocks = G.zpart ? ((long long)2 * G.nchunks * P.ny * P.nx + kBlock - 1) / kBlock : 0;
-  if (!jc) np = 0;
-  const long long corner_blocks = (8LL * np + kBlock - 1) / kBlock;
-  const long long blocks = run_blocks + edge_blocks + row_blocks + zplane_blocks + corner_blocks;
-  if (blocks <= 0) return;
+                               const int *zslot, cudaStream_t st) {
+  const int vec = P.nx % 2 == 0 ? 2 : 1;
+  auto blocks = [](long long threads) { return (unsigned)((threads + kBlock - 1) / kBlock); };
+  BoundaryBlocks D;
+  D.runs = blocks(32LL * nruns);
+  D.edge = blocks((long long)P.nz * P.ny * G.ntx);
+  D.row = G.ypart ? blocks((long long)P.nz * G.nty * 2 * (P.nx / vec)) : 0;
+  const unsigned plane = G.zpart ? blocks((long long)2 * G.nchunks * P.ny * (P.nx / vec)) : 0;
+  D.by_ntx = make_fastdiv((uint32_t)G.ntx);
+  D.by_nty = make_fastdiv((uint32_t)G.nty);
+  D.by_run = make_fastdiv((uint32_t)(P.nx / vec));
   with_storage(P, [&](auto t) {
     using T = std::remove_pointer_t<decltype(t)>;
-    k_boundary_densities<T><<<(unsigned)blocks, kBlock, 0, st>>>(
-        P, G, static_cast<const T *>(store), rest, rho_next, runs, nruns, (int)corner_blocks, (int)run_blocks,
-        (int)edge_blocks, (int)row_blocks, out, zslot, pn, np, jc);
+    auto *kernel = vec == 2 ? k_boundary_densities<T, 2> : k_boundary_densities<T, 1>;
+    kernel<<<D.runs + D.edge + D.row + plane, kBlock, 0, st>>>(P, G, D, static_cast<const T *>(store), rest, rho_next,
+                                                               runs, nruns, out, zslot);
   });
 }
 

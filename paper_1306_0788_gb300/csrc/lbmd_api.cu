@@ -54,9 +54,9 @@ struct lbmd_ctx {
   cudaStream_t side = nullptr;
   cudaEvent_t ev_int = nullptr, ev_sorted = nullptr, ev_coupled = nullptr, ev_sub = nullptr;
   bool sort_pending = false;
-  // one pass with particles: ev_integrated (the particle update done, on side) orders the boundary
-  // kernel, which forms the next step's corner j' (jc) at the updated positions, after it
-  cudaEvent_t ev_integrated = nullptr;
+  // one pass with particles: the next step's corner j' (jc) is formed on side, at the sorted updated
+  // particles, once the lattice update is done (ev_collided), beside the boundary densities on st
+  cudaEvent_t ev_collided = nullptr;
   // the device-memory getters: the caller's stream's queued work before their writes (dev_in),
   // and their writes before what the caller queues next (dev_out); created on first use
   cudaEvent_t ev_dev_in = nullptr, ev_dev_out = nullptr;
@@ -443,7 +443,6 @@ int ensure_corner_j(lbmd_ctx *c) {
 
 // Sorts the unsorted particles pt into pa[1 - pcur] and row_start[1 - pcur] on st, and makes these
 // the current ones.  update: pt is first formed from pa[pcur] by the particle update.
-// ev_integrated is recorded once pt holds the updated particles.
 int sort_particles(lbmd_ctx *c, bool update, cudaStream_t st) {
   const StepParams &P = c->P;
   const ParticleArrays &from = c->pa[c->pcur], &to = c->pa[1 - c->pcur];
@@ -452,14 +451,12 @@ int sort_particles(lbmd_ctx *c, bool update, cudaStream_t st) {
   c->pcur = 1 - c->pcur;
   if (sort_fits_one_block(P.nrows, P.np)) {
     launch_sort_small(P, update ? &from : nullptr, c->pt, c->pf, to, start, c->slot_of_id, bits, c->err, st);
-    if (update) CK(cudaEventRecord(c->ev_integrated, st), "event");
     return launched(c, "particle sort");
   }
   if (update)
     launch_integrate_bin(P, from, c->pt, c->pf, c->sort, to.cell, bits, c->err, st);
   else
     launch_bin(P, c->pt, c->sort, c->err, st);
-  if (update) CK(cudaEventRecord(c->ev_integrated, st), "event");
   launch_place(P, c->sort, c->pt, to, start, c->slot_of_id, bits, st);
   return launched(c, "particle sort", 4);  // bin, scan, scatter, place
 }
@@ -619,7 +616,7 @@ int one_step(lbmd_ctx *c, unsigned long long step, cudaEvent_t t0, cudaEvent_t t
     CK(cudaEventRecord(c->ev_sorted, c->side), "event");
     c->sort_pending = true;
   } else if (P.np > 0) {
-    if (onepass) {  // no density pass stored j': the previous step's boundary kernel formed it at the corners
+    if (onepass) {  // no density pass stored j': the previous step formed it at the corners
       if (!c->jc_valid) return fail(c, LBMD_E_STATE, "one-pass coupling without the corner j' of the current state");
       launch_couple_jc(P, c->pa[c->pcur], ci, rho, c->jc, c->pf, c->st);
     } else
@@ -644,12 +641,17 @@ int one_step(lbmd_ctx *c, unsigned long long step, cudaEvent_t t0, cudaEvent_t t
     launch_collide(P, fin, fout, rest_in, rest_out, rho, gpa, gpf, gci, c->err, c->st);
   if ((r = launched(c, "collide"))) return r;
   if (t1) CK(cudaEventRecordWithFlags(t1, c->st, flags), "event");
-  const bool corner_j = onepass && P.np > 0 && !sub;  // the boundary kernel forms the next step's jc
+  const bool corner_j = onepass && P.np > 0 && !sub;
+  if (corner_j) {  // the next step's jc, at the sorted particles
+    CK(cudaEventRecord(c->ev_collided, c->st), "event");
+    CK(cudaStreamWaitEvent(c->side, c->ev_collided, 0), "stream wait");
+    launch_corner_jprime(P, c->pa[c->pcur], P.np, fout, c->jc, c->side);
+    if ((r = launched(c, "corner j'"))) return r;
+    CK(cudaEventRecord(c->ev_sorted, c->side), "event");
+  }
   if (onepass) {
-    if (corner_j) CK(cudaStreamWaitEvent(c->st, c->ev_integrated, 0), "stream wait");
     launch_boundary_densities(P, c->op_geom, fout, rest_out, c->rho_buf[1 - c->cur], c->op_runs, c->op_nruns,
-                              c->op_out, c->op_zslot, c->pt, corner_j ? P.np : 0,
-                              corner_j ? c->jc : nullptr, c->st);
+                              c->op_out, c->op_zslot, c->st);
     if ((r = launched(c, "boundary densities"))) return r;
   }
   if (join && (r = join_sort(c))) return r;
@@ -844,7 +846,7 @@ int lbmd_create(const lbmd_params *prm, void *stream, lbmd_ctx **out, unsigned *
       (e = cudaEventCreateWithFlags(&c->ev_sorted, cudaEventDisableTiming)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&c->ev_coupled, cudaEventDisableTiming)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&c->ev_sub, cudaEventDisableTiming)) != cudaSuccess ||
-      (e = cudaEventCreateWithFlags(&c->ev_integrated, cudaEventDisableTiming)) != cudaSuccess) {
+      (e = cudaEventCreateWithFlags(&c->ev_collided, cudaEventDisableTiming)) != cudaSuccess) {
     cudaGetLastError();
     lbmd_destroy(c);
     return fail(nullptr, LBMD_E_CUDA, std::string("stream / event creation: ") + cudaGetErrorString(e));
@@ -877,7 +879,7 @@ void lbmd_destroy(lbmd_ctx *c) {
   if (c->ev_sorted) cudaEventDestroy(c->ev_sorted);
   if (c->ev_coupled) cudaEventDestroy(c->ev_coupled);
   if (c->ev_sub) cudaEventDestroy(c->ev_sub);
-  if (c->ev_integrated) cudaEventDestroy(c->ev_integrated);
+  if (c->ev_collided) cudaEventDestroy(c->ev_collided);
   if (c->ev_dev_in) cudaEventDestroy(c->ev_dev_in);
   if (c->ev_dev_out) cudaEventDestroy(c->ev_dev_out);
   drop_graphs(c);

@@ -296,12 +296,10 @@ void launch_collide_onepass(const StepParams &P, const void *fin, void *fout, co
                             CellIndex ci, unsigned *err, OnePassGeom G, int grid, cudaStream_t st);
 // Adds the partial sums of `out` where they belong and pulls the densities of the listed boundary
 // runs from the new populations, in one launch.  zslot[z]: -1 where z is neither the first nor the
-// last plane of its chunk, else its slot in the z arrays of `out`.  With jc (not NULL), the same
-// launch also forms j' of the new populations at the 8 corners of the cells of the np particles
-// pn, into jc[pid * 8 + corner] (what launch_couple_jc reads).
+// last plane of its chunk, else its slot in the z arrays of `out`.
 void launch_boundary_densities(const StepParams &P, OnePassGeom G, const void *store, const float *rest,
                                float *rho_next, const BoundaryRun *runs, int nruns, OnePassOut out,
-                               const int *zslot, const ParticleArrays &pn, int np, float4 *jc, cudaStream_t st);
+                               const int *zslot, cudaStream_t st);
 // Blocks of the one-pass update resident on one SM (its persistent grid is this times the SMs).
 int onepass_blocks_per_sm();
 void launch_fields(const StepParams &P, const void *store, const float *rest, const float *rho, float *rhoA,
@@ -351,8 +349,7 @@ void launch_sort_small(const StepParams &P, const ParticleArrays *update_from, c
                        unsigned *node_bits, unsigned *err, cudaStream_t st);
 void launch_couple(const StepParams &P, const ParticleArrays &pa, CellIndex ci, const float *rho,
                    const float *jp, const ParticleForces &pf, cudaStream_t st);
-// The same with j' at the corners from jc (8 float4 per particle id, launch_corner_jprime or the
-// one-pass update's boundary kernel).
+// The same with j' at the corners from jc (8 float4 per particle id, launch_corner_jprime).
 void launch_couple_jc(const StepParams &P, const ParticleArrays &pa, CellIndex ci, const float *rho,
                       const float4 *jc, const ParticleForces &pf, cudaStream_t st);
 // j' of the populations `store` (element type P.storage) at the 8 corners of the cells of the np
