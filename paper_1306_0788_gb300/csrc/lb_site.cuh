@@ -351,8 +351,11 @@ __device__ __forceinline__ void for_corner_bits(const StepParams &P, int4 c, F f
 // sub-stepping, the substep index above it.  A row is sorted by x cell; with kBisect the
 // node's two cells are found in it by bisection (the K records per particle of sub-stepping
 // make rows of hundreds of entries), otherwise the row is scanned once (short rows: the
-// plain scan keeps the update's register budget).
-template <bool kBisect = false>
+// plain scan keeps the update's register budget).  kAhead: the four rows' entries are all looked up
+// before the first is walked, one latency instead of four (one pass at 128^3 with 2500 particles, twenty
+// steps: 2889 -> 2865 us; ten of 256^3 with 20,000: 10867 -> 10806).  Only the one-pass update has the
+// registers for it: 64^3 with 1000 particles 1115 -> 1125 us, fluctuating MRT at 256^3 14829 -> 15049.
+template <bool kBisect = false, bool kAhead = false>
 __device__ __forceinline__ void gather_coupling(const StepParams &P, int x, int y, int z, float rA, float rB,
                                                 const ParticleArrays &pa, const ParticleForces &pf,
                                                 CellIndex ci, bool with_momentum, float3 &gA, float3 &gB) {
@@ -378,40 +381,47 @@ __device__ __forceinline__ void gather_coupling(const StepParams &P, int x, int 
       gB.x += wt * (-sB * ff.x - pB.x); gB.y += wt * (-sB * ff.y - pB.y); gB.z += wt * (-sB * ff.z - pB.z);
     }
   };
+  int q0[4], q1[4];
+  auto look_up = [&](int r) {
+    const int oz = r >> 1, oy = r & 1;
+    const int cz = oz ? (z == 0 ? P.nz - 1 : z - 1) : z, cy = oy ? (y == 0 ? P.ny - 1 : y - 1) : y;
+    const int *start = ci.row_start + (cz * P.ny + cy);
+    q0[r] = __ldg(start);
+    q1[r] = __ldg(start + 1);
+  };
+  if constexpr (kAhead) {
 #pragma unroll
-  for (int oz = 0; oz < 2; ++oz) {
-    const int cz = oz ? (z == 0 ? P.nz - 1 : z - 1) : z;
+    for (int r = 0; r < 4; ++r) look_up(r);
+  }
 #pragma unroll
-    for (int oy = 0; oy < 2; ++oy) {
-      const int cy = oy ? (y == 0 ? P.ny - 1 : y - 1) : y;
-      const int row = cz * P.ny + cy;
-      const int q0 = __ldg(ci.row_start + row), q1 = __ldg(ci.row_start + row + 1);
-      if (kBisect) {
-        if (q0 == q1) continue;
+  for (int r = 0; r < 4; ++r) {
+    const int oz = r >> 1, oy = r & 1;
+    if constexpr (!kAhead) look_up(r);
+    if (kBisect) {
+      if (q0[r] == q1[r]) continue;
+      for (int ox = 0; ox < 2; ++ox) {
+        const int cx = ox ? (x == 0 ? P.nx - 1 : x - 1) : x;
+        int lo = q0[r], hi = q1[r];
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (__ldg(&pa.cell[mid].x) < cx)
+            lo = mid + 1;
+          else
+            hi = mid;
+        }
+        for (int q = lo; q < q1[r]; ++q) {
+          const int4 c = __ldg(pa.cell + q);
+          if (c.x != cx) break;
+          add(q, ox, oy, oz, c.w);
+        }
+      }
+    } else {
+      for (int q = q0[r]; q < q1[r]; ++q) {
+        const int4 c = __ldg(pa.cell + q);
+#pragma unroll
         for (int ox = 0; ox < 2; ++ox) {
           const int cx = ox ? (x == 0 ? P.nx - 1 : x - 1) : x;
-          int lo = q0, hi = q1;
-          while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (__ldg(&pa.cell[mid].x) < cx)
-              lo = mid + 1;
-            else
-              hi = mid;
-          }
-          for (int q = lo; q < q1; ++q) {
-            const int4 c = __ldg(pa.cell + q);
-            if (c.x != cx) break;
-            add(q, ox, oy, oz, c.w);
-          }
-        }
-      } else {
-        for (int q = q0; q < q1; ++q) {
-          const int4 c = __ldg(pa.cell + q);
-#pragma unroll
-          for (int ox = 0; ox < 2; ++ox) {
-            const int cx = ox ? (x == 0 ? P.nx - 1 : x - 1) : x;
-            if (c.x == cx) add(q, ox, oy, oz, c.w);
-          }
+          if (c.x == cx) add(q, ox, oy, oz, c.w);
         }
       }
     }
@@ -709,7 +719,7 @@ __device__ __forceinline__ void collide_core_at(const StepParams &P, const Coord
   // (fluctuating MRT, bound by instruction issue), 9 of 878 (one pass, FP32), 4 of 580 (FP16), and
   // the batched update of 24 replicas about 30 of 800.
   if (kParticles && node_touched(P, c, ci.node_bits))
-    gather_coupling<kBisect>(P, c.x, c.y, c.z, rA, rB, pa, pf, ci, true, gA, gB);
+    gather_coupling<kBisect, Rho::kStaged>(P, c.x, c.y, c.z, rA, rB, pa, pf, ci, true, gA, gB);
   const float r = rA + rB;
   if (!(rA > 0.f) || !(rB > 0.f) || !isfinite(r)) atomicOr(err, isfinite(r) ? kErrNegDensity : kErrNonFinite);
   const float rinv = 1.f / r;
