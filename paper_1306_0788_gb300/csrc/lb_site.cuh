@@ -430,6 +430,20 @@ __device__ __forceinline__ void gather_coupling(const StepParams &P, int x, int 
 
 // ------------------------------------------------------------------ fluctuating MRT
 
+// log2 x and 1 / sqrt(x) by the hardware approximations for normal x > 0: without the scaling around the
+// instruction by which __log2f and rsqrtf serve subnormal arguments too (the fluctuating MRT update takes
+// 18 of each per node: ten steps at 256^3 14860 -> 14707 us, the same bits).
+__device__ __forceinline__ float log2_normal(float x) {
+  float y;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rsqrt_normal(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
 // Unit normals 4k .. 4k+3 of the fluid noise at one site and step: Philox4x32-10 (Salmon et
 // al., SC'11) with counter (site, step low, step high, 0x464c0000 + k) and key = seed (its round
 // keys formed once, StepParams::noise_keys), uniforms from the top 24 bits, Box-Muller on both
@@ -448,8 +462,9 @@ __device__ __forceinline__ float4 fluid_normals4(const uint2 *__restrict__ keys,
   const float2 ur = __ffma2_rn(make_float2((float)(r.x >> 8), (float)(r.z >> 8)), sc, h);
   const float2 ua = __ffma2_rn(make_float2((float)(r.y >> 8), (float)(r.w >> 8)), sc, h);
   // u0 = 1 (v = 2^24 - 1 rounds up) gives x = 0: the floor keeps 0 * rsqrt from being NaN
-  const float2 x = __fmul2_rn(make_float2(-2.f, -2.f), make_float2(__logf(ur.x), __logf(ur.y)));
-  const float2 rad = __fmul2_rn(x, make_float2(rsqrtf(fmaxf(x.x, 1e-30f)), rsqrtf(fmaxf(x.y, 1e-30f))));
+  const float m2ln2 = -1.38629436111989061883f;  // -2 ln u = (-2 ln 2) log2 u
+  const float2 x = __fmul2_rn(make_float2(m2ln2, m2ln2), make_float2(log2_normal(ur.x), log2_normal(ur.y)));
+  const float2 rad = __fmul2_rn(x, make_float2(rsqrt_normal(fmaxf(x.x, 1e-30f)), rsqrt_normal(fmaxf(x.y, 1e-30f))));
   const float two_pi = 6.28318530717958647692f;
   const float2 ang = __fmul2_rn(make_float2(two_pi, two_pi), ua);
   float s1, c1, s3, c3;
@@ -548,7 +563,7 @@ __device__ __forceinline__ void mrt_update(const StepParams &P, unsigned long lo
   if (P.fluct) {
     // sqrt(rho_A), sqrt(rho_B) and sqrt(rho_A rho_B / rho) from reciprocal square roots, as the
     // Box-Muller radius (a density of 0 gives 0)
-    const float sA = rA * rsqrtf(fmaxf(rA, 1e-30f)), sB = rB * rsqrtf(fmaxf(rB, 1e-30f));
+    const float sA = rA * rsqrt_normal(fmaxf(rA, 1e-30f)), sB = rB * rsqrt_normal(fmaxf(rB, 1e-30f));
     const float am = P.noise[1] * sA * sB * rsqrtf(rA + rB);
     // A: normals 0-3 (momentum, shared; then mode 4), 4-15 (modes 5-16), 16, 17 (modes 17, 18)
     float4 q = fluid_normals4(P.noise_keys, step, site, 0);
