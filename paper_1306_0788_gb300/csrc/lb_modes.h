@@ -51,4 +51,7 @@ LBMD_MODE_HD constexpr int mode_norm9(int k) {
          : k == 16 ? 18 : k == 17 ? 12 : 4;
 }
 
+// what a mode enters the populations of the diagonal directions with: w_i / b_k, w_i = 1/36
+LBMD_MODE_HD constexpr float mode_scale(int k) { return 1.f / (4.f * mode_norm9(k)); }
+
 }  // namespace lbmd

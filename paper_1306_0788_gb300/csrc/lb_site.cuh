@@ -451,9 +451,10 @@ __device__ __forceinline__ float rsqrt_normal(float x) {
 // are the hardware approximations (absolute error ~1e-6 on a normal, far below what the
 // populations can resolve), and so is the radius: x rsqrt(x), a few ulp from sqrt(x); the
 // generator's integer stream is exact.  A uniform (v + 1/2) 2^-24 is one FFMA: the scaling by a
-// power of two is exact, so one rounding of v 2^-24 + 2^-25 gives the same float.
+// power of two is exact, so one rounding of v 2^-24 + 2^-25 gives the same float.  The first two
+// normals come times scale.x, the last two times scale.y.
 __device__ __forceinline__ float4 fluid_normals4(const uint2 *__restrict__ keys, unsigned long long step,
-                                                 unsigned site, unsigned k) {
+                                                 unsigned site, unsigned k, float2 scale) {
   const uint4 r = philox4x32_10_keyed(make_uint4(site, (unsigned)step, (unsigned)(step >> 32), 0x464c0000u + k),
                                       keys);
   // the two Box-Muller pairs side by side: (u0, u2) give the radii, (u1, u3) the angles
@@ -464,7 +465,8 @@ __device__ __forceinline__ float4 fluid_normals4(const uint2 *__restrict__ keys,
   // u0 = 1 (v = 2^24 - 1 rounds up) gives x = 0: the floor keeps 0 * rsqrt from being NaN
   const float m2ln2 = -1.38629436111989061883f;  // -2 ln u = (-2 ln 2) log2 u
   const float2 x = __fmul2_rn(make_float2(m2ln2, m2ln2), make_float2(log2_normal(ur.x), log2_normal(ur.y)));
-  const float2 rad = __fmul2_rn(x, make_float2(rsqrt_normal(fmaxf(x.x, 1e-30f)), rsqrt_normal(fmaxf(x.y, 1e-30f))));
+  const float2 rad = __fmul2_rn(
+      __fmul2_rn(x, make_float2(rsqrt_normal(fmaxf(x.x, 1e-30f)), rsqrt_normal(fmaxf(x.y, 1e-30f)))), scale);
   const float two_pi = 6.28318530717958647692f;
   const float2 ang = __fmul2_rn(make_float2(two_pi, two_pi), ua);
   float s1, c1, s3, c3;
@@ -480,152 +482,177 @@ __device__ __forceinline__ float4 fluid_normals4(const uint2 *__restrict__ keys,
 // back to populations f_i = w_i sum_k e_k(c_i) m_k / b_k.  The equilibrium moments of
 // f^eq(rho_z, u) are rho_z u (momentum), rho_z u u (stress), 0 (kinetic); those of the forcing
 // term are (2 + lambda_M)/2 g, and G for the stress (appendix), 0 for the kinetic modes.
-// Directions come in opposite pairs (2p + 1, 2p + 2) and every e_k is even or odd in c, so both
-// transforms work on the pair sums and differences: half the arithmetic of the plain sums.
-__device__ __host__ constexpr bool mode_even(int k) { return k == 0 || (k >= 4 && k <= 9) || k >= 16; }
+//
+// Both transforms are factored, the two components together on (A, B) pairs with the packed two-lane
+// FP32 instructions.  Directions come in opposite pairs (2p + 1, 2p + 2) and every e_k is even or odd in c,
+// so they work on the pair sums and differences; and on the sums and differences of the two diagonal
+// pairs of a coordinate plane, on which every e_k is a small combination: 42 packed instructions for the
+// 104 nonzero terms of the plain sums each way.  (The update is bound by the FMA pipes.)
 
-// The collision of both components with the fluctuating MRT operator (Eq. MODES), the two
-// components' arithmetic run together on (A, B) pairs with the packed two-lane FP32
-// instructions.  With noise: the three momentum normals are shared by A (+) and B (-), amplitude
+// sum and difference of (A, B) pairs, and their scaling
+__device__ __forceinline__ float2 pair_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 pair_sub(float2 a, float2 b) { return __ffma2_rn(make_float2(-1.f, -1.f), b, a); }
+__device__ __forceinline__ float2 pair_scale(float a, float2 v) { return __fmul2_rn(make_float2(a, a), v); }
+__device__ __forceinline__ float2 pair_fma(float a, float2 b, float2 c) { return __ffma2_rn(make_float2(a, a), b, c); }
+
+// The modes of the populations fA, fB.
+__device__ __forceinline__ void modes_of(const float (&fA)[kQ], const float (&fB)[kQ], float2 (&m)[kQ]) {
+  float2 s[9], d[9];  // pair sums and differences: x, y, z axes; xy, xz, yz diagonals, two each
+#pragma unroll
+  for (int p = 0; p < 9; ++p) {
+    const float2 u = make_float2(fA[2 * p + 1], fB[2 * p + 1]), v = make_float2(fA[2 * p + 2], fB[2 * p + 2]);
+    s[p] = pair_add(u, v);
+    d[p] = pair_sub(u, v);
+  }
+  const float2 f0 = make_float2(fA[0], fB[0]);
+  // odd modes: per axis a, the a-momenta of the two diagonal planes that hold it
+  const float2 xXY = pair_add(d[3], d[4]), yXY = pair_sub(d[3], d[4]);
+  const float2 xXZ = pair_add(d[5], d[6]), zXZ = pair_sub(d[5], d[6]);
+  const float2 yYZ = pair_add(d[7], d[8]), zYZ = pair_sub(d[7], d[8]);
+  const float2 X = pair_add(xXY, xXZ), Y = pair_add(yXY, yYZ), Z = pair_add(zXZ, zYZ);
+  m[1] = pair_add(d[0], X);
+  m[2] = pair_add(d[1], Y);
+  m[3] = pair_add(d[2], Z);
+  m[10] = pair_fma(-2.f, d[0], X);
+  m[11] = pair_fma(-2.f, d[1], Y);
+  m[12] = pair_fma(-2.f, d[2], Z);
+  m[13] = pair_sub(xXY, xXZ);
+  m[14] = pair_sub(yYZ, yXY);
+  m[15] = pair_sub(zXZ, zYZ);
+  // even modes
+  const float2 xy = pair_add(s[3], s[4]), xz = pair_add(s[5], s[6]), yz = pair_add(s[7], s[8]);
+  m[7] = pair_sub(s[3], s[4]);
+  m[8] = pair_sub(s[7], s[8]);
+  m[9] = pair_sub(s[5], s[6]);
+  const float2 A = pair_add(pair_add(s[0], s[1]), s[2]), D = pair_add(pair_add(xy, xz), yz);
+  const float2 G = pair_add(f0, D);
+  m[0] = pair_add(A, G);
+  m[4] = pair_sub(D, f0);
+  m[16] = pair_fma(-2.f, A, G);
+  const float2 T = pair_fma(3.f, s[0], make_float2(-A.x, -A.y)), U = pair_fma(-3.f, yz, D);
+  m[5] = pair_add(U, T);
+  m[17] = pair_sub(U, T);
+  const float2 V = pair_sub(s[1], s[2]), W = pair_sub(xy, xz);
+  m[6] = pair_add(W, V);
+  m[18] = pair_sub(W, V);
+}
+
+// The moving populations from the modes, n[k] = m_k / b_k times the weight 1/36 of the diagonal
+// directions (the axes' is twice that).
+__device__ __forceinline__ void populations_of(const float2 (&n)[kQ], float (&fA)[kQ], float (&fB)[kQ]) {
+  float2 even[9], odd[9];
+  const float2 a = pair_sub(n[5], n[17]), b = pair_sub(n[6], n[18]);
+  const float2 c = pair_add(n[5], n[17]), d = pair_add(n[6], n[18]);
+  const float2 axis = pair_fma(-4.f, n[16], pair_scale(2.f, n[0])), diag = pair_add(n[16], pair_add(n[0], n[4]));
+  const float2 yz = pair_fma(-2.f, a, axis), xyz = pair_add(diag, c), yz2 = pair_fma(-2.f, c, diag);
+  even[0] = pair_fma(4.f, a, axis);
+  even[1] = pair_fma(2.f, b, yz);
+  even[2] = pair_fma(-2.f, b, yz);
+  const float2 exy = pair_add(xyz, d), exz = pair_sub(xyz, d);
+  even[3] = pair_add(exy, n[7]);
+  even[4] = pair_sub(exy, n[7]);
+  even[5] = pair_add(exz, n[9]);
+  even[6] = pair_sub(exz, n[9]);
+  even[7] = pair_add(yz2, n[8]);
+  even[8] = pair_sub(yz2, n[8]);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) odd[k] = pair_fma(-4.f, n[10 + k], pair_scale(2.f, n[1 + k]));
+  const float2 X = pair_add(n[1], n[10]), Y = pair_add(n[2], n[11]), Z = pair_add(n[3], n[12]);
+  const float2 xXY = pair_add(X, n[13]), xXZ = pair_sub(X, n[13]);
+  const float2 yYZ = pair_add(Y, n[14]), yXY = pair_sub(Y, n[14]);
+  const float2 zXZ = pair_add(Z, n[15]), zYZ = pair_sub(Z, n[15]);
+  odd[3] = pair_add(xXY, yXY);
+  odd[4] = pair_sub(xXY, yXY);
+  odd[5] = pair_add(xXZ, zXZ);
+  odd[6] = pair_sub(xXZ, zXZ);
+  odd[7] = pair_add(yYZ, zYZ);
+  odd[8] = pair_sub(yYZ, zYZ);
+#pragma unroll
+  for (int p = 0; p < 9; ++p) {
+    const float2 fi = pair_add(even[p], odd[p]), fj = pair_sub(even[p], odd[p]);
+    fA[2 * p + 1] = fi.x;
+    fB[2 * p + 1] = fi.y;
+    fA[2 * p + 2] = fj.x;
+    fB[2 * p + 2] = fj.y;
+  }
+}
+
+// The collision of both components with the fluctuating MRT operator (Eq. MODES) from the modes m of
+// modes_of.  With noise: the three momentum normals are shared by A (+) and B (-), amplitude
 // over sqrt(rho_A rho_B / rho); the stress and kinetic modes take normals 3-17 (A) and 18-32 (B)
 // of the site's 36.  Each normal is added to its relaxed mode as it is drawn, so that no
-// component's noise is held whole.
+// component's noise is held whole.  The modes are relaxed straight to what populations_of takes: the
+// factors of StepParams include mode_scale.
 __device__ __forceinline__ void mrt_update(const StepParams &P, unsigned long long step, unsigned site,
-                                           float fA[kQ], float fB[kQ], float rA, float rB, float ux, float uy,
-                                           float uz, float3 gA, float3 gB) {
-  constexpr int kPairs = (kQ - 1) / 2;
-  // modes m_k = sum_i e_k(c_i) f_i of both components, from the pair sums and differences
-  float2 m[kQ];
-  {
-    float2 sp[kPairs], dp[kPairs];
-#pragma unroll
-    for (int p = 0; p < kPairs; ++p) {
-      const float2 u = make_float2(fA[2 * p + 1], fB[2 * p + 1]), v = make_float2(fA[2 * p + 2], fB[2 * p + 2]);
-      sp[p] = __fadd2_rn(u, v);
-      dp[p] = __fadd2_rn(u, make_float2(-v.x, -v.y));
-    }
-    const float2 f0 = make_float2(fA[0], fB[0]);
-#pragma unroll
-    for (int k = 0; k < kQ; ++k) {
-      const float e0 = (float)mode_poly(k, 0, 0, 0);
-      float2 a = mode_even(k) ? make_float2(e0 * f0.x, e0 * f0.y) : make_float2(0.f, 0.f);
-#pragma unroll
-      for (int p = 0; p < kPairs; ++p) {
-        const int i = 2 * p + 1;
-        const int e = mode_poly(k, kCx[i], kCy[i], kCz[i]);
-        const float2 v = mode_even(k) ? sp[p] : dp[p];
-        if (e == 1)
-          a = __fadd2_rn(a, v);
-        else if (e == -1)
-          a = __fadd2_rn(a, make_float2(-v.x, -v.y));
-        else if (e != 0)
-          a = __ffma2_rn(make_float2((float)e, (float)e), v, a);
-      }
-      m[k] = a;
-    }
-  }
+                                           float2 (&m)[kQ], float (&fA)[kQ], float (&fB)[kQ], float rA, float rB,
+                                           float ux, float uy, float uz, float3 gA, float3 gB) {
   // equilibrium moments rho_z (u, u u) and the forcing term's moments of each component; relaxed
   const float uu = ux * ux + uy * uy + uz * uz;
   const float2 rz = make_float2(rA, rB);
   const float2 gx = make_float2(gA.x, gB.x), gy = make_float2(gA.y, gB.y), gz = make_float2(gA.z, gB.z);
   const float2 ug = make_float2(ux * gA.x + uy * gA.y + uz * gA.z, ux * gB.x + uy * gB.y + uz * gB.z);
-  // scaling, sum and difference of (A, B) pairs (packed: the compiler does not pair scalar ones)
-  auto sc = [](float a, float2 v) { return __fmul2_rn(make_float2(a, a), v); };
-  auto ad = [](float2 a, float2 b) { return __fadd2_rn(a, b); };
-  auto sb = [](float2 a, float2 b) { return __ffma2_rn(make_float2(-1.f, -1.f), b, a); };
-  const float2 meq[10] = {rz,
-                          sc(ux, rz),
-                          sc(uy, rz),
-                          sc(uz, rz),
-                          sc(uu, rz),
-                          sc(3.f * ux * ux - uu, rz),
-                          sc(uy * uy - uz * uz, rz),
-                          sc(ux * uy, rz),
-                          sc(uy * uz, rz),
-                          sc(uz * ux, rz)};
-  const float2 mg[10] = {make_float2(0.f, 0.f),
-                         sc(P.force[1], gx),
-                         sc(P.force[2], gy),
-                         sc(P.force[3], gz),
-                         sc(P.force[4], ug),
-                         sc(P.force[5], sb(sc(3.f * ux, gx), ug)),
-                         sc(P.force[6], sb(sc(uy, gy), sc(uz, gz))),
-                         sc(P.force[7], ad(sc(ux, gy), sc(uy, gx))),
-                         sc(P.force[8], ad(sc(uy, gz), sc(uz, gy))),
-                         sc(P.force[9], ad(sc(uz, gx), sc(ux, gz)))};
+  auto sc = [](float a, float2 v) { return pair_scale(a, v); };
+  auto relax = [&](int k, float2 meq, float2 mg) {
+    m[k] = pair_fma(P.relax[k], pair_sub(m[k], meq), pair_fma(mode_scale(k), meq, sc(P.force[k], mg)));
+  };
+  m[0] = sc(mode_scale(0), rz);
+  relax(1, sc(ux, rz), gx);
+  relax(2, sc(uy, rz), gy);
+  relax(3, sc(uz, rz), gz);
+  relax(4, sc(uu, rz), ug);
+  relax(5, sc(3.f * ux * ux - uu, rz), pair_sub(sc(3.f * ux, gx), ug));
+  relax(6, sc(uy * uy - uz * uz, rz), pair_sub(sc(uy, gy), sc(uz, gz)));
+  relax(7, sc(ux * uy, rz), pair_fma(ux, gy, sc(uy, gx)));
+  relax(8, sc(uy * uz, rz), pair_fma(uy, gz, sc(uz, gy)));
+  relax(9, sc(uz * ux, rz), pair_fma(uz, gx, sc(ux, gz)));
 #pragma unroll
-  for (int k = 1; k < kQ; ++k) {
-    if (k < 10)
-      m[k] = ad(__ffma2_rn(make_float2(P.relax[k], P.relax[k]), sb(m[k], meq[k]), meq[k]), mg[k]);
-    else
-      m[k] = sc(P.relax[k], m[k]);
-  }
+  for (int k = 10; k < kQ; ++k) m[k] = sc(P.relax[k], m[k]);
   if (P.fluct) {
     // sqrt(rho_A), sqrt(rho_B) and sqrt(rho_A rho_B / rho) from reciprocal square roots, as the
     // Box-Muller radius (a density of 0 gives 0)
     const float sA = rA * rsqrt_normal(fmaxf(rA, 1e-30f)), sB = rB * rsqrt_normal(fmaxf(rB, 1e-30f));
     const float am = P.noise[1] * sA * sB * rsqrtf(rA + rB);
     // A: normals 0-3 (momentum, shared; then mode 4), 4-15 (modes 5-16), 16, 17 (modes 17, 18)
-    float4 q = fluid_normals4(P.noise_keys, step, site, 0);
-    const float2 amAB = make_float2(am, -am);
-    m[1] = __ffma2_rn(amAB, make_float2(q.x, q.x), m[1]);
-    m[2] = __ffma2_rn(amAB, make_float2(q.y, q.y), m[2]);
-    m[3] = __ffma2_rn(amAB, make_float2(q.z, q.z), m[3]);
-    m[4].x += P.noise[4] * sA * q.w;
+    float4 q = fluid_normals4(P.noise_keys, step, site, 0, make_float2(am, 1.f));
+    const float2 pm = make_float2(1.f, -1.f);
+    m[1] = __ffma2_rn(pm, make_float2(q.x, q.x), m[1]);
+    m[2] = __ffma2_rn(pm, make_float2(q.y, q.y), m[2]);
+    m[3] = __ffma2_rn(make_float2(am, -am), make_float2(q.z, q.z), m[3]);
+    m[4].x += P.noise[4] * (sA * q.w);
 #pragma unroll
     for (int c = 1; c <= 3; ++c) {
-      q = fluid_normals4(P.noise_keys, step, site, c);
+      q = fluid_normals4(P.noise_keys, step, site, c, make_float2(sA, sA));
       const int k = 4 * c + 1;
-      m[k].x += P.noise[k] * sA * q.x;
-      m[k + 1].x += P.noise[k + 1] * sA * q.y;
-      m[k + 2].x += P.noise[k + 2] * sA * q.z;
-      m[k + 3].x += P.noise[k + 3] * sA * q.w;
+      m[k].x += P.noise[k] * q.x;
+      m[k + 1].x += P.noise[k + 1] * q.y;
+      m[k + 2].x += P.noise[k + 2] * q.z;
+      m[k + 3].x += P.noise[k + 3] * q.w;
     }
-    q = fluid_normals4(P.noise_keys, step, site, 4);
-    m[17].x += P.noise[17] * sA * q.x;
-    m[18].x += P.noise[18] * sA * q.y;
+    q = fluid_normals4(P.noise_keys, step, site, 4, make_float2(sA, sB));
+    m[17].x += P.noise[17] * q.x;
+    m[18].x += P.noise[18] * q.y;
     // B: modes 4, 5 from the last two of that draw, then 6-18
-    m[4].y += P.noise[4] * sB * q.z;
-    m[5].y += P.noise[5] * sB * q.w;
+    m[4].y += P.noise[4] * q.z;
+    m[5].y += P.noise[5] * q.w;
 #pragma unroll
     for (int c = 5; c <= 7; ++c) {
-      q = fluid_normals4(P.noise_keys, step, site, c);
+      q = fluid_normals4(P.noise_keys, step, site, c, make_float2(sB, sB));
       const int k = 4 * c - 14;
-      m[k].y += P.noise[k] * sB * q.x;
-      m[k + 1].y += P.noise[k + 1] * sB * q.y;
-      m[k + 2].y += P.noise[k + 2] * sB * q.z;
-      m[k + 3].y += P.noise[k + 3] * sB * q.w;
+      m[k].y += P.noise[k] * q.x;
+      m[k + 1].y += P.noise[k + 1] * q.y;
+      m[k + 2].y += P.noise[k + 2] * q.z;
+      m[k + 3].y += P.noise[k + 3] * q.w;
     }
-    q = fluid_normals4(P.noise_keys, step, site, 8);
-    m[18].y += P.noise[18] * sB * q.x;
+    q = fluid_normals4(P.noise_keys, step, site, 8, make_float2(sB, sB));
+    m[18].y += P.noise[18] * q.x;
   }
-  // scaled by 1 / b_k for the way back
-#pragma unroll
-  for (int k = 0; k < kQ; ++k) m[k] = sc(9.f / (float)mode_norm9(k), m[k]);
-  // moving populations from the modes; the rest population takes what the node's density
-  // (unchanged by the collision) leaves, so that the FP32 weights, whose sum is not exactly 1,
-  // do not bias the mass every step
+  populations_of(m, fA, fB);
+  // the rest population takes what the node's density (unchanged by the collision) leaves, so that
+  // neither the FP32 weights, whose sum is not exactly 1, nor rounding bias the mass every step
   float2 moving = make_float2(0.f, 0.f);
 #pragma unroll
-  for (int p = 0; p < kPairs; ++p) {
-    const int i = 2 * p + 1;
-    float2 even = make_float2(0.f, 0.f), odd = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int k = 0; k < kQ; ++k) {
-      const int e = mode_poly(k, kCx[i], kCy[i], kCz[i]);
-      if (e == 0) continue;
-      if (mode_even(k))
-        even = __ffma2_rn(make_float2((float)e, (float)e), m[k], even);
-      else
-        odd = __ffma2_rn(make_float2((float)e, (float)e), m[k], odd);
-    }
-    const float2 fi = sc(kW[i], ad(even, odd)), fj = sc(kW[i], sb(even, odd));
-    fA[i] = fi.x;
-    fB[i] = fi.y;
-    fA[i + 1] = fj.x;
-    fB[i + 1] = fj.y;
-    moving = ad(moving, ad(fi, fj));
-  }
+  for (int i = 1; i < kQ; i += 2)
+    moving = pair_add(moving, pair_add(make_float2(fA[i], fB[i]), make_float2(fA[i + 1], fB[i + 1])));
   fA[0] = rA - moving.x;
   fB[0] = rB - moving.y;
 }
@@ -685,19 +712,29 @@ __device__ __forceinline__ void collide_core_at(const StepParams &P, const Coord
   // The two components go through the same arithmetic: it runs on (A, B) pairs with the
   // packed two-lane FP32 instructions.  Directions come in opposite pairs (2p + 1, 2p + 2): the
   // densities sum the pair sums, the momenta the pair differences (c_{2p+2} = -c_{2p+1}).
-  float2 r2s = make_float2(fA[0], fB[0]);
-  float2 jx2 = make_float2(0.f, 0.f), jy2 = jx2, jz2 = jx2;
+  float2 r2s, jx2, jy2, jz2;
+  float2 m[kMRT ? kQ : 1];
+  if constexpr (kMRT) {
+    modes_of(fA, fB, m);
+    r2s = m[0];
+    jx2 = m[1];
+    jy2 = m[2];
+    jz2 = m[3];
+  } else {
+    r2s = make_float2(fA[0], fB[0]);
+    jx2 = jy2 = jz2 = make_float2(0.f, 0.f);
 #pragma unroll
-  for (int i = 1; i < kQ; i += 2) {
-    const float2 a = make_float2(fA[i], fB[i]), b = make_float2(fA[i + 1], fB[i + 1]);
-    r2s = __fadd2_rn(r2s, __fadd2_rn(a, b));
-    const float2 d = __fadd2_rn(a, make_float2(-b.x, -b.y));
-    if (kCx[i] > 0) jx2 = __fadd2_rn(jx2, d);
-    if (kCx[i] < 0) jx2 = __fadd2_rn(jx2, make_float2(-d.x, -d.y));
-    if (kCy[i] > 0) jy2 = __fadd2_rn(jy2, d);
-    if (kCy[i] < 0) jy2 = __fadd2_rn(jy2, make_float2(-d.x, -d.y));
-    if (kCz[i] > 0) jz2 = __fadd2_rn(jz2, d);
-    if (kCz[i] < 0) jz2 = __fadd2_rn(jz2, make_float2(-d.x, -d.y));
+    for (int i = 1; i < kQ; i += 2) {
+      const float2 a = make_float2(fA[i], fB[i]), b = make_float2(fA[i + 1], fB[i + 1]);
+      r2s = __fadd2_rn(r2s, __fadd2_rn(a, b));
+      const float2 d = __fadd2_rn(a, make_float2(-b.x, -b.y));
+      if (kCx[i] > 0) jx2 = __fadd2_rn(jx2, d);
+      if (kCx[i] < 0) jx2 = __fadd2_rn(jx2, make_float2(-d.x, -d.y));
+      if (kCy[i] > 0) jy2 = __fadd2_rn(jy2, d);
+      if (kCy[i] < 0) jy2 = __fadd2_rn(jy2, make_float2(-d.x, -d.y));
+      if (kCz[i] > 0) jz2 = __fadd2_rn(jz2, d);
+      if (kCz[i] < 0) jz2 = __fadd2_rn(jz2, make_float2(-d.x, -d.y));
+    }
   }
   const float jx = jx2.x + jx2.y, jy = jy2.x + jy2.y, jz = jz2.x + jz2.y;
   if (kShifted) r2s = __fadd2_rn(r2s, make_float2(shift_sum(P, 0), shift_sum(P, 1)));
@@ -741,8 +778,8 @@ __device__ __forceinline__ void collide_core_at(const StepParams &P, const Coord
   const float ux = (jx + 0.5f * (gA.x + gB.x)) * rinv;
   const float uy = (jy + 0.5f * (gA.y + gB.y)) * rinv;
   const float uz = (jz + 0.5f * (gA.z + gB.z)) * rinv;
-  if (kMRT) {
-    mrt_update(P, step, s32, fA, fB, rA, rB, ux, uy, uz, gA, gB);
+  if constexpr (kMRT) {
+    mrt_update(P, step, s32, m, fA, fB, rA, rB, ux, uy, uz, gA, gB);
   } else {
     // BGK + forcing, f* = (1 - 1/tau) f + (1/tau) f^eq + Delta^g, per pair of opposite directions
     // (c_j = -c_i), with f^eq and Delta^g split into parts even and odd in c.  Per component, with

@@ -85,12 +85,15 @@ void fill_step_params(const lbmd_params *prm, StepParams &P) {
   const double lb = mrt ? prm->lambda_bulk : ls, lm = mrt ? prm->lambda_mom : ls, lg = mrt ? prm->lambda_ghost : ls;
   for (int k = 0; k < kQ; ++k) {
     const double l = k == 0 ? 0.0 : k <= 3 ? lm : k == 4 ? lb : k <= 9 ? ls : lg;
-    P.relax[k] = (float)(1.0 + l);
-    P.force[k] = (float)(k == 0 ? 0.0 : k <= 3 ? 0.5 * (2.0 + lm) : k == 4 ? 2.0 + lb : k <= 6 ? 2.0 + ls
-                                        : k <= 9 ? 0.5 * (2.0 + ls) : 0.0);
+    const double scale = 0.25 / mode_norm9(k);  // mode_scale
+    P.relax[k] = (float)(scale * (1.0 + l));
+    P.force[k] = (float)(scale * (k == 0 ? 0.0 : k <= 3 ? 0.5 * (2.0 + lm) : k == 4 ? 2.0 + lb : k <= 6 ? 2.0 + ls
+                                                 : k <= 9 ? 0.5 * (2.0 + ls) : 0.0));
     const double keep = 1.0 - (1.0 + l) * (1.0 + l);
     const double bk = mode_norm9(k) / 9.0;
-    P.noise[k] = (float)(k == 0 ? 0.0 : k <= 3 ? std::sqrt(prm->kT * keep) : std::sqrt(3.0 * prm->kT * bk * keep));
+    P.noise[k] = (float)(scale * (k == 0   ? 0.0
+                                  : k <= 3 ? std::sqrt(prm->kT * keep)
+                                           : std::sqrt(3.0 * prm->kT * bk * keep)));
   }
 }
 

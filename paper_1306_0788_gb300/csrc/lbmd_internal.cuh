@@ -68,7 +68,8 @@ struct StepParams {
   // fluctuating MRT (collision == LBMD_COLLISION_MRT): per mode k, relax[k] = 1 + lambda_k,
   // force[k] the factor of the forcing moment ((2 + lambda)/2 for the momenta, 2 + lambda for
   // the bulk and the normal shear modes, (2 + lambda)/2 for the off-diagonal ones), noise[k]
-  // the amplitude over sqrt(rho_z) (over sqrt(rho_A rho_B / rho) for the momenta, k = 1..3)
+  // the amplitude over sqrt(rho_z) (over sqrt(rho_A rho_B / rho) for the momenta, k = 1..3); all three
+  // times mode_scale(k)
   int collision;
   bool fluct;            // kT > 0: draw the mode noise
   // MD sub-stepping: K particle substeps per lattice step; the particle noise amplitude of a
