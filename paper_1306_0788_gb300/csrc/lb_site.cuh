@@ -251,6 +251,31 @@ __device__ __forceinline__ int shift(const NOff &o, int cx, int cy, int cz) {
          (cz < 0 ? o.m[2] : cz > 0 ? o.p[2] : 0);
 }
 
+// The element of `base` at a byte offset.  With a base the same for the whole warp the load adds the
+// 32-bit offset itself, and one offset serves every direction's plane of the populations and the densities,
+// where an element index took a 64-bit multiply-add each (fluctuating MRT, whose FMA pipes also have the
+// noise generator's multiplications: ten steps at 256^3 14367 -> 13968 us, twenty of 100x90x110 2004 -> 1977).
+template <class V>
+__device__ __forceinline__ V load_at(const V *__restrict__ base, unsigned byte) {
+  return __ldg(reinterpret_cast<const V *>(reinterpret_cast<const char *>(base) + byte));
+}
+
+// Byte offsets of site s32 and its neighbours in arrays of elements of `size` bytes (at most 8: 8 N < 2^32).
+struct ByteOffsets {
+  NOff o;
+  unsigned s;
+  __device__ __forceinline__ ByteOffsets(const NOff &n, unsigned s32, int size) : s(s32 * size) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      o.m[a] = n.m[a] * size;
+      o.p[a] = n.p[a] * size;
+    }
+  }
+  __device__ __forceinline__ unsigned operator()(int cx, int cy, int cz) const {
+    return s + (unsigned)shift(o, cx, cy, cz);
+  }
+};
+
 // Densities rho_z = sum_i f_zi (appendix, zeroth mode) of the node c at site s32, and j' = sum_z sum_i
 // f_zi c_i.
 struct NodeMoments {
@@ -680,8 +705,13 @@ __device__ __forceinline__ void collide_core_at(const StepParams &P, const Coord
                                                 const float *__restrict__ rest_in, float (&fA)[kQ],
                                                 float (&fB)[kQ], float &rA_out, float &rB_out,
                                                 const Rho &staged = Rho{}) {
-  const NOff o = neighbour_offsets(P, c);
   const unsigned N32 = (unsigned)P.N, s32 = (unsigned)s;
+  const NOff o = neighbour_offsets(P, c);
+  // (byte offsets in the FMA-bound update only: in the others they cost more registers than they save
+  // arithmetic -- density pass and update of FP16 at 256^3, ten steps, 8556 -> 9993 us with them, of
+  // FP32 at 64^3, fifty steps, 1128 -> 1154)
+  constexpr bool kBytes = kMRT && !kSplitRest<T>;
+  const ByteOffsets at(o, s32, sizeof(float2));
   // 16-bit storage with the BGK update: the moving populations stay shifted (f - w_i rho0, as
   // stored) through the update, the shifts folded into its constants, and the FP32 rest
   // population closes the node's mass
@@ -704,7 +734,9 @@ __device__ __forceinline__ void collide_core_at(const StepParams &P, const Coord
     const float2 *fin2 = reinterpret_cast<const float2 *>(fin);
 #pragma unroll
     for (int i = 0; i < kQ; ++i) {
-      const float2 v = __ldg(fin2 + i * N32 + (unsigned)((int)s32 + shift(o, -kCx[i], -kCy[i], -kCz[i])));  // pull r - c_i
+      const float2 v =  // pull r - c_i
+          kBytes ? load_at(fin2 + (size_t)i * N32, at(-kCx[i], -kCy[i], -kCz[i]))
+                 : __ldg(fin2 + i * N32 + (unsigned)((int)s32 + shift(o, -kCx[i], -kCy[i], -kCz[i])));
       fA[i] = v.x;
       fB[i] = v.y;
     }
@@ -751,8 +783,11 @@ __device__ __forceinline__ void collide_core_at(const StepParams &P, const Coord
       rp = staged(kCx[i], kCy[i], kCz[i]);
       rm = staged(-kCx[i], -kCy[i], -kCz[i]);
     } else {
-      rp = __ldg(rho2 + (unsigned)((int)s32 + shift(o, kCx[i], kCy[i], kCz[i])));
-      rm = __ldg(rho2 + (unsigned)((int)s32 + shift(o, -kCx[i], -kCy[i], -kCz[i])));
+      auto neighbour = [&](int cx, int cy, int cz) {
+        return kBytes ? load_at(rho2, at(cx, cy, cz)) : __ldg(rho2 + (unsigned)((int)s32 + shift(o, cx, cy, cz)));
+      };
+      rp = neighbour(kCx[i], kCy[i], kCz[i]);
+      rm = neighbour(-kCx[i], -kCy[i], -kCz[i]);
     }
     const float2 d = __ffma2_rn(make_float2(-1.f, -1.f), rm, rp);
     if (kCx[i]) Sx = __ffma2_rn(make_float2(kW[i] * kCx[i], kW[i] * kCx[i]), d, Sx);
