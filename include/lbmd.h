@@ -219,15 +219,16 @@ int lbmd_set_graphs(lbmd_ctx *ctx, int on);
  * of the update (the x edges of each 32-column tile, the first and last row of each 8-row tile
  * and the first and last plane of each z-chunk, 8 to 32 planes) by adding the partial sums the blocks
  * wrote -- or, on lattices too thin for them (tiles of 1-2 rows, one plane), by pulling their
- * populations -- and forms j' at the corners of the particles' cells for the next step's
+ * populations; another forms j' at the corners of the particles' cells for the next step's
  * coupling.  The one-pass update
  * reads the populations once per step instead of twice.  passes = 0 (the default) takes one
- * pass with FP32 storage on lattices large enough (about 96^3 and up, a little larger where the
- * tiles of 32 x 8 columns are ragged), two passes otherwise (with 16-bit storage the update is
+ * pass with FP32 storage on lattices large enough (about 96^3 and up, with the MRT collision about 144^3,
+ * larger where the tiles of 32 x 8 columns are ragged) if there is device memory for its partial sums,
+ * two passes otherwise (with 16-bit storage the update is
  * bound by instruction issue, not by the bytes the second pass reads); without particles, lattices
  * of up to 65536 nodes take the two passes in one launch (the same bits).  Both give the
  * same step up to FP32 rounding order (the densities are sums in another order).  One pass
- * needs the BGK collision and md_substeps = 1 (else LBMD_E_INVALID_ARG for passes = 1).  Drops
+ * needs md_substeps = 1, and passes = 1 the BGK collision too (else LBMD_E_INVALID_ARG).  Drops
  * the recorded graphs.  lbmd_get_lattice_passes returns the update the next step takes (1 or 2;
  * setting it up, the first time, allocates the partial-sum buffers) or a negative
  * LBMD_E_* code. */

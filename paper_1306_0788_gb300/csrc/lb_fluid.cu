@@ -269,7 +269,7 @@ __device__ __forceinline__ void stage_plane(const StepParams &P, const float *__
   cp_async_commit();
 }
 
-template <class T, bool kParticles>
+template <class T, bool kParticles, bool kMRT = false>
 __global__ void __launch_bounds__(kOPThreads, 3)
     k_collide_onepass(StepParams P, const T *__restrict__ fin, T *__restrict__ fout, const float *__restrict__ rho,
                       float *__restrict__ rho_next, OnePassOut out, ParticleArrays pa, ParticleForces pf,
@@ -331,9 +331,9 @@ __global__ void __launch_bounds__(kOPThreads, 3)
       float rA, rB;
       const StagedRho st{ring, (z + kRhoSlots - 1) & (kRhoSlots - 1), z & (kRhoSlots - 1),
                          (z + 1) & (kRhoSlots - 1), w + 1, lane + 1};
-      collide_core_at<T, kParticles, false, false, StagedRho>(P, Coord{x, y, z}, s, P.step, fin, rho, pa, pf, ci,
+      collide_core_at<T, kParticles, kMRT, false, StagedRho>(P, Coord{x, y, z}, s, P.step, fin, rho, pa, pf, ci,
                                                               err, rest_in, fA, fB, rA, rB, st);
-      store_node<T, false, true, true>(P, (unsigned)s, fout, rest_out, fA, fB, rA, rB);
+      store_node<T, kMRT, true, true>(P, (unsigned)s, fout, rest_out, fA, fB, rA, rB);
     } else {
 #pragma unroll
       for (int i = 0; i < kQ; ++i) fA[i] = fB[i] = 0.f;
@@ -870,12 +870,11 @@ void launch_collide_onepass(const StepParams &P, const void *fin, void *fout, co
     using T = std::remove_pointer_t<decltype(t)>;
     const T *a = static_cast<const T *>(fin);
     T *b = static_cast<T *>(fout);
-    if (P.np > 0)
-      k_collide_onepass<T, true><<<grid, kOPThreads, 0, st>>>(P, a, b, rho, rho_next, out, pa, pf, ci, err, rest_in,
-                                                              rest_out, G);
-    else
-      k_collide_onepass<T, false><<<grid, kOPThreads, 0, st>>>(P, a, b, rho, rho_next, out, pa, pf, ci, err, rest_in,
-                                                               rest_out, G);
+    auto *kernel = P.np > 0 ? k_collide_onepass<T, true> : k_collide_onepass<T, false>;
+    if constexpr (!kSplitRest<T>)
+      if (P.collision == LBMD_COLLISION_MRT)
+        kernel = P.np > 0 ? k_collide_onepass<T, true, true> : k_collide_onepass<T, false, true>;
+    kernel<<<grid, kOPThreads, 0, st>>>(P, a, b, rho, rho_next, out, pa, pf, ci, err, rest_in, rest_out, G);
   });
 }
 
@@ -919,8 +918,14 @@ bool is_noisy_update_of(const void *fn) {
          is(&k_step_small<T, true>);
 }
 
+bool is_noisy_onepass(const void *fn) {
+  return fn == reinterpret_cast<const void *>(&k_collide_onepass<float, true, true>) ||
+         fn == reinterpret_cast<const void *>(&k_collide_onepass<float, false, true>);
+}
+
 bool is_noisy_update(const void *fn) {
-  return is_noisy_update_of<float>(fn) || is_noisy_update_of<__half>(fn) || is_noisy_update_of<__nv_bfloat16>(fn);
+  return is_noisy_onepass(fn) || is_noisy_update_of<float>(fn) || is_noisy_update_of<__half>(fn) ||
+         is_noisy_update_of<__nv_bfloat16>(fn);
 }
 
 template <class... A>
@@ -929,8 +934,8 @@ constexpr int arity(void (*)(A...)) {
 }
 
 cudaError_t set_update_step(cudaGraphExec_t exec, cudaGraphNode_t node, unsigned long long step) {
-  constexpr int kArgs = arity(&k_collide<float, false, true>);
-  static_assert(kArgs == arity(&k_step_small<float, true>), "the noisy updates take the same parameters");
+  constexpr int kArgs = arity(&k_collide<float, false, true>), kOnePassArgs = arity(&k_collide_onepass<float, false, true>);
+  static_assert(kArgs == arity(&k_step_small<float, true>), "these noisy updates take the same parameters");
   cudaKernelNodeParams kp;
   cudaError_t e = cudaGraphKernelNodeGetParams(node, &kp);
   if (e != cudaSuccess) return e;
@@ -938,8 +943,9 @@ cudaError_t set_update_step(cudaGraphExec_t exec, cudaGraphNode_t node, unsigned
   StepParams P;
   std::memcpy(&P, kp.kernelParams[0], sizeof(P));  // the node's own copy of the parameters
   P.step = step;
-  void *args[kArgs];
-  for (int k = 0; k < kArgs; ++k) args[k] = kp.kernelParams[k];
+  const int nargs = is_noisy_onepass(kp.func) ? kOnePassArgs : kArgs;
+  void *args[kArgs > kOnePassArgs ? kArgs : kOnePassArgs];
+  for (int k = 0; k < nargs; ++k) args[k] = kp.kernelParams[k];
   args[0] = &P;
   kp.kernelParams = args;
   kp.extra = nullptr;

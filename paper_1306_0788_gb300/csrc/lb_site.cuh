@@ -896,7 +896,7 @@ template <class T, bool kMRT = false, bool kWrite = true, bool kKeep = false>
 __device__ __forceinline__ void store_node(const StepParams &P, unsigned s32, T *__restrict__ fout,
                                            float *__restrict__ rest_out, float (&fA)[kQ], float (&fB)[kQ],
                                            float rA, float rB, bool write = true) {
-  static_assert(!(kMRT && kKeep), "the stored values are kept for the BGK update only");
+  static_assert(!(kMRT && kKeep && kSplitRest<T>), "with MRT the stored values are kept in FP32 only");
   const unsigned N32 = (unsigned)P.N;
   constexpr bool kShifted = kSplitRest<T> && !kMRT;
   if constexpr (kSplitRest<T>) {

@@ -54,6 +54,7 @@ struct lbmd_ctx {
   cudaStream_t side = nullptr;
   cudaEvent_t ev_int = nullptr, ev_sorted = nullptr, ev_coupled = nullptr, ev_sub = nullptr;
   bool sort_pending = false;
+  bool onepass_no_room = false;  // the automatic choice found no device memory for the one-pass update
   // one pass with particles: the next step's corner j' (jc) is formed on side, at the sorted updated
   // particles, once the lattice update is done (ev_collided), beside the boundary densities on st
   cudaEvent_t ev_collided = nullptr;
@@ -266,12 +267,12 @@ void free_particles(lbmd_ctx *c) {
   c->cap = 0;
 }
 
-// One-pass update: BGK, one particle update per lattice step.  Chosen by the lattice size
-// unless set (lbmd_set_lattice_passes); see onepass_pays and onepass_chunks.
+// One-pass update: BGK, or MRT in FP32 (by size only), one particle update per lattice step.  Chosen by
+// the lattice size unless set (lbmd_set_lattice_passes); see onepass_pays and onepass_chunks.
 constexpr int kOnePassChunkPlanes = 16;
 
 bool onepass_allowed(const lbmd_ctx *c) {
-  return c->P.collision == LBMD_COLLISION_BGK && c->P.substeps == 1;
+  return (c->P.collision == LBMD_COLLISION_BGK || c->P.storage == LBMD_STORAGE_FP32) && c->P.substeps == 1;
 }
 
 // Whether one pass is the faster update, from what both took per step without particles (FP32,
@@ -280,9 +281,13 @@ bool onepass_allowed(const lbmd_ctx *c) {
 // 1124 / 886.  Two passes take about 72 ps per node there (less where the lattice stays in L2), one
 // pass 8 us and 53 ps per lane of its 32 x 8 tiles, idle ones included: it loses where tiles are
 // ragged (100 = 3 x 32 + 4 columns) and where the lattice is small.
+// Fluctuating MRT, whose update is nearer to what the FMA pipes can do than to what HBM can: 96^3 71.2 /
+// 74.0, 100 x 90 x 110 81.0 / 110.5, 128^3 162 / 160, 160^3 303 / 296, 192^3 514 / 502, 200 x 180 x 210 549 /
+// 592, 256^3 1198 / 1143: 71 ps per node against 10 us more and 67 ps per lane.
 bool onepass_pays(const StepParams &P) {
   const long long ntx = (P.nx + kOnePassCols - 1) / kOnePassCols, nty = (P.ny + kOnePassRows - 1) / kOnePassRows;
   const double lanes = (double)(ntx * nty * P.nz) * (kOnePassCols * kOnePassRows);
+  if (P.collision == LBMD_COLLISION_MRT) return 67.0 * lanes + 10.0e6 < 71.0 * (double)P.N;
   return 53.0 * lanes + 8.0e6 < 72.0 * (double)P.N;
 }
 
@@ -350,16 +355,9 @@ void free_onepass(lbmd_ctx *c) {
   c->op_grid = 0;
 }
 
-// Sets up the one-pass update (persistent grid, boundary runs) once per context; in the automatic
-// mode only for lattices large enough.  Allocates: call it before any capture.
-int prepare_onepass(lbmd_ctx *c) {
-  // set up already (op_grid; the run list may be empty: every node finished from partial sums)
-  if (!onepass_allowed(c) || c->passes == 2 || c->op_grid > 0) return LBMD_OK;
+// Sets up the one-pass update: its grid, chunks, partial sums and boundary runs.
+int setup_onepass(lbmd_ctx *c) {
   const StepParams &P = c->P;
-  // automatic: one pass for FP32 storage where it pays (the 16-bit update is bound by instruction
-  // issue, and the one-pass update's extra instructions cost it more than the second pass over half
-  // the bytes)
-  if (c->passes == 0 && (P.storage != LBMD_STORAGE_FP32 || !onepass_pays(P))) return LBMD_OK;  // two passes
   free_onepass(c);  // what an earlier attempt that failed part-way left
   const int ntx = (P.nx + kOnePassCols - 1) / kOnePassCols, nty = (P.ny + kOnePassRows - 1) / kOnePassRows;
   // neighbouring column tiles of a chunk are launched together (they march in step, so the sectors
@@ -415,6 +413,23 @@ int prepare_onepass(lbmd_ctx *c) {
   c->op_nruns = (int)runs.size();
   c->op_geom = OnePassGeom{ntx, nty, nchunks, ypart, zpart};
   c->op_grid = grid;
+  return LBMD_OK;
+}
+
+// setup_onepass once per context, where the next step takes one pass.  Allocates: call it before any
+// capture.
+int prepare_onepass(lbmd_ctx *c) {
+  // set up already (op_grid; the run list may be empty: every node finished from partial sums)
+  if (!onepass_allowed(c) || c->passes == 2 || c->op_grid > 0) return LBMD_OK;
+  if (c->passes == 1) return setup_onepass(c);
+  // automatic: one pass for FP32 storage where it pays (the 16-bit update is bound by instruction
+  // issue, and the one-pass update's extra instructions cost it more than the second pass over half
+  // the bytes) and where there is room for its partial sums
+  if (c->onepass_no_room || c->P.storage != LBMD_STORAGE_FP32 || !onepass_pays(c->P)) return LBMD_OK;  // two passes
+  const int r = setup_onepass(c);
+  if (!r || cudaGetLastError() != cudaErrorMemoryAllocation) return r;
+  free_onepass(c);
+  c->onepass_no_room = true;
   return LBMD_OK;
 }
 
@@ -1158,11 +1173,12 @@ int lbmd_set_graphs(lbmd_ctx *c, int on) {
 int lbmd_set_lattice_passes(lbmd_ctx *c, int passes) {
   if (!c) return LBMD_E_INVALID_ARG;
   if (passes < 0 || passes > 2) return fail(c, LBMD_E_INVALID_ARG, "passes must be 0 (by size), 1 or 2");
-  if (passes == 1 && !onepass_allowed(c))
+  if (passes == 1 && (c->P.collision != LBMD_COLLISION_BGK || !onepass_allowed(c)))
     return fail(c, LBMD_E_INVALID_ARG, "the one-pass update takes the BGK collision with md_substeps = 1");
   cudaSetDevice(c->dev);
   drop_graphs(c);
   if (passes != c->passes) {
+    c->onepass_no_room = false;
     free_onepass(c);  // set up again for the new choice at the next step
     c->jc_valid = false;
   }
