@@ -34,12 +34,13 @@ HBM_NOMINAL_GBS = 7900.0
 # 2706.7 + 2717.8 MB, two-pass FP32 2690.3 + 2515.6 MB, FP16 1479.4 + 1299.3 MB, BF16 1479.5 +
 # 1299.2 MB (a metric set that takes one ncu pass, so the full-size launch is captured).
 COLLIDE_TRAFFIC_BYTES_PER_NODE = {("fp32", 1): 323.3, ("fp32", 2): 310.3, ("bf16", 2): 165.6, ("fp16", 2): 165.6}
-# The fluctuating MRT update is bound by instruction issue, not by HBM: warp instructions per
-# node of k_collide<float, true, true> (smsp__inst_executed.sum / nodes of one ncu capture of the
-# 128^3 case), and the issue peak of the GPU: one warp instruction per cycle per scheduler, 4
-# schedulers per SM, 152 SMs, at the SM clock.
-MRT_WARP_INSTR_PER_NODE = 49.55
-MRT_TRAFFIC_BYTES_PER_NODE = 289.7  # DRAM bytes per node of the same capture (160.3 read + 129.4 written)
+# The fluctuating MRT update is bound by its arithmetic, not by HBM: warp instructions per node of
+# the FP32 update with particles, by lattice passes (smsp__inst_executed.sum / nodes of one ncu capture at
+# 160^3 with 4900 particles), and the issue peak of the GPU: one warp instruction per cycle per
+# scheduler, 4 schedulers per SM, 152 SMs, at the SM clock.
+MRT_WARP_INSTR_PER_NODE = {1: 52.45, 2: 40.96}
+# DRAM bytes per node of the two-pass MRT update (ncu, 128^3: 160.3 read + 129.4 written)
+MRT_TRAFFIC_BYTES_PER_NODE = {2: 289.7}
 SMS, SCHEDULERS_PER_SM = 152, 4
 
 # The slab/droplet workload uses the density scale of the paper's ferrofluid example (Sec. 4.5):
@@ -403,17 +404,20 @@ def collide_roofline(m, peak, peak_kind):
     if m["mrt"]:
         clk = m["clocks"].get("sm_mhz") or 2070.0
         issue_peak = SMS * SCHEDULERS_PER_SM * clk * 1e6
-        issued = MRT_WARP_INSTR_PER_NODE * N / (m["kernel_ms"] * 1e-3)
+        per_node = MRT_WARP_INSTR_PER_NODE[m["lattice_passes"]]
+        traffic = MRT_TRAFFIC_BYTES_PER_NODE.get(m["lattice_passes"]) if m["storage"] == "fp32" else None
+        issued = per_node * N / (m["kernel_ms"] * 1e-3)
         return {"bound": "alu", "scope": "kernel only (the lattice update)",
-                "kernel": "k_collide (pull streaming + Shan-Chen + coupling gather + fluctuating MRT with Philox "
+                "kernel": ("k_collide_onepass" if m["lattice_passes"] == 1 else "k_collide") +
+                          " (pull streaming + Shan-Chen + coupling gather + fluctuating MRT with Philox "
                           "noise, both components)",
                 "achieved": round(issued / 1e12, 4), "peak": round(issue_peak / 1e12, 4),
                 "peak_kind": "derived: 152 SMs x 4 schedulers x 1 warp instruction per cycle x the median SM "
                              "clock under load", "unit": "T warp-instructions/s",
-                "frac": round(issued / issue_peak, 4), "instructions_per_node": MRT_WARP_INSTR_PER_NODE,
+                "frac": round(issued / issue_peak, 4), "instructions_per_node": per_node,
                 "kernel_ms": round(m["kernel_ms"], 5), "kernel_launches": m["kernel_launches"],
                 "hbm_frac": round(achieved / peak, 4),
-                "traffic": int(MRT_TRAFFIC_BYTES_PER_NODE * N) if m["storage"] == "fp32" else None}
+                "traffic": int(traffic * N) if traffic else None}
     onep = m["lattice_passes"] == 1
     return {"bound": "hbm", "scope": "kernel only (the lattice update)",
             "kernel": ("k_collide_onepass (pull streaming + Shan-Chen + coupling gather + BGK/forcing, both components, "
