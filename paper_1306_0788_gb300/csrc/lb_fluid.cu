@@ -269,6 +269,9 @@ __device__ __forceinline__ void stage_plane(const StepParams &P, const float *__
   cp_async_commit();
 }
 
+// The one-pass update of the tile and chunk of the block.  kMRT (FP32 storage): the fluctuating MRT collision,
+// 1147 us at 256^3 with 20,000 particles for the two-pass update's 884 and its density pass's 376: bound by its
+// arithmetic, 52.5 warp instructions per node.
 template <class T, bool kParticles, bool kMRT = false>
 __global__ void __launch_bounds__(kOPThreads, 3)
     k_collide_onepass(StepParams P, const T *__restrict__ fin, T *__restrict__ fout, const float *__restrict__ rho,
