@@ -378,8 +378,8 @@ __device__ __forceinline__ void for_corner_bits(const StepParams &P, int4 c, F f
 // make rows of hundreds of entries), otherwise the row is scanned once (short rows: the
 // plain scan keeps the update's register budget).  kAhead: the four rows' entries are all looked up
 // before the first is walked, one latency instead of four (one pass at 128^3 with 2500 particles, twenty
-// steps: 2889 -> 2865 us; ten of 256^3 with 20,000: 10867 -> 10806).  Only the one-pass update has the
-// registers for it: 64^3 with 1000 particles 1115 -> 1125 us, fluctuating MRT at 256^3 14829 -> 15049.
+// steps: 2889 -> 2865 us; ten of 256^3 with 20,000: 10867 -> 10806, with fluctuating MRT 13601 -> 13483).  Not in
+// the two-pass update: 64^3 with 1000 particles 1115 -> 1125 us, fluctuating MRT at 256^3 14829 -> 15049.
 template <bool kBisect = false, bool kAhead = false>
 __device__ __forceinline__ void gather_coupling(const StepParams &P, int x, int y, int z, float rA, float rB,
                                                 const ParticleArrays &pa, const ParticleForces &pf,
@@ -511,8 +511,9 @@ __device__ __forceinline__ float4 fluid_normals4(const uint2 *__restrict__ keys,
 // Both transforms are factored, the two components together on (A, B) pairs with the packed two-lane
 // FP32 instructions.  Directions come in opposite pairs (2p + 1, 2p + 2) and every e_k is even or odd in c,
 // so they work on the pair sums and differences; and on the sums and differences of the two diagonal
-// pairs of a coordinate plane, on which every e_k is a small combination: 42 packed instructions for the
-// 104 nonzero terms of the plain sums each way.  (The update is bound by the FMA pipes.)
+// pairs of a coordinate plane, on which every e_k is a small combination: 40 packed instructions one way and
+// 43 the other for the 104 nonzero terms of the plain sums (ten steps at 256^3, two passes, 14709 -> 14368 us;
+// the update is bound by the FMA pipes).
 
 // sum and difference of (A, B) pairs, and their scaling
 __device__ __forceinline__ float2 pair_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
