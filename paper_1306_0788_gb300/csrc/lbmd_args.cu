@@ -126,7 +126,6 @@ int apply_types(StepParams &P, double kT, double dt, int ntypes, const lbmd_ptyp
   if (ntypes < 1 || ntypes > LBMD_MAX_TYPES || !types || npairs < 0 || (npairs > 0 && !pairs))
     return why = "bad type table", LBMD_E_INVALID_ARG;
   StepParams Q = P;  // applied only if every entry is valid
-  Q.any_lam = false;
   for (int t = 0; t < ntypes; ++t) {
     const lbmd_ptype &T = types[t];
     if (!(T.mass > 0.0) || !(T.gamma >= 0.0)) return why = "mass must be > 0, gamma >= 0", LBMD_E_INVALID_ARG;
@@ -135,13 +134,16 @@ int apply_types(StepParams &P, double kT, double dt, int ntypes, const lbmd_ptyp
     D.kappa[1] = (float)T.kappa_B;
     D.lam[0] = (float)T.lambda_A;
     D.lam[1] = (float)T.lambda_B;
-    Q.any_lam = Q.any_lam || D.lam[0] != 0.f || D.lam[1] != 0.f;
     D.gamma = (float)T.gamma;
     D.inv_mass = (float)(1.0 / T.mass);
     D.mass = (float)T.mass;
     D.noise_amp = (float)std::sqrt(2.0 * kT * T.gamma / dt);
     if (T.gamma * dt / T.mass > 0.5) w |= LBMD_WARN_GAMMA_DT;
   }
+  // the whole table: particles set before may be of a type that this one does not list, whose
+  // parameters stay
+  Q.any_lam = false;
+  for (const TypeParams &D : Q.types) Q.any_lam = Q.any_lam || D.lam[0] != 0.f || D.lam[1] != 0.f;
   for (int i = 0; i < LBMD_MAX_TYPES * LBMD_MAX_TYPES; ++i) Q.pairs[i] = PairParams{0.f, 0.f, 0.f, 0.f};
   for (int k = 0; k < npairs; ++k) {
     const lbmd_pair &pp = pairs[k];
