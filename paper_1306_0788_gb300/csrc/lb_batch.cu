@@ -69,9 +69,9 @@ struct BatchDev {
   ParticleArrays S;      // the same particles sorted by (row, x cell, id) during a step
   ParticleForces pf;     // forces, indexed like S (and like U after the update)
   int *row_of, *row_count, *row_start, *row_cursor, *bsum, *perm;
-  // CellIndex::node_bits of the replicas with particles, [nwords] for the present step at
-  // node_bits[*parity] (set from the particles' positions by the step before, or by a repack); the
-  // other half is cleared and takes the next step's
+  // FP32 storage (kMarkNodes): CellIndex::node_bits of the replicas with particles, [nwords] for the
+  // present step at node_bits[*parity] (set from the particles' positions by the step before, or by a
+  // repack); the other half is cleared and takes the next step's.  nwords = 0: none are kept
   unsigned *node_bits[2];
   int *parity;
   int nwords;
@@ -80,6 +80,14 @@ struct BatchDev {
 };
 
 // ------------------------------------------------------------------ lattice kernels
+
+// Whether the density pass stores j' and the update gathers at the marked nodes only, or the one at
+// every node and the other after a look at the node's rows.  Marks pay in FP32: eight replicas of 64^3
+// with 635 particles each 207 us a step, without them 209, 24 of 18^3 to 125^3 about 3 %.  In 16 bits,
+// where both kernels are bound by instruction issue and not by the 12 bytes of j', they cost more
+// than they save: the eight 170 us a step with marks, 154 without, 100 of 32^3 with 88 each 237 and 219.
+template <class T>
+constexpr bool kMarkNodes = !site::kSplitRest<T>;
 
 // tuning != 0: time the update without side effects on the state -- no particle coupling (the
 // sorted particle arrays are only valid inside a step) and, with 16-bit storage, the FP32 rest
@@ -168,7 +176,7 @@ __global__ void __launch_bounds__(kBThreads, 4) kb_moments(const BatchDev *__res
     for (int k = threadIdx.x; k < ts; k += kBThreads) {
       const long long s = c.base + k;
       if (s >= c.P.N) break;
-      site::moments<T>(c.P, s, c.fin, c.rest_in, c.rho, c.jp, c.ci.node_bits);
+      site::moments<T>(c.P, s, c.fin, c.rest_in, c.rho, c.jp, kMarkNodes<T> ? c.ci.node_bits : nullptr);
     }
     __syncthreads();  // the next context is complete; this one is free for the tile after it
     t = tn;
@@ -198,8 +206,8 @@ __global__ void __launch_bounds__(kBThreads, kMinBlocks) kb_collide(const BatchD
       const long long s = c.base + k;
       if (s >= c.P.N) break;
       if (c.ci.row_start)
-        site::collide<T, true, kMRT>(c.P, s, c.step, c.fin, c.fout, c.rho, c.pa, c.pf, c.ci, c.err, c.rest_in,
-                                     c.rest_out);
+        site::collide<T, true, kMRT, false, kMarkNodes<T>>(c.P, s, c.step, c.fin, c.fout, c.rho, c.pa, c.pf, c.ci,
+                                                           c.err, c.rest_in, c.rest_out);
       else
         site::collide<T, false, kMRT>(c.P, s, c.step, c.fin, c.fout, c.rho, c.pa, c.pf, c.ci, c.err, c.rest_in,
                                       c.rest_out);
@@ -211,8 +219,9 @@ __global__ void __launch_bounds__(kBThreads, kMinBlocks) kb_collide(const BatchD
 
 // ------------------------------------------------------------------ particle sort
 
-// Sets the node bits of the particle of `slot` in cell c.
+// Sets the node bits of the particle of `slot` in cell c (where they are kept).
 __device__ __forceinline__ void mark_nodes(const BatchDev *__restrict__ B, int slot, int4 c, unsigned *node_bits) {
+  if (B->nwords == 0) return;
   unsigned *bits = node_bits + B->lay[slot].bits0;
   site::for_corner_bits(B->rep[slot].P, c, [&](long long w, unsigned b) { atomicOr(bits + w, b); });
 }
@@ -887,7 +896,7 @@ int repack(lbmd_batch *b) {
       sl.lay.row0 = nrows;
       sl.lay.bits0 = nwords;
       nrows += sl.P.nrows;
-      nwords += sl.P.nrows * node_words(sl.P.nx);
+      if (b->storage == LBMD_STORAGE_FP32) nwords += sl.P.nrows * node_words(sl.P.nx);  // kMarkNodes
     } else {
       sl.lay.row0 = sl.lay.bits0 = 0;
     }
@@ -932,7 +941,7 @@ int repack(lbmd_batch *b) {
   b->hb.pslot = b->d_pslot;
   r = upload_tables(b);
   if (r) return r;
-  if (np > 0) {
+  if (nwords > 0) {
     kb_mark<<<std::max(1, std::min(b->grid_particles, (np + kBPThreads - 1) / kBPThreads)), kBPThreads, 0, b->st>>>(b->d_batch);
     BK(cudaGetLastError(), "mark nodes");
     b->launches++;

@@ -698,7 +698,8 @@ struct GlobalRho {
 // MODES, `step` being the noise counter).  On return fA, fB hold the post-collision values
 // (16-bit storage with BGK: the moving ones shifted by w_i rho0, as stored) and rA, rB the node's
 // densities before the collision.
-template <class T, bool kParticles, bool kMRT = false, bool kBisect = false, class Rho = GlobalRho>
+// kMarked: ci.node_bits says which nodes gather (else every node looks up its rows).
+template <class T, bool kParticles, bool kMRT = false, bool kBisect = false, class Rho = GlobalRho, bool kMarked = true>
 __device__ __forceinline__ void collide_core_at(const StepParams &P, const Coord c, long long s,
                                                 unsigned long long step, const T *__restrict__ fin,
                                                 const float *__restrict__ rho, const ParticleArrays &pa,
@@ -805,8 +806,9 @@ __device__ __forceinline__ void collide_core_at(const StepParams &P, const Coord
   // One load decides for the nodes that no particle reaches, almost all of them.  Looking up the
   // four rows of every node instead cost the update at 256^3 with 20,000 particles 50 of 1056 us
   // (fluctuating MRT, bound by instruction issue), 9 of 878 (one pass, FP32), 4 of 580 (FP16), and
-  // the batched update of 24 replicas about 30 of 800.
-  if (kParticles && node_touched(P, c, ci.node_bits))
+  // the batched update of 24 replicas in FP32 about 30 of 800 (in 16 bits it costs them time: see
+  // kMarkNodes of the batch).
+  if (kParticles && (!kMarked || node_touched(P, c, ci.node_bits)))
     gather_coupling<kBisect, Rho::kStaged>(P, c.x, c.y, c.z, rA, rB, pa, pf, ci, true, gA, gB);
   const float r = rA + rB;
   if (!(rA > 0.f) || !(rB > 0.f) || !isfinite(r)) atomicOr(err, isfinite(r) ? kErrNegDensity : kErrNonFinite);
@@ -877,14 +879,14 @@ __device__ __forceinline__ void collide_core_at(const StepParams &P, const Coord
 }
 
 // collide_core at site s, its coordinates computed from the index.
-template <class T, bool kParticles, bool kMRT = false, bool kBisect = false>
+template <class T, bool kParticles, bool kMRT = false, bool kBisect = false, bool kMarked = true>
 __device__ __forceinline__ void collide_core(const StepParams &P, long long s, unsigned long long step,
                                              const T *__restrict__ fin, const float *__restrict__ rho,
                                              const ParticleArrays &pa, const ParticleForces &pf, CellIndex ci,
                                              unsigned *err, const float *__restrict__ rest_in, float (&fA)[kQ],
                                              float (&fB)[kQ], float &rA_out, float &rB_out) {
-  collide_core_at<T, kParticles, kMRT, kBisect>(P, site_coord(P, s), s, step, fin, rho, pa, pf, ci, err, rest_in,
-                                                fA, fB, rA_out, rB_out);
+  collide_core_at<T, kParticles, kMRT, kBisect, GlobalRho, kMarked>(P, site_coord(P, s), s, step, fin, rho, pa, pf, ci,
+                                                                    err, rest_in, fA, fB, rA_out, rB_out);
 }
 
 // The store of the update at site s32 (values from collide_core).  With 16-bit storage rest_out
@@ -962,7 +964,7 @@ __device__ __forceinline__ void store_node(const StepParams &P, unsigned s32, T 
 }
 
 // The whole lattice update of one step at site s: collide_core, then the store.
-template <class T, bool kParticles, bool kMRT = false, bool kBisect = false>
+template <class T, bool kParticles, bool kMRT = false, bool kBisect = false, bool kMarked = true>
 __device__ __forceinline__ void collide(const StepParams &P, long long s, unsigned long long step,
                                         const T *__restrict__ fin,
                                         T *__restrict__ fout, const float *__restrict__ rho,
@@ -970,7 +972,7 @@ __device__ __forceinline__ void collide(const StepParams &P, long long s, unsign
                                         unsigned *err, const float *__restrict__ rest_in,
                                         float *__restrict__ rest_out) {
   float fA[kQ], fB[kQ], rA, rB;
-  collide_core<T, kParticles, kMRT, kBisect>(P, s, step, fin, rho, pa, pf, ci, err, rest_in, fA, fB, rA, rB);
+  collide_core<T, kParticles, kMRT, kBisect, kMarked>(P, s, step, fin, rho, pa, pf, ci, err, rest_in, fA, fB, rA, rB);
   store_node<T, kMRT>(P, (unsigned)s, fout, rest_out, fA, fB, rA, rB);
 }
 
