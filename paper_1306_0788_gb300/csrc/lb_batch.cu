@@ -603,6 +603,8 @@ size_t particle_bytes(const StepParams &P, int np_max) {
   return (size_t)np_max * kParticleBytes * 5 / 4 + ((size_t)P.nrows + 1) * 3 * 4;  // 25 % capacity slack; rows
 }
 
+constexpr int kMixBGK = 1, kMixMRT = 2, kMixParticles = 4;
+
 }  // namespace
 
 struct lbmd_batch {
@@ -642,10 +644,10 @@ struct lbmd_batch {
   bool shaped = false;
   int tile_sites = 1024, grid_moments = 0, grid_collide = 0, grid_particles = 0;
   int collide_blocks = 2;  // register budget of the update kernel: blocks per SM
-  // collisions among the replicas of the tables: bit 0 BGK, bit 1 MRT (the update launches only
-  // the variants in use)
+  // what is among the replicas of the tables (kMix*): a step launches only the update's variants in
+  // use, and the particle kernels only where there are particles
   int mix = 0;
-  std::map<int, cudaGraphExec_t> graphs;  // by steps per graph and mix: 4 n + mix
+  std::map<int, cudaGraphExec_t> graphs;  // by steps per graph and mix: 8 n + mix
   int64_t launches = 0;
   std::string msg;
 };
@@ -932,8 +934,8 @@ int repack(lbmd_batch *b) {
   if (!b->shaped) b->tile_sites = default_tile(b, act);
   int r = build_tiles(b, act);
   if (r) return r;
-  b->mix = 0;
-  for (int s : act) b->mix |= b->slots[s].P.collision == LBMD_COLLISION_MRT ? 2 : 1;
+  b->mix = np > 0 ? kMixParticles : 0;
+  for (int s : act) b->mix |= b->slots[s].P.collision == LBMD_COLLISION_MRT ? kMixMRT : kMixBGK;
   b->hb.nrep = (int)act.size();
   b->hb.np = np;
   b->hb.nrows = nrows;
@@ -967,25 +969,20 @@ void launch_batched_moments(lbmd_batch *b, int grid) {
 }
 
 // The BGK replicas with the tuned shape, then the MRT ones (two blocks of 256 per SM: at three the
-// tile context spills heavily); a variant no replica uses is not launched.  Returns the number of
-// launches.
-int launch_batched_collide(lbmd_batch *b, int grid, int min_blocks, int tuning) {
-  int n = 0;
+// tile context spills heavily); a variant no replica uses is not launched.
+void launch_batched_collide(lbmd_batch *b, int grid, int min_blocks, int tuning) {
   with_batch_storage(b->storage, [&](auto t) {
     using T = std::remove_pointer_t<decltype(t)>;
-    if (b->mix & 1) {
+    if (b->mix & kMixBGK) {
       if (min_blocks == 2)
         kb_collide<T, 2, false><<<grid, kBThreads, 0, b->st>>>(b->d_batch, tuning);
       else
         kb_collide<T, 3, false><<<grid, kBThreads, 0, b->st>>>(b->d_batch, tuning);
-      ++n;
     }
-    if (b->mix & 2) {
+    if (b->mix & kMixMRT) {
       kb_collide<T, 2, true><<<2 * b->sms, kBThreads, 0, b->st>>>(b->d_batch, tuning);
-      ++n;
     }
   });
-  return n;
 }
 
 // The drift check of the replicas due (two launches; a replica not due costs its tiles a test).
@@ -997,42 +994,54 @@ void launch_drift(lbmd_batch *b) {
   kb_drift_finish<<<2 * b->sms, kBThreads, 0, b->st>>>(b->d_batch);
 }
 
-// Enqueues one step; returns the number of kernel launches.
+// Enqueues one step.
 // The particle sort and the pair forces depend on the particles only: they run on the side
 // stream beside the density pass, forked from st at the start of the step and joined before the
 // coupling (sorted rows); the particle update follows there once the coupling is done, beside the
 // lattice update, and is joined before the end of the step.
-int enqueue_step(lbmd_batch *b) {
+// Without particles none of it is launched: beside the lattice update, even blocks with nothing to do
+// take slots from its own (tiles of 1024 sites, three blocks per SM: eight replicas of 64^3 in FP16 136 us
+// a step with the empty launches, 121 without, 400 of 16^3 in FP32 155 and 149).
+void enqueue_step(lbmd_batch *b) {
   const BatchDev *B = b->d_batch;
   const int gp = b->grid_particles;
+  const bool parts = b->mix & kMixParticles;
   cudaStream_t sd = b->side;
-  cudaEventRecord(b->ev_fork, b->st);
-  cudaStreamWaitEvent(sd, b->ev_fork, 0);
-  kb_bin<<<gp, kBPThreads, 0, sd>>>(B);
-  kb_scan_partial<<<gp, site::kScanThreads, 0, sd>>>(B);
-  kb_scan_top<<<1, site::kScanThreads, 0, sd>>>(B);
-  kb_scan_final<<<gp, site::kScanThreads, 0, sd>>>(B);
-  kb_scatter<<<gp, kBPThreads, 0, sd>>>(B);
-  kb_row_sort<<<gp, kBPThreads, 0, sd>>>(B);
-  kb_permute<<<gp, kBPThreads, 0, sd>>>(B);
-  cudaEventRecord(b->ev_sorted, sd);
+  if (parts) {
+    cudaEventRecord(b->ev_fork, b->st);
+    cudaStreamWaitEvent(sd, b->ev_fork, 0);
+    kb_bin<<<gp, kBPThreads, 0, sd>>>(B);
+    kb_scan_partial<<<gp, site::kScanThreads, 0, sd>>>(B);
+    kb_scan_top<<<1, site::kScanThreads, 0, sd>>>(B);
+    kb_scan_final<<<gp, site::kScanThreads, 0, sd>>>(B);
+    kb_scatter<<<gp, kBPThreads, 0, sd>>>(B);
+    kb_row_sort<<<gp, kBPThreads, 0, sd>>>(B);
+    kb_permute<<<gp, kBPThreads, 0, sd>>>(B);
+    cudaEventRecord(b->ev_sorted, sd);
+  }
   launch_batched_moments(b, b->grid_moments);
-  cudaStreamWaitEvent(b->st, b->ev_sorted, 0);
-  // the coupling and the pair forces walk chains of dependent loads per particle: a grid of
-  // kPairGrid times the particle grid (blocks beyond the resident ones queue) leaves each of their
-  // threads about one particle instead of a few in a row
-  kb_couple<<<kPairGrid * gp, kBPThreads, 0, b->st>>>(B);
-  cudaEventRecord(b->ev_coupled, b->st);
-  kb_pairs<<<kPairGrid * gp, kBPThreads, 0, sd>>>(B);
-  // the particle update beside the lattice update, which reads the sorted copy
-  cudaStreamWaitEvent(sd, b->ev_coupled, 0);
-  kb_integrate<<<gp, kBPThreads, 0, sd>>>(B);
-  cudaEventRecord(b->ev_moved, sd);
-  const int nc = launch_batched_collide(b, b->grid_collide, b->collide_blocks, 0);
-  cudaStreamWaitEvent(b->st, b->ev_moved, 0);
+  if (parts) {
+    cudaStreamWaitEvent(b->st, b->ev_sorted, 0);
+    // the coupling and the pair forces walk chains of dependent loads per particle: a grid of
+    // kPairGrid times the particle grid (blocks beyond the resident ones queue) leaves each of their
+    // threads about one particle instead of a few in a row
+    kb_couple<<<kPairGrid * gp, kBPThreads, 0, b->st>>>(B);
+    cudaEventRecord(b->ev_coupled, b->st);
+    kb_pairs<<<kPairGrid * gp, kBPThreads, 0, sd>>>(B);
+    // the particle update beside the lattice update, which reads the sorted copy
+    cudaStreamWaitEvent(sd, b->ev_coupled, 0);
+    kb_integrate<<<gp, kBPThreads, 0, sd>>>(B);
+    cudaEventRecord(b->ev_moved, sd);
+  }
+  launch_batched_collide(b, b->grid_collide, b->collide_blocks, 0);
+  if (parts) cudaStreamWaitEvent(b->st, b->ev_moved, 0);
   kb_advance<<<1, 256, 0, b->st>>>(B);
   launch_drift(b);
-  return 14 + nc;
+}
+
+// Kernel launches of a step.
+int step_launches(const lbmd_batch *b) {
+  return 4 + (b->mix & kMixParticles ? 10 : 0) + (b->mix & kMixBGK ? 1 : 0) + (b->mix & kMixMRT ? 1 : 0);
 }
 
 void drop_graphs(lbmd_batch *b) {
@@ -1040,20 +1049,19 @@ void drop_graphs(lbmd_batch *b) {
   b->graphs.clear();
 }
 
-// The graph of n steps for the current mix of collisions (captured once per n and mix);
+// The graph of n steps for the current mix (captured once per n and mix);
 // *launches receives its kernel launches.
 int graph_for(lbmd_batch *b, int n, cudaGraphExec_t *out, int *launches) {
-  const int key = 4 * n + b->mix;
+  const int key = 8 * n + b->mix;
   auto it = b->graphs.find(key);
-  int per_step = 0;
+  *launches = n * step_launches(b);
   if (it != b->graphs.end()) {
     *out = it->second;
-    *launches = n * (14 + ((b->mix & 1) != 0) + ((b->mix & 2) != 0));
     return LBMD_OK;
   }
   cudaGraph_t g = nullptr;
   BK(cudaStreamBeginCapture(b->st, cudaStreamCaptureModeThreadLocal), "begin capture");
-  for (int k = 0; k < n; ++k) per_step = enqueue_step(b);
+  for (int k = 0; k < n; ++k) enqueue_step(b);
   cudaError_t e = cudaStreamEndCapture(b->st, &g);
   if (e != cudaSuccess) return bcuda(b, e, "end capture");
   cudaGraphExec_t x = nullptr;
@@ -1062,7 +1070,6 @@ int graph_for(lbmd_batch *b, int n, cudaGraphExec_t *out, int *launches) {
   if (e != cudaSuccess) return bcuda(b, e, "instantiate graph");
   b->graphs[key] = x;
   *out = x;
-  *launches = n * per_step;
   return LBMD_OK;
 }
 
