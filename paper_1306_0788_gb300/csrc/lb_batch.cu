@@ -796,16 +796,30 @@ std::vector<int> active_slots(const lbmd_batch *b) {
   return act;
 }
 
-// The tile size without tuning: the largest that leaves the update's blocks two tiles each.  24 replicas
-// of 18^3 to 125^3 (13.1 M sites, 42,000 particles), ms per step: tiles of 512 / 1024 / 2048 / 4096 sites
-// at 8 blocks of 128 registers per SM queued 1.157 / 1.114 / 1.116 / 1.091; at 2 per SM 1.149 / 1.127 / 1.121 /
-// 1.100; at 3 blocks of 80 registers 1.194 / 1.168 / 1.171 / 1.188 (1024 was the default).
+// The launch shape without tuning, from the step times of 40 sets of replicas (one of 16^3 to 24 of up to 128^3,
+// 4 k to 34 M sites, with and without particles), over tiles of 256 to 8192 sites and 2 or 3 blocks per SM,
+// resident or queued.  FP32: blocks of 128 registers, two per SM, sixteen queued, which even out what tiles
+// with more or fewer particles take; 16 bits, bound by instruction issue: three resident ones of 80.  The
+// tile is the largest, up to 2048 sites in FP32 and 1024 in 16 bits, that gives each resident block one:
+// larger ones leave blocks idle, smaller ones cost more tile contexts.  FP32, 14 sets of the serving
+// distribution (5 to 17 M sites with particles) against 1024 sites at three resident blocks, the
+// default before: 0.92 to 0.96 of its step time; 4096 sites at eight queued 0.91 to 0.99; 2048 and 1024 at two
+// resident 0.93 to 0.98 and 0.94 to 0.97.  Eight queued blocks for both storages with tiles of at most two a
+// block lost up to 27 % on sets of small replicas and 5 to 11 % in 16 bits.
+struct DefaultShape {
+  int tile_sites, collide_blocks, grid;  // most sites of a tile, blocks per SM resident, launched
+};
+constexpr DefaultShape default_shape(int storage) {
+  return storage == LBMD_STORAGE_FP32 ? DefaultShape{2048, 2, 16} : DefaultShape{1024, 3, 3};
+}
+
 int default_tile(const lbmd_batch *b, const std::vector<int> &act) {
-  int ts = 4096;
+  const DefaultShape D = default_shape(b->storage);
+  int ts = D.tile_sites;
   for (; ts > kBThreads; ts /= 2) {
     long long tiles = 0;
     for (int s : act) tiles += (b->slots[s].P.N + ts - 1) / ts;
-    if (tiles >= 2LL * b->grid_collide) break;
+    if (tiles >= (long long)D.collide_blocks * b->sms) break;
   }
   return ts;
 }
@@ -1172,7 +1186,8 @@ int lbmd_batch_create(size_t mem_budget, int storage, int max_slots, void *strea
   b->max_slots = max_slots;
   b->slots.resize(max_slots);
   b->grid_moments = 4 * b->sms;
-  b->grid_collide = 8 * b->sms;
+  b->collide_blocks = default_shape(storage).collide_blocks;
+  b->grid_collide = default_shape(storage).grid * b->sms;
   b->grid_particles = 8 * b->sms;
   b->hb.rep = b->d_rep;
   b->hb.state = b->d_state;
