@@ -53,6 +53,7 @@ struct RepLayout {   // per slot, written by the host at each repack
   int row0;          // first row of the replica in the shared row space (-1: no particles)
   int p0;            // first slot of the replica in the particle arrays
   int bits0;         // first word of the replica in the node bits
+  int chunk0;        // first chunk of the replica in the sums of the drift check
 };
 
 struct BatchDev {
@@ -75,7 +76,8 @@ struct BatchDev {
   unsigned *node_bits[2];
   int *parity;
   int nwords;
-  double *tile_sums;     // [ntiles][5] FP64 sums of the drift check
+  double *chunk_sums;    // [nchunks][5] FP64 sums of the drift check, kDriftSites sites of a replica each
+  int nchunks;
   double *drift;         // [max_slots][10]: reference totals [5], last check {step, dA, dB, dP, n}
 };
 
@@ -446,7 +448,11 @@ __device__ __forceinline__ bool drift_due(const RepDev &R, const RepState &S) {
          (S.ref_req || (S.step % (unsigned long long)R.diag_every == 0 && S.step != S.checked));
 }
 
-// FP64 sums [M_A, M_B, Px, Py, Pz] of every tile of the replicas due for a drift check, over
+// The sums are grouped by chunks of a replica of fixed size, and not by the tiles of the lattice
+// kernels, whose size follows the other replicas: the totals of a replica are the same in any mix.
+constexpr int kDriftSites = 1024;
+
+// FP64 sums [M_A, M_B, Px, Py, Pz] of every chunk of the replicas due for a drift check, over
 // the current buffer (streaming permutes populations, so the stored values sum alike).
 template <class T>
 __global__ void __launch_bounds__(kBThreads) kb_drift_sums(const BatchDev *__restrict__ B) {
@@ -459,24 +465,31 @@ __global__ void __launch_bounds__(kBThreads) kb_drift_sums(const BatchDev *__res
     any = any || drift_due(B->rep[slot], B->state[slot]);
   }
   if (!__syncthreads_or(any)) return;
-  const int ts = B->tile_sites;
-  for (int t = blockIdx.x; t < B->ntiles; t += gridDim.x) {
-    const int slot = B->tile_slot[t];
+  for (int c = blockIdx.x; c < B->nchunks; c += gridDim.x) {
+    int lo = 0, hi = B->nrep - 1;  // the replica of chunk c: the last one that starts at or before it
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (B->lay[B->rep_slot[mid]].chunk0 <= c)
+        lo = mid;
+      else
+        hi = mid - 1;
+    }
+    const int slot = B->rep_slot[lo];
     const RepDev &R = B->rep[slot];
     const RepState &S = B->state[slot];
     if (!drift_due(R, S)) continue;  // uniform across the block
     const StepParams &P = R.P;
     const T *f = static_cast<const T *>(R.pop[S.cur]);
-    const long long base = (long long)(t - B->lay[slot].tile0) * ts;
+    const long long base = (long long)(c - B->lay[slot].chunk0) * kDriftSites;
     site::TotalSums sums;
-    for (int k = threadIdx.x; k < ts; k += kBThreads) {
+    for (int k = threadIdx.x; k < kDriftSites; k += kBThreads) {
       const long long s = base + k;
       if (s >= P.N) break;
       sums.add([&](int i) { return site::pop_pair<T>(P, f, R.rest, i, (unsigned)s); });
     }
     sums.flush();
     const double *acc = sums.acc;
-    __syncthreads();  // sh is free (previous tile)
+    __syncthreads();  // sh is free (previous chunk)
 #pragma unroll
     for (int k = 0; k < 5; ++k) sh[k][threadIdx.x] = acc[k];
     __syncthreads();
@@ -488,11 +501,11 @@ __global__ void __launch_bounds__(kBThreads) kb_drift_sums(const BatchDev *__res
     }
     if (threadIdx.x == 0)
 #pragma unroll
-      for (int k = 0; k < 5; ++k) B->tile_sums[(long long)t * 5 + k] = sh[k][0];
+      for (int k = 0; k < 5; ++k) B->chunk_sums[(long long)c * 5 + k] = sh[k][0];
   }
 }
 
-// Per replica due: its tiles' sums plus the momentum of its particles, in a fixed order; then
+// Per replica due: its chunks' sums plus the momentum of its particles, in a fixed order; then
 // either the new reference or the comparison with it (kErrDrift beyond the tolerance: the
 // replica takes no further step, like after any device error).
 __global__ void __launch_bounds__(kBThreads) kb_drift_finish(const BatchDev *__restrict__ B) {
@@ -503,11 +516,11 @@ __global__ void __launch_bounds__(kBThreads) kb_drift_finish(const BatchDev *__r
     RepState &S = B->state[slot];
     if (!drift_due(R, S)) continue;  // uniform across the block
     const RepLayout &L = B->lay[slot];
-    const int nt = (int)((R.P.N + B->tile_sites - 1) / B->tile_sites);
+    const int nc = (int)((R.P.N + kDriftSites - 1) / kDriftSites);
     double acc[5] = {0, 0, 0, 0, 0};
-    for (int t = threadIdx.x; t < nt; t += kBThreads)
+    for (int c = threadIdx.x; c < nc; c += kBThreads)
 #pragma unroll
-      for (int k = 0; k < 5; ++k) acc[k] += B->tile_sums[(long long)(L.tile0 + t) * 5 + k];
+      for (int k = 0; k < 5; ++k) acc[k] += B->chunk_sums[(long long)(L.chunk0 + c) * 5 + k];
     for (int p = threadIdx.x; p < R.P.np; p += kBThreads) {
       const int q = L.p0 + p;
       const float4 v = B->U.vel[q];
@@ -583,7 +596,7 @@ struct Slot {
   std::vector<int4> hc;
   std::vector<float4> hf, hv;
   std::vector<int> hid;
-  RepLayout lay{-1, -1, 0, 0};
+  RepLayout lay{-1, -1, 0, 0, 0};
   bool ref_pending = false;  // a drift reference is requested and not yet taken
 };
 
@@ -638,7 +651,7 @@ struct lbmd_batch {
   double *diag_partial = nullptr, *diag_out = nullptr;
   int diag_cap = 0;
   double *d_drift = nullptr;  // [max_slots][10] (BatchDev::drift)
-  double *d_tile_sums = nullptr;  // [tile_cap][5] (BatchDev::tile_sums)
+  size_t chunk_cap = 0;            // capacity of the drift check's sums (chunks)
   bool dirty = true;
   // launch shape; until it is set or tuned, each repack chooses the tile size (default_tile)
   bool shaped = false;
@@ -764,10 +777,8 @@ int build_tiles(lbmd_batch *b, const std::vector<int> &act) {
   if (tiles.size() > 0x7fffffffull) return bfail(b, LBMD_E_INVALID_ARG, "too many tiles");
   if (tiles.size() > b->tile_cap) {
     pfree(b, b->d_tile_slot);
-    pfree(b, b->d_tile_sums);
     const size_t cap = tiles.size() + tiles.size() / 4;
     BK(palloc(b, &b->d_tile_slot, cap), "tile table");
-    BK(palloc(b, &b->d_tile_sums, 5 * cap), "tile sums");
     b->tile_cap = cap;
   }
   if (!tiles.empty())
@@ -776,7 +787,6 @@ int build_tiles(lbmd_batch *b, const std::vector<int> &act) {
   b->hb.ntiles = (int)tiles.size();
   b->hb.tile_sites = b->tile_sites;
   b->hb.tile_slot = b->d_tile_slot;
-  b->hb.tile_sums = b->d_tile_sums;
   return LBMD_OK;
 }
 
@@ -940,6 +950,21 @@ int repack(lbmd_batch *b) {
     b->bcap = bcap;
   }
   BK(cudaMemsetAsync(b->hb.row_count, 0, sizeof(int) * (nrows + 1), b->st), "clear rows");
+  // chunks of the drift check
+  long long nchunks = 0;
+  for (int s : act) {
+    b->slots[s].lay.chunk0 = (int)nchunks;
+    nchunks += (b->slots[s].P.N + kDriftSites - 1) / kDriftSites;
+  }
+  if (nchunks > 0x7fffffffLL) return bfail(b, LBMD_E_INVALID_ARG, "too many sites");
+  if ((size_t)nchunks > b->chunk_cap) {
+    pfree(b, b->hb.chunk_sums);
+    b->chunk_cap = 0;
+    const size_t cap = (size_t)(nchunks + nchunks / 4);
+    BK(palloc(b, &b->hb.chunk_sums, 5 * cap), "drift sums");
+    b->chunk_cap = cap;
+  }
+  b->hb.nchunks = (int)nchunks;
   // replicas, tiles
   std::vector<int> rep_slot(act.begin(), act.end());
   if (!rep_slot.empty())
@@ -1107,12 +1132,10 @@ void lbmd_batch_destroy(lbmd_batch *b) {
   pfree(b, b->hb.row_of); pfree(b, b->hb.perm); pfree(b, b->d_pslot);
   pfree(b, b->hb.row_count); pfree(b, b->hb.row_start); pfree(b, b->hb.row_cursor); pfree(b, b->hb.bsum);
   pfree(b, b->hb.node_bits[0]); pfree(b, b->hb.node_bits[1]);
-  pfree(b, b->d_tile_slot);
+  pfree(b, b->d_tile_slot); pfree(b, b->hb.chunk_sums);
   cudaStreamSynchronize(b->st);
   if (b->pool) cudaMemPoolDestroy(b->pool);
   cudaFree(b->d_rep); cudaFree(b->d_state); cudaFree(b->d_lay); cudaFree(b->d_left); cudaFree(b->d_rep_slot);
-  pfree(b, b->d_tile_sums);
-  cudaStreamSynchronize(b->st);
   cudaFree(b->hb.parity);
   cudaFree(b->d_batch); cudaFree(b->diag_partial); cudaFree(b->diag_out); cudaFree(b->d_drift);
   if (b->own_stream) cudaStreamDestroy(b->st);
