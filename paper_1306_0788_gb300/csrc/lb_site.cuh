@@ -133,63 +133,110 @@ __device__ __forceinline__ float2 pop_pair(const StepParams &P, const T *buf, co
   }
 }
 
-// Sums of (A, B) pairs of FP32 values almost without rounding error: each lane is kept as an
-// unevaluated pair (hi, lo) of FP32 numbers, each addition split by Knuth's error-free two-sum
-// (s + e == hi + x exactly; plain FP32 additions, nothing the compiler may contract), on both lanes at
-// once with the packed instructions.  The pair holds about 48 significant bits; FP64 arithmetic is
-// slow on this GPU (a converted addition costs about a hundred FP32 ones), so the FP64 reductions add
-// only the sums of a few nodes, hi + lo, in FP64.
+// a + b (two lanes at once, with the packed instructions) or a - b; e: what its rounding left out, exactly
+// (Knuth's two-sum: plain FP32 additions, nothing the compiler may contract).
+template <bool kMinus = false>
+__device__ __forceinline__ float2 two_sum(float2 a, float2 b, float2 &e) {
+  const float2 minus = make_float2(-1.f, -1.f);
+  const float2 s = kMinus ? __ffma2_rn(minus, b, a) : __fadd2_rn(a, b);
+  const float2 part = __ffma2_rn(minus, a, s);  // of b, what reached s
+  const float2 ea = __ffma2_rn(minus, __ffma2_rn(minus, part, s), a);
+  e = kMinus ? __ffma2_rn(minus, __fadd2_rn(b, part), ea) : __fadd2_rn(ea, __ffma2_rn(minus, part, b));
+  return s;
+}
+__device__ __forceinline__ float two_sum(float a, float b, float &e) {
+  const float s = __fadd_rn(a, b), part = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, part)), __fsub_rn(b, part));
+  return s;
+}
+
+// Sums of FP32 values almost without rounding error, two lanes at once: each is kept as an unevaluated pair
+// (hi, lo) of FP32 numbers, about 48 significant bits.  FP64 arithmetic is slow on this GPU (a converted
+// addition costs about a hundred FP32 ones), so the FP64 reductions form the sums of a node this way.
 struct FloatPair2 {
   float2 hi{0.f, 0.f}, lo{0.f, 0.f};
-  // adds x, or (kMinus) subtracts it
-  template <bool kMinus = false>
   __device__ __forceinline__ void add(float2 x) {
-    const float2 minus = make_float2(-1.f, -1.f);
-    const float2 s = kMinus ? __ffma2_rn(minus, x, hi) : __fadd2_rn(hi, x);
-    const float2 part = __ffma2_rn(minus, hi, s);  // of x, what reached s
-    const float2 e = __ffma2_rn(minus, __ffma2_rn(minus, part, s), hi);
-    lo = __fadd2_rn(lo, kMinus ? __ffma2_rn(minus, __fadd2_rn(x, part), e)
-                               : __fadd2_rn(e, __ffma2_rn(minus, part, x)));
-    hi = s;
+    float2 e;
+    hi = two_sum(hi, x, e);
+    lo = __fadd2_rn(lo, e);
   }
-  __device__ __forceinline__ double a() const { return (double)hi.x + (double)lo.x; }
-  __device__ __forceinline__ double b() const { return (double)hi.y + (double)lo.y; }
+  // adds x, known to the error ex
+  __device__ __forceinline__ void add(float2 x, float2 ex) {
+    float2 e;
+    hi = two_sum(hi, x, e);
+    lo = __fadd2_rn(lo, __fadd2_rn(e, ex));
+  }
 };
 
-// The conserved sums [M_A, M_B, Px, Py, Pz] of the nodes a thread visits (over stored values:
-// streaming permutes populations, so they sum alike), in FP64 over groups of kNodes nodes: 340 packed
-// FP32 instructions and 8 FP64 ones per node.
+// Sums of FloatPair2 values: three FP32 parts each lane, the roundings of the first caught in the second and
+// those of the second in the third, about 72 significant bits.
+struct FloatTriple2 {
+  float2 hi{0.f, 0.f}, mid{0.f, 0.f}, lo{0.f, 0.f};
+  __device__ __forceinline__ void add(const FloatPair2 &x) {
+    float2 e, e1, e2;
+    hi = two_sum(hi, x.hi, e);
+    mid = two_sum(mid, x.lo, e1);
+    mid = two_sum(mid, e, e2);
+    lo = __fadd2_rn(lo, __fadd2_rn(e1, e2));
+  }
+  __device__ __forceinline__ double x() const { return (double)hi.x + ((double)mid.x + (double)lo.x); }
+  __device__ __forceinline__ double y() const { return (double)hi.y + ((double)mid.y + (double)lo.y); }
+};
+
+// The conserved sums [M_A, M_B, Px, Py, Pz] of the nodes a thread visits (over stored values: streaming
+// permutes populations, so they sum alike): each node's in pairs, groups of kNodes nodes in triples, which lose
+// nothing of them, and the groups in FP64.  The momenta come from the nine differences of opposite
+// directions, added over the components.  The totals of 256^3 with the call, FP32: 531 us; with four momentum
+// sums a component in place of the differences 591, with the nodes added in FP64 one by one 1037.  (Pairs
+// carried over the group held 48 bits of it, fewer than FP64's 53: 2.6e-7 off where momenta of 1e5 cancel
+// within groups, with the triples below 1e-8.)
 struct TotalSums {
   static constexpr int kNodes = 4;
   double acc[5] = {0, 0, 0, 0, 0};
-  FloatPair2 m, px, py, pz;
+  FloatTriple2 tm, txy, tz;  // (M_A, M_B), (Px, Py), and Pz in two parts
   int n = 0;
   // adds a node whose (A, B) pair of direction i is value(i)
   template <class F>
   __device__ __forceinline__ void add(F value) {
+    FloatPair2 m, pxy, pz;
+    m.add(value(0));
+    float d[9], e[9];  // directions 2 p + 1 and 2 p + 2 are opposite: x, y, z, then xy, xz, yz two each
 #pragma unroll
-    for (int i = 0; i < kQ; ++i) {
-      const float2 v = value(i);
+    for (int p = 0; p < 9; ++p) {
+      const float2 u = value(2 * p + 1), v = value(2 * p + 2);
+      m.add(u);
       m.add(v);
-      if (kCx[i] > 0) px.add(v);
-      if (kCx[i] < 0) px.add<true>(v);
-      if (kCy[i] > 0) py.add(v);
-      if (kCy[i] < 0) py.add<true>(v);
-      if (kCz[i] > 0) pz.add(v);
-      if (kCz[i] < 0) pz.add<true>(v);
+      float2 ed;
+      const float2 dp = two_sum<true>(u, v, ed);
+      d[p] = two_sum(dp.x, dp.y, e[p]);
+      e[p] += ed.x + ed.y;
     }
+    pxy.add(make_float2(d[0], d[1]), make_float2(e[0], e[1]));
+    pxy.add(make_float2(d[3], d[3]), make_float2(e[3], e[3]));
+    pxy.add(make_float2(d[4], -d[4]), make_float2(e[4], -e[4]));
+    pxy.add(make_float2(d[5], d[7]), make_float2(e[5], e[7]));
+    pxy.add(make_float2(d[6], d[8]), make_float2(e[6], e[8]));
+    pz.add(make_float2(d[2], d[5]), make_float2(e[2], e[5]));
+    pz.add(make_float2(-d[6], d[7]), make_float2(-e[6], e[7]));
+    pz.add(make_float2(-d[8], 0.f), make_float2(-e[8], 0.f));
+    tm.add(m);
+    txy.add(pxy);
+    tz.add(pz);
     if (++n == kNodes) flush();
   }
   __device__ __forceinline__ void flush() {
-    acc[0] += m.a();
-    acc[1] += m.b();
-    acc[2] += px.a() + px.b();
-    acc[3] += py.a() + py.b();
-    acc[4] += pz.a() + pz.b();
-    m = px = py = pz = FloatPair2{};
+    acc[0] += tm.x();
+    acc[1] += tm.y();
+    acc[2] += txy.x();
+    acc[3] += txy.y();
+    acc[4] += tz.x() + tz.y();
+    tm = txy = tz = FloatTriple2{};
     n = 0;
   }
 };
+static_assert(kCx[7] == 1 && kCy[7] == 1 && kCx[9] == 1 && kCy[9] == -1 && kCx[11] == 1 && kCz[11] == 1 &&
+                  kCx[13] == 1 && kCz[13] == -1 && kCy[15] == 1 && kCz[15] == 1 && kCy[17] == 1 && kCz[17] == -1,
+              "the diagonal pairs as TotalSums takes them");
 
 struct Coord {
   int x, y, z;
