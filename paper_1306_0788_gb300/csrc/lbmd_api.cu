@@ -37,7 +37,8 @@ struct StepGraph {
   };
   std::vector<Update> updates;
 };
-constexpr int kGraphUnavailable = 1;  // record_steps: take the steps one by one instead
+// What recording a graph returns where the steps can be taken without it: one by one, or by shorter graphs.
+constexpr int kGraphUnavailable = 1, kGraphShorter = 2;
 }  // namespace
 
 struct lbmd_ctx {
@@ -131,6 +132,7 @@ struct lbmd_ctx {
   cudaStream_t gst = nullptr;
   StepGraph graph[kGraphLevels][2][2];
   int64_t replayed = 0;  // steps replayed since the graphs were dropped
+  int graph_levels = kGraphLevels;  // lengths in use: those past it could not be recorded
   unsigned long long *step_base = nullptr;
   int64_t dev_step = -1;
   cudaEvent_t ph[2 * kShortGraph] = {};  // stand-ins for the timing events while recording
@@ -677,14 +679,16 @@ int one_step(lbmd_ctx *c, unsigned long long step, cudaEvent_t t0, cudaEvent_t t
   return LBMD_OK;
 }
 
+void drop_graph(StepGraph &g) {
+  if (g.exec) cudaGraphExecDestroy(g.exec);  // a launch in flight completes first
+  if (g.graph) cudaGraphDestroy(g.graph);
+  g = StepGraph{};
+}
+
 void drop_graphs(lbmd_ctx *c) {
   for (auto &level : c->graph)
     for (auto &row : level)
-      for (StepGraph &g : row) {
-        if (g.exec) cudaGraphExecDestroy(g.exec);  // a launch in flight completes first
-        if (g.graph) cudaGraphDestroy(g.graph);
-        g = StepGraph{};
-      }
+      for (StepGraph &g : row) drop_graph(g);
   c->replayed = 0;
 }
 
@@ -766,8 +770,10 @@ int record_steps(lbmd_ctx *c, StepGraph &g, int nsteps) {
     for (int q = 0; q < 2 * kShortGraph && ei == cudaSuccess && c->prof; ++q)
       if (!g.ev_node[q]) ei = cudaErrorInvalidValue;
   }
+  // what its launch would fail to allocate fails here
+  if (ei == cudaSuccess && nsteps > kShortGraph) ei = cudaGraphUpload(g.exec, c->st);
   if (ei != cudaSuccess) {
-    drop_graphs(c);
+    drop_graph(g);
     cudaGetLastError();
     return cuda_fail(c, ei, "graph instantiation");
   }
@@ -782,12 +788,13 @@ int record_steps(lbmd_ctx *c, StepGraph &g, int nsteps) {
 // The graph length for the next of n steps: the longest that fits and is recorded, or due for it.
 int graph_level(const lbmd_ctx *c, int n) {
   int level = 0;
-  for (int k = 1; k < kGraphLevels && !c->prof; ++k)
+  for (int k = 1; k < c->graph_levels && !c->prof; ++k)
     if (kGraphSteps[k] <= n && c->replayed >= kGraphAfter[k]) level = k;
   return level;
 }
 
-// kGraphSteps[level] steps by one launch of the graph recorded for the current buffers.
+// kGraphSteps[level] steps by one launch of the graph recorded for the current buffers; or none, and
+// kGraphShorter, where a longer graph cannot be recorded.
 int replay_steps(lbmd_ctx *c, int level) {
   StepGraph &g = c->graph[level][c->cur][c->pcur];
   const int nsteps = kGraphSteps[level];
@@ -795,7 +802,17 @@ int replay_steps(lbmd_ctx *c, int level) {
   if ((r = prepare_onepass(c))) return r;
   if (uses_onepass(c) && ((r = ensure_densities(c)) || (r = ensure_corner_j(c))))
     return r;  // before recording: not in the graph
-  if (!g.exec && (r = record_steps(c, g, nsteps))) return r;
+  if (!g.exec) {
+    const std::string msg = c->msg;
+    r = record_steps(c, g, nsteps);
+    if (level > 0 && r && r != kGraphUnavailable) {
+      // (no memory for it, say) the graphs in use go on; an error of the device shows at their launch
+      c->msg = msg;
+      c->graph_levels = level;
+      return kGraphShorter;
+    }
+    if (r) return r;
+  }
   if (c->dev_step != c->steps) {  // steps were taken without the graph since it last ran
     launch_set_step(c->step_base, (unsigned long long)c->steps, c->st);
     if ((r = launched(c, "step counter"))) return r;
@@ -1137,10 +1154,10 @@ int lbmd_step(lbmd_ctx *c, int nsteps) {
     if (c->graphs)
       while (s + kShortGraph <= n) {
         const int level = graph_level(c, n - s);
-        if ((r = replay_steps(c, level))) {
-          if (r != kGraphUnavailable) return r;
-          break;
-        }
+        r = replay_steps(c, level);
+        if (r == kGraphShorter) continue;
+        if (r == kGraphUnavailable) break;
+        if (r) return r;
         s += kGraphSteps[level];
       }
     if (s < n) {
@@ -1167,6 +1184,7 @@ int lbmd_set_graphs(lbmd_ctx *c, int on) {
   cudaSetDevice(c->dev);
   drop_graphs(c);
   c->graphs = on != 0;
+  c->graph_levels = kGraphLevels;
   return LBMD_OK;
 }
 
