@@ -613,7 +613,9 @@ size_t lattice_bytes(const StepParams &P, size_t elem) {
 
 size_t particle_bytes(const StepParams &P, int np_max) {
   if (np_max <= 0) return 0;
-  return (size_t)np_max * kParticleBytes * 5 / 4 + ((size_t)P.nrows + 1) * 3 * 4;  // 25 % capacity slack; rows
+  size_t b = (size_t)np_max * kParticleBytes * 5 / 4 + ((size_t)P.nrows + 1) * 3 * 4;  // 25 % capacity slack; rows
+  if (P.storage == LBMD_STORAGE_FP32) b += 2 * (size_t)P.nrows * node_words(P.nx) * 4 * 5 / 4;  // node bits
+  return b;
 }
 
 constexpr int kMixBGK = 1, kMixMRT = 2, kMixParticles = 4;
