@@ -246,6 +246,9 @@ int ensure_records(lbmd_ctx *c, long long n) {
   }
   if (e == cudaSuccess) e = alloc_sort_entries(c->rec_sort, (size_t)n);
   if (e == cudaSuccess) e = dalloc(&c->rec_row_start, (size_t)c->P.nrows + 1);
+  // the first step clears the nodes of the cells here (with more particles than before, lbmd_set_particles
+  // has cleared all): cells of the lattice, whatever it holds
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->rec[1].cell, 0, sizeof(int4) * (size_t)n, c->st);
   if (e != cudaSuccess) {
     cudaGetLastError();
     free_records(c);
@@ -543,7 +546,7 @@ int substep_particles(lbmd_ctx *c, ParticleArrays &pa, ParticleForces &pf, CellI
     // (pair reach: particles may have left their row by one cell)
     launch_substep(Q, from, to, S, rows, P.reach > 0 ? P.reach + 1 : 0, c->rho_buf[c->cur], c->jp,
                    c->nbonds ? c->bond_start : nullptr, c->bond_other, c->slot_of_id, c->pf, sub, c->rec[0], rs,
-                   c->node_bits[0], c->err, c->st);
+                   c->rec[1].cell, c->node_bits[0], c->err, c->st);
     if ((r = launched(c, "particle substep"))) return r;
   }
   // sort the (binned) records by (row, x cell, substep * np + id): the same counting sort as particles

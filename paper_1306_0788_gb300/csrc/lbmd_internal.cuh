@@ -372,11 +372,12 @@ void launch_particle_momentum(const StepParams &P, const ParticleArrays &pa, dou
                               cudaStream_t st);
 // MD sub-stepping: one particle substep (coupling and pair forces at C, the substep's reaction
 // records, binned in rs for their sort, and the update into D); S, ci: the step's sorted particles.
-// The first substep clears node_bits, which launch_rec_place sets.
+// Each clears in node_bits its share of the cells `marked` (substeps x particles: those of the last step's
+// records, whose nodes are the set ones); launch_rec_place then sets the new ones.
 void launch_substep(const StepParams &P, const ParticleArrays &C, const ParticleArrays &D, const ParticleArrays &S,
                     CellIndex ci, int pair_reach, const float *rho, const float *jp, const int *bond_start,
                     const int *bond_other, const int *slot_of_id, const ParticleForces &pf, int sub,
-                    const ReactionRecords &rec, const SortScratch &rs, unsigned *node_bits, unsigned *err,
-                    cudaStream_t st);
+                    const ReactionRecords &rec, const SortScratch &rs, const int4 *marked, unsigned *node_bits,
+                    unsigned *err, cudaStream_t st);
 
 }  // namespace lbmd
