@@ -1,6 +1,7 @@
-"""A longer step graph that cannot be recorded (no memory for it, say) is done without: the run goes on with
-the shorter ones, with the same bits and no error.  The failure comes from a build of the library in which
-cudaGraphInstantiate refuses graphs of more than a given number of nodes."""
+"""What is only faster is done without where the device has no room for it: a longer step graph that cannot
+be recorded (the shorter ones go on, with the same bits), the partial sums of the one-pass update (two
+passes).  The failures come from a build of the library in which cudaGraphInstantiate refuses graphs of more
+than a given number of nodes and cudaMalloc, while the environment says so, every allocation."""
 import os
 import shutil
 import subprocess
@@ -21,7 +22,11 @@ static inline cudaError_t refuse_long(cudaGraphExec_t *x, cudaGraph_t g, unsigne
   const char *most = std::getenv("MOST_GRAPH_NODES");
   return most && n > (size_t)std::atol(most) ? cudaErrorMemoryAllocation : cudaGraphInstantiate(x, g, flags);
 }
+static inline cudaError_t refuse_malloc(void **p, size_t n) {
+  return cudaMalloc(p, std::getenv("REFUSE_MALLOC") ? (size_t)1 << 60 : n);  // (as no memory: the last error is set)
+}
 #define cudaGraphInstantiate refuse_long
+#define cudaMalloc refuse_malloc
 """
 
 CHILD = r"""
@@ -48,7 +53,7 @@ print(L.lbmd_step_count(ctx), L.lbmd_last_error(ctx) or "-",
 
 @pytest.fixture(scope="module")
 def refusing(tmp_path_factory):
-    """A copy of the package whose library refuses long graphs."""
+    """A copy of the package with that library."""
     from paper_1306_0788_gb300 import build
     build.build()
     top = tmp_path_factory.mktemp("refusing")
@@ -69,20 +74,57 @@ def refusing(tmp_path_factory):
     return str(top)
 
 
-def _run(path, particles, steps, most=None):
-    env = dict(os.environ, PYTHONPATH=path)
-    if most:
-        env["MOST_GRAPH_NODES"] = str(most)
-    r = subprocess.run([sys.executable, "-c", CHILD, str(particles), steps], env=env, cwd=path, capture_output=True,
-                       text=True, timeout=300)
+def _child(path, code, *args, **env):
+    r = subprocess.run([sys.executable, "-c", code, *args], env=dict(os.environ, PYTHONPATH=path, **env), cwd=path,
+                       capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr
     return r.stdout.split()
+
+
+def _run(path, particles, steps, **env):
+    return _child(path, CHILD, str(particles), steps, **env)
 
 
 # fluid alone: 3, 9 and 33 nodes in graphs of 2, 8 and 32 steps; with particles 11, 41 and 161
 @pytest.mark.parametrize("particles,steps,most", [(0, "200,31", 5), (0, "4300,64", 20), (50, "170,20", 20),
                                                   (50, "4200,7", 100)])
 def test_run_goes_on_with_shorter_graphs(refusing, particles, steps, most):
-    got = _run(refusing, particles, steps, most)
+    got = _run(refusing, particles, steps, MOST_GRAPH_NODES=str(most))
     assert got == _run(ROOT, particles, steps)
     assert got[0] == str(sum(int(n) for n in steps.split(",")))
+
+
+NO_ROOM = r"""
+import os
+import numpy as np
+from paper_1306_0788_gb300 import lbmd as L
+rng = np.random.default_rng(1)
+dims = (160, 160, 160)
+rho = [rng.uniform(0.95, 1.05, dims[::-1]).astype(np.float32) for _ in range(2)]
+mrt = dict(g_AB=0.8, kT=1e-5, collision=L.LBMD_COLLISION_MRT)
+
+def steps(ctx, n):
+    L.lbmd_init_fluid(ctx, *rho)
+    L.lbmd_step(ctx, n)
+    return [L.lbmd_get_populations(ctx, k, dims[::-1]) for k in range(2)]
+
+ctx, _ = L.lbmd_create(L.params(dims, **mrt))
+L.lbmd_set_graphs(ctx, False)
+L.lbmd_init_fluid(ctx, *rho)
+os.environ["REFUSE_MALLOC"] = "1"
+assert L.lbmd_get_lattice_passes(ctx) == 2
+without = steps(ctx, 3)
+del os.environ["REFUSE_MALLOC"]
+assert L.lbmd_get_lattice_passes(ctx) == 2
+L.lbmd_set_lattice_passes(ctx, 2)
+assert all(np.array_equal(a, b) for a, b in zip(without, steps(ctx, 3)))
+L.lbmd_set_lattice_passes(ctx, 0)
+assert L.lbmd_get_lattice_passes(ctx) == 1
+steps(ctx, 3)
+L.lbmd_sync(ctx)
+print("done")
+"""
+
+
+def test_two_passes_where_there_is_no_room_for_the_partial_sums(refusing):
+    assert _child(refusing, NO_ROOM) == ["done"]
