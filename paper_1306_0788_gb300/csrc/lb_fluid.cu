@@ -532,7 +532,8 @@ __global__ void __launch_bounds__(kBlock) k_boundary_densities(StepParams P, One
   const float2 *ze2 = reinterpret_cast<const float2 *>(out.zedge);
   float2 *rho2 = reinterpret_cast<float2 *>(rho_next);
   const unsigned nx = (unsigned)P.nx, ny = (unsigned)P.ny, ntx = (unsigned)G.ntx, nty = (unsigned)G.nty;
-  // 32-bit index arithmetic: nodes and partial sums are fewer than 2^32 / 19
+  // 32-bit index arithmetic: 19 N < 2^32.  The longest array, the y-edge sums padded to whole tiles along x, has
+  // 2 nz nty 32 ntx entries, with at least 2 columns and 3 rows (ypart) at most 32 / 3 of N
   if (bid < D.edge) {
     const unsigned t = bid * kBlock + threadIdx.x;
     if (t >= (unsigned)P.nz * ny * ntx) return;

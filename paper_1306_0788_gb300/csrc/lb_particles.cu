@@ -19,7 +19,8 @@ inline unsigned pgrid(long long n) { return (unsigned)((n + kPBlock - 1) / kPBlo
 //   bin      the row of each particle, its rank of arrival in the row (the histogram's counter
 //            before it), and the histogram summed over the kScanRows rows of each scan block
 //   scan     rows -> first sorted slot: a block scans its rows from the sum of the block totals
-//            before it (one launch; the totals are few), and clears the counters for the next sort
+//            before it (one launch; a total for 2048 rows), and clears the counters for the next sort:
+//            21 us for 2 M rows, 547 for 67 M (a lattice of one column), beside updates of 186 and 3033
 //   scatter  each particle's sort key to a slot of its row, in arrival order
 //   place    a particle's slot in its row is the number of smaller keys there; it moves
 // The keys of a row are distinct, so the order, and every gather after it, is deterministic

@@ -945,7 +945,7 @@ __device__ __forceinline__ void collide_core(const StepParams &P, long long s, u
 template <class T, bool kMRT = false, bool kWrite = true, bool kKeep = false>
 __device__ __forceinline__ void store_node(const StepParams &P, unsigned s32, T *__restrict__ fout,
                                            float *__restrict__ rest_out, float (&fA)[kQ], float (&fB)[kQ],
-                                           float rA, float rB, bool write = true) {
+                                           float rA, float rB) {
   static_assert(!(kMRT && kKeep && kSplitRest<T>), "with MRT the stored values are kept in FP32 only");
   const unsigned N32 = (unsigned)P.N;
   constexpr bool kShifted = kSplitRest<T> && !kMRT;
@@ -959,7 +959,7 @@ __device__ __forceinline__ void store_node(const StepParams &P, unsigned s32, T 
 #pragma unroll
         for (int i = 1; i < kQ; ++i) {
           const unsigned w = Pair16<T>::enc(make_float2(fA[i], fB[i]));
-          if (kWrite && write) wout[(size_t)i * N32] = w;
+          if (kWrite) wout[(size_t)i * N32] = w;
           const float2 d = Pair16<T>::dec(w);
           m = __ffma2_rn(make_float2(-1.f, -1.f), d, m);
           fA[i] = d.x;
@@ -972,12 +972,12 @@ __device__ __forceinline__ void store_node(const StepParams &P, unsigned s32, T 
 #pragma unroll
         for (int i = 1; i < kQ; ++i) {
           const unsigned w = Pair16<T>::enc(make_float2(fA[i], fB[i]));
-          if (kWrite && write) wout[(size_t)i * N32] = w;
+          if (kWrite) wout[(size_t)i * N32] = w;
           Pair16<T>::add_to(w, nm);
         }
         m = make_float2(-nm.x, -nm.y);
       }
-      if (kWrite && write && rest_out) {
+      if (kWrite && rest_out) {
         rest_out[s32] = m.x;
         rest_out[N32 + s32] = m.y;
       }
@@ -1004,9 +1004,8 @@ __device__ __forceinline__ void store_node(const StepParams &P, unsigned s32, T 
     }
   } else if (kWrite) {
     float2 *fout2 = reinterpret_cast<float2 *>(fout) + s32;  // direction i at fout2[i N]
-    if (write)
 #pragma unroll
-      for (int i = 0; i < kQ; ++i) fout2[(size_t)i * N32] = make_float2(fA[i], fB[i]);
+    for (int i = 0; i < kQ; ++i) fout2[(size_t)i * N32] = make_float2(fA[i], fB[i]);
   }
 }
 

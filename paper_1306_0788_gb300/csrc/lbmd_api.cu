@@ -17,7 +17,9 @@ namespace {
 // particles 702 us with graphs of two steps, 579 of ten, 556 of fifty; of 45x37x29 fluid only 468,
 // 356, 337; of 64^3 with 1000 particles 1273, 1122, 1092.  Recording takes 6 us per step of fluid
 // alone and about 35 with particles (0.2 and 1.3 ms for 32 steps), so the longer graphs are recorded
-// once a context has replayed as many steps as make up for it.
+// once a context has replayed as many steps as make up for it with particles: 8 steps save about 2.2 us a
+// step, 280 us in 128 steps, 32 steps 0.4, 1.5 ms in 4096.  (Fluid alone would make up for it in about 22 and
+// 500 steps.)
 constexpr int kGraphLevels = 3;
 constexpr int kGraphSteps[kGraphLevels] = {2, 8, 32};
 constexpr int64_t kGraphAfter[kGraphLevels] = {0, 128, 4096};  // steps replayed since the last setter
@@ -404,6 +406,8 @@ int setup_onepass(lbmd_ctx *c) {
     CK(dalloc(&c->op_zslot, zslot.size()), "plane table");
     CK(cudaMemcpy(c->op_zslot, zslot.data(), sizeof(int) * zslot.size(), cudaMemcpyHostToDevice), "plane table");
   }
+  // the kernels index the sums in 32 bits: at most 32 / 3 N entries here, with N < 2^32 / 19
+  static_assert(kOnePassCols <= 3 * kQ, "2 nz nty ntx kOnePassCols < 2^32 for nx >= 2, ny >= 3");
   if (ypart) {
     CK(dalloc(&c->op_out.yedge, (size_t)2 * P.nz * nty * ntx * kOnePassCols * 2), "edge sums");
     CK(dalloc(&c->op_out.diag, (size_t)P.nz * nty * ntx * 4 * 2), "edge sums");

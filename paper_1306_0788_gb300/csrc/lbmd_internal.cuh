@@ -289,7 +289,7 @@ void launch_collide(const StepParams &P, const void *fin, void *fout, const floa
 // not be the same buffer: blocks read the rest populations of nodes that others update.
 void launch_step_small(const StepParams &P, const void *fin, void *fout, const float *rest_in, float *rest_out,
                        unsigned *err, cudaStream_t st);
-// One-pass update (BGK, md_substeps = 1): writes the populations of the next step, the densities
+// One-pass update (BGK, or MRT with FP32 storage; md_substeps = 1): writes the populations of the next step, the densities
 // rho_next of the nodes whose sources are all in one block, and the partial sums of `out` for the
 // others; launch_boundary_densities then finishes those.
 void launch_collide_onepass(const StepParams &P, const void *fin, void *fout, const float *rest_in, float *rest_out,
@@ -301,7 +301,7 @@ void launch_collide_onepass(const StepParams &P, const void *fin, void *fout, co
 void launch_boundary_densities(const StepParams &P, OnePassGeom G, const void *store, const float *rest,
                                float *rho_next, const BoundaryRun *runs, int nruns, OnePassOut out,
                                const int *zslot, cudaStream_t st);
-// Blocks of the one-pass update resident on one SM (its persistent grid is this times the SMs).
+// Blocks of the one-pass update resident on one SM (its grid: a block for each tile of each chunk).
 int onepass_blocks_per_sm();
 void launch_fields(const StepParams &P, const void *store, const float *rest, const float *rho, float *rhoA,
                    float *rhoB, float *u, cudaStream_t st);
