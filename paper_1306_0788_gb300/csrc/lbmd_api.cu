@@ -348,6 +348,19 @@ bool uses_one_launch(const lbmd_ctx *c) {
   return small_lattice(c->P) && c->np == 0 && c->passes == 0 && !uses_onepass(c);
 }
 
+void drop_graph(StepGraph &g) {
+  if (g.exec) cudaGraphExecDestroy(g.exec);  // a launch in flight completes first
+  if (g.graph) cudaGraphDestroy(g.graph);
+  g = StepGraph{};
+}
+
+void drop_graphs(lbmd_ctx *c) {
+  for (auto &level : c->graph)
+    for (auto &row : level)
+      for (StepGraph &g : row) drop_graph(g);
+  c->replayed = 0;
+}
+
 // Frees what prepare_onepass set up.
 void free_onepass(lbmd_ctx *c) {
   dfree(c->op_runs);
@@ -423,6 +436,17 @@ int setup_onepass(lbmd_ctx *c) {
   c->op_geom = OnePassGeom{ntx, nty, nchunks, ypart, zpart};
   c->op_grid = grid;
   return LBMD_OK;
+}
+
+// Gives the one-pass update's partial sums back where the automatic choice took them, for another allocation
+// that finds no room: two passes from the next step on.  Whether there were any.
+bool release_onepass(lbmd_ctx *c) {
+  if (c->passes != 0 || c->op_grid == 0) return false;
+  drop_graphs(c);
+  free_onepass(c);
+  c->onepass_no_room = true;
+  c->jc_valid = false;
+  return true;
 }
 
 // setup_onepass once per context, where the next step takes one pass.  Allocates: call it before any
@@ -684,19 +708,6 @@ int one_step(lbmd_ctx *c, unsigned long long step, cudaEvent_t t0, cudaEvent_t t
   c->rho_valid = onepass;  // the two-pass update leaves the new state's densities to its next step
   c->jc_valid = corner_j;
   return LBMD_OK;
-}
-
-void drop_graph(StepGraph &g) {
-  if (g.exec) cudaGraphExecDestroy(g.exec);  // a launch in flight completes first
-  if (g.graph) cudaGraphDestroy(g.graph);
-  g = StepGraph{};
-}
-
-void drop_graphs(lbmd_ctx *c) {
-  for (auto &level : c->graph)
-    for (auto &row : level)
-      for (StepGraph &g : row) drop_graph(g);
-  c->replayed = 0;
 }
 
 // Records nsteps steps from the current buffers into g: on the private stream gst, with
@@ -1037,24 +1048,37 @@ int lbmd_set_particles(lbmd_ctx *c, int n, const double *x, const double *v, con
     const int r = convert_particles(P, n, x, v, type, q, hc, hf, hv, hid, why);
     if (r) return fail(c, r, why);
   }
-  if (n > c->cap) {
-    free_particles(c);
-    cudaError_t e = cudaSuccess;
-    for (ParticleArrays *a : {&c->pa[0], &c->pa[1], &c->pt}) {
-      if (e != cudaSuccess || (e = dalloc(&a->cell, n)) != cudaSuccess ||
-          (e = dalloc(&a->frac, n)) != cudaSuccess || (e = dalloc(&a->vel, n)) != cudaSuccess)
-        break;
-      e = dalloc(&a->pid, n);
+  // an allocation, again without the one-pass update's partial sums if there is no room beside them
+  auto with_room = [c](auto alloc) {
+    cudaError_t e = alloc();
+    if (e == cudaErrorMemoryAllocation && release_onepass(c)) {
+      cudaGetLastError();
+      e = alloc();
     }
-    if (e == cudaSuccess) e = dalloc(&c->pf.fric, n);
-    if (e == cudaSuccess) e = dalloc(&c->pf.psA, n);
-    if (e == cudaSuccess) e = dalloc(&c->pf.psB, n);
-    if (e == cudaSuccess) e = dalloc(&c->pf.fsr, n);
-    if (e == cudaSuccess) e = dalloc(&c->pf.pair, n);
-    if (e == cudaSuccess) e = dalloc(&c->pf.total, n);
-    if (e == cudaSuccess) e = dalloc(&c->slot_of_id, n);
-    if (e == cudaSuccess) e = alloc_sort_entries(c->sort, (size_t)n);
-    if (e == cudaSuccess) e = dalloc(&c->jc, (size_t)n * 8);
+    return e;
+  };
+  if (n > c->cap) {
+    auto alloc = [c, n] {
+      free_particles(c);
+      cudaError_t e = cudaSuccess;
+      for (ParticleArrays *a : {&c->pa[0], &c->pa[1], &c->pt}) {
+        if (e != cudaSuccess || (e = dalloc(&a->cell, n)) != cudaSuccess ||
+            (e = dalloc(&a->frac, n)) != cudaSuccess || (e = dalloc(&a->vel, n)) != cudaSuccess)
+          break;
+        e = dalloc(&a->pid, n);
+      }
+      if (e == cudaSuccess) e = dalloc(&c->pf.fric, n);
+      if (e == cudaSuccess) e = dalloc(&c->pf.psA, n);
+      if (e == cudaSuccess) e = dalloc(&c->pf.psB, n);
+      if (e == cudaSuccess) e = dalloc(&c->pf.fsr, n);
+      if (e == cudaSuccess) e = dalloc(&c->pf.pair, n);
+      if (e == cudaSuccess) e = dalloc(&c->pf.total, n);
+      if (e == cudaSuccess) e = dalloc(&c->slot_of_id, n);
+      if (e == cudaSuccess) e = alloc_sort_entries(c->sort, (size_t)n);
+      if (e == cudaSuccess) e = dalloc(&c->jc, (size_t)n * 8);
+      return e;
+    };
+    const cudaError_t e = with_room(alloc);
     if (e != cudaSuccess) {
       cudaGetLastError();
       free_particles(c);
@@ -1066,13 +1090,17 @@ int lbmd_set_particles(lbmd_ctx *c, int n, const double *x, const double *v, con
   }
   if (!c->sort.row_count) {  // rows are needed by the lattice kernels' gather even without particles
     const size_t nb = (size_t)scan_blocks(P.nrows);
-    for (int *&start : c->row_start)
-      if (!start) CK(dalloc(&start, (size_t)P.nrows + 1), "alloc rows");
-    for (unsigned *&bits : c->node_bits)
-      if (!bits) CK(dalloc(&bits, node_words(P.nx) * (size_t)P.nrows), "alloc rows");
-    if (!c->sort.block_count) CK(dalloc(&c->sort.block_count, nb), "alloc rows");
+    auto alloc = [c, &P, nb] {
+      cudaError_t e = cudaSuccess;
+      for (int *&start : c->row_start)
+        if (e == cudaSuccess && !start) e = dalloc(&start, (size_t)P.nrows + 1);
+      for (unsigned *&bits : c->node_bits)
+        if (e == cudaSuccess && !bits) e = dalloc(&bits, node_words(P.nx) * (size_t)P.nrows);
+      if (e == cudaSuccess && !c->sort.block_count) e = dalloc(&c->sort.block_count, nb);
+      return e == cudaSuccess ? dalloc(&c->sort.row_count, (size_t)P.nrows) : e;
+    };
+    CK(with_room(alloc), "alloc rows");
     CK(cudaMemsetAsync(c->sort.block_count, 0, sizeof(int) * nb, c->st), "clear rows");
-    CK(dalloc(&c->sort.row_count, (size_t)P.nrows), "alloc rows");
     CK(cudaMemsetAsync(c->sort.row_count, 0, sizeof(int) * (size_t)P.nrows, c->st), "clear rows");
   }
   c->np = n;

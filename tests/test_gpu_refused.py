@@ -1,7 +1,8 @@
 """What is only faster is done without where the device has no room for it: a longer step graph that cannot
 be recorded (the shorter ones go on, with the same bits), the partial sums of the one-pass update (two
-passes).  The failures come from a build of the library in which cudaGraphInstantiate refuses graphs of more
-than a given number of nodes and cudaMalloc, while the environment says so, every allocation."""
+passes), also where particles find no room beside them later.  The failures come from a build of the library in
+which cudaGraphInstantiate refuses graphs of more than a given number of nodes and cudaMalloc, while the
+environment says so, every allocation or those past a number of bytes in all."""
 import os
 import shutil
 import subprocess
@@ -16,17 +17,32 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 REFUSE = r"""
 #include <cuda_runtime.h>
 #include <cstdlib>
+#include <map>
 static inline cudaError_t refuse_long(cudaGraphExec_t *x, cudaGraph_t g, unsigned long long flags) {
   size_t n = 0;
   cudaGraphGetNodes(g, nullptr, &n);
   const char *most = std::getenv("MOST_GRAPH_NODES");
   return most && n > (size_t)std::atol(most) ? cudaErrorMemoryAllocation : cudaGraphInstantiate(x, g, flags);
 }
+static std::map<void *, size_t> held;
+static size_t total = 0;
+extern "C" size_t bytes_held() { return total; }
 static inline cudaError_t refuse_malloc(void **p, size_t n) {
-  return cudaMalloc(p, std::getenv("REFUSE_MALLOC") ? (size_t)1 << 60 : n);  // (as no memory: the last error is set)
+  const char *most = std::getenv("MOST_BYTES");
+  if (std::getenv("REFUSE_MALLOC") || (most && total + n > (size_t)std::atoll(most)))
+    return cudaMalloc(p, (size_t)1 << 60);  // as no memory: the last error is set
+  const cudaError_t e = cudaMalloc(p, n);
+  if (e == cudaSuccess) total += held[*p] = n;
+  return e;
+}
+static inline cudaError_t counted_free(void *p) {
+  total -= held[p];
+  held.erase(p);
+  return cudaFree(p);
 }
 #define cudaGraphInstantiate refuse_long
 #define cudaMalloc refuse_malloc
+#define cudaFree counted_free
 """
 
 CHILD = r"""
@@ -128,3 +144,53 @@ print("done")
 
 def test_two_passes_where_there_is_no_room_for_the_partial_sums(refusing):
     assert _child(refusing, NO_ROOM) == ["done"]
+
+
+NO_ROOM_BESIDE = r"""
+import ctypes, os
+import numpy as np
+from paper_1306_0788_gb300 import lbmd as L
+held = L._lib.bytes_held
+held.restype = ctypes.c_size_t
+rng = np.random.default_rng(1)
+dims, n = (160, 160, 160), 20000
+rho = [rng.uniform(0.95, 1.05, dims[::-1]).astype(np.float32) for _ in range(2)]
+x = rng.uniform(0, 160, (n, 3))
+
+def context():
+    ctx, _ = L.lbmd_create(L.params(dims, g_AB=0.8, kT=1e-5, collision=L.LBMD_COLLISION_MRT))
+    L.lbmd_set_types(ctx, [L.lbmd_ptype(0.0, 0.0, 0.0, 0.0, 0.1, 200.0)])
+    L.lbmd_init_fluid(ctx, *rho)
+    return ctx
+
+def with_particles(ctx):
+    before = held()
+    L.lbmd_set_particles(ctx, x, np.zeros_like(x), np.zeros(n, dtype=np.int32))
+    return held() - before
+
+def steps(ctx):
+    L.lbmd_init_fluid(ctx, *rho)
+    L.lbmd_step(ctx, 3)
+    return [L.lbmd_get_populations(ctx, k, dims[::-1]) for k in range(2)] + list(L.lbmd_get_particles(ctx, n))
+
+two = context()
+L.lbmd_set_lattice_passes(two, 2)
+size = with_particles(two)
+want = steps(two)
+L.lbmd_destroy(two)
+for short in (1, size // 2, size):  # rows, then particle arrays, find no room
+    ctx = context()
+    L.lbmd_step(ctx, 2)
+    assert L.lbmd_get_lattice_passes(ctx) == 1
+    os.environ["MOST_BYTES"] = str(held() + size - short)
+    with_particles(ctx)
+    del os.environ["MOST_BYTES"]
+    assert L.lbmd_get_lattice_passes(ctx) == 2
+    assert all(np.array_equal(a, b) for a, b in zip(want, steps(ctx)))
+    L.lbmd_destroy(ctx)
+print("done")
+"""
+
+
+def test_particles_take_the_room_of_the_partial_sums(refusing):
+    assert _child(refusing, NO_ROOM_BESIDE) == ["done"]
