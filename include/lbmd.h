@@ -198,7 +198,7 @@ int lbmd_step(lbmd_ctx *ctx, int nsteps);
  * two coupled steps, recorded at the first such call for the current buffers on a private
  * stream and launched into the context stream; an odd last step is launched directly.  After 128
  * steps since the last setter, eight at a time where a call asks for as many, after 4096, 32; where
- * a longer graph cannot be recorded (no memory for it, say), the shorter ones go on.  The
+ * there is no memory for a longer graph, the shorter ones go on.  The
  * results are bit-identical to on = 0, where every kernel is launched one by one; the graph
  * saves the launch latency that dominates small lattices.  The particle kernels read their noise
  * counter from a device-resident step base; the fluctuating MRT update gets its counter written

@@ -788,8 +788,6 @@ int record_steps(lbmd_ctx *c, StepGraph &g, int nsteps) {
     for (int q = 0; q < 2 * kShortGraph && ei == cudaSuccess && c->prof; ++q)
       if (!g.ev_node[q]) ei = cudaErrorInvalidValue;
   }
-  // what its launch would fail to allocate fails here
-  if (ei == cudaSuccess && nsteps > kShortGraph) ei = cudaGraphUpload(g.exec, c->st);
   if (ei != cudaSuccess) {
     drop_graph(g);
     cudaGetLastError();
@@ -812,7 +810,7 @@ int graph_level(const lbmd_ctx *c, int n) {
 }
 
 // kGraphSteps[level] steps by one launch of the graph recorded for the current buffers; or none, and
-// kGraphShorter, where a longer graph cannot be recorded.
+// kGraphShorter, where a longer graph cannot be recorded or finds no memory.
 int replay_steps(lbmd_ctx *c, int level) {
   StepGraph &g = c->graph[level][c->cur][c->pcur];
   const int nsteps = kGraphSteps[level];
@@ -842,7 +840,16 @@ int replay_steps(lbmd_ctx *c, int level) {
   }
   for (const StepGraph::Update &u : g.updates)
     CK(set_update_step(g.exec, u.node, (unsigned long long)c->steps + u.off), "update counter");
-  CK(cudaGraphLaunch(g.exec, c->st), "graph launch");
+  // (the first launch of a graph allocates; uploading it when it is recorded made every later launch whose
+  // counters are patched 3 us slower)
+  const cudaError_t launch = cudaGraphLaunch(g.exec, c->st);
+  if (launch == cudaErrorMemoryAllocation && level > 0) {
+    cudaGetLastError();
+    drop_graph(g);
+    c->graph_levels = level;
+    return kGraphShorter;
+  }
+  CK(launch, "graph launch");
   if (c->prof) c->ev_used += 2 * kShortGraph;
   c->launches += g.launches;
   c->steps += nsteps;

@@ -1,7 +1,7 @@
 """What is only faster is done without where the device has no room for it: a longer step graph that cannot
 be recorded (the shorter ones go on, with the same bits), the partial sums of the one-pass update (two
 passes), also where particles find no room beside them later.  The failures come from a build of the library in
-which cudaGraphInstantiate refuses graphs of more than a given number of nodes and cudaMalloc, while the
+which cudaGraphInstantiate or cudaGraphLaunch refuses graphs of more than a given number of nodes and cudaMalloc, while the
 environment says so, every allocation or those past a number of bytes in all."""
 import os
 import shutil
@@ -18,11 +18,19 @@ REFUSE = r"""
 #include <cuda_runtime.h>
 #include <cstdlib>
 #include <map>
+static std::map<cudaGraphExec_t, size_t> nodes;
 static inline cudaError_t refuse_long(cudaGraphExec_t *x, cudaGraph_t g, unsigned long long flags) {
   size_t n = 0;
   cudaGraphGetNodes(g, nullptr, &n);
   const char *most = std::getenv("MOST_GRAPH_NODES");
-  return most && n > (size_t)std::atol(most) ? cudaErrorMemoryAllocation : cudaGraphInstantiate(x, g, flags);
+  if (most && n > (size_t)std::atol(most)) return cudaErrorMemoryAllocation;
+  const cudaError_t e = cudaGraphInstantiate(x, g, flags);
+  if (e == cudaSuccess) nodes[*x] = n;
+  return e;
+}
+static inline cudaError_t refuse_launch(cudaGraphExec_t x, cudaStream_t st) {
+  const char *most = std::getenv("MOST_LAUNCHED_NODES");
+  return most && nodes[x] > (size_t)std::atol(most) ? cudaErrorMemoryAllocation : cudaGraphLaunch(x, st);
 }
 static std::map<void *, size_t> held;
 static size_t total = 0;
@@ -41,6 +49,7 @@ static inline cudaError_t counted_free(void *p) {
   return cudaFree(p);
 }
 #define cudaGraphInstantiate refuse_long
+#define cudaGraphLaunch refuse_launch
 #define cudaMalloc refuse_malloc
 #define cudaFree counted_free
 """
@@ -104,8 +113,9 @@ def _run(path, particles, steps, **env):
 # fluid alone: 3, 9 and 33 nodes in graphs of 2, 8 and 32 steps; with particles 11, 41 and 161
 @pytest.mark.parametrize("particles,steps,most", [(0, "200,31", 5), (0, "4300,64", 20), (50, "170,20", 20),
                                                   (50, "4200,7", 100)])
-def test_run_goes_on_with_shorter_graphs(refusing, particles, steps, most):
-    got = _run(refusing, particles, steps, MOST_GRAPH_NODES=str(most))
+@pytest.mark.parametrize("call", ["MOST_GRAPH_NODES", "MOST_LAUNCHED_NODES"])
+def test_run_goes_on_with_shorter_graphs(refusing, particles, steps, most, call):
+    got = _run(refusing, particles, steps, **{call: str(most)})
     assert got == _run(ROOT, particles, steps)
     assert got[0] == str(sum(int(n) for n in steps.split(",")))
 
