@@ -425,7 +425,7 @@ int lbmd_batch_get_drift(lbmd_batch *batch, int slot, double out[5]);
  * count]), and the register budget of the update, collide_blocks = 3 (80 registers, three
  * blocks of 256 threads per SM) or 2 (up to 128 registers).  cfg[5] = {tile_sites,
  * grid_moments, grid_collide, collide_blocks, grid_particles}.  Results do not depend on it.  Until it is
- * set or tuned, the tile size follows the number of sites whenever replicas join or leave. */
+ * set or tuned, tile size and update grid follow the number of sites whenever replicas join or leave. */
 int lbmd_batch_set_config(lbmd_batch *batch, int tile_sites, int grid_moments, int grid_collide,
                           int collide_blocks);
 int lbmd_batch_get_config(const lbmd_batch *batch, int cfg[5]);

@@ -655,14 +655,14 @@ struct lbmd_batch {
   double *d_drift = nullptr;  // [max_slots][10] (BatchDev::drift)
   size_t chunk_cap = 0;            // capacity of the drift check's sums (chunks)
   bool dirty = true;
-  // launch shape; until it is set or tuned, each repack chooses the tile size (default_tile)
+  // launch shape; until it is set or tuned, each repack chooses tile size and grid_collide (default_shape)
   bool shaped = false;
   int tile_sites = 1024, grid_moments = 0, grid_collide = 0, grid_particles = 0;
   int collide_blocks = 2;  // register budget of the update kernel: blocks per SM
   // what is among the replicas of the tables (kMix*): a step launches only the update's variants in
   // use, and the particle kernels only where there are particles
   int mix = 0;
-  std::map<int, cudaGraphExec_t> graphs;  // by steps per graph and mix: 8 n + mix
+  std::map<std::pair<int, int>, cudaGraphExec_t> graphs;  // by 8 n + mix (n steps) and grid_collide
   int64_t launches = 0;
   std::string msg;
 };
@@ -811,29 +811,38 @@ std::vector<int> active_slots(const lbmd_batch *b) {
 // The launch shape without tuning, from the step times of 40 sets of replicas (one of 16^3 to 24 of up to 128^3,
 // 4 k to 34 M sites, with and without particles), over tiles of 256 to 8192 sites and 2 or 3 blocks per SM,
 // resident or queued.  FP32: blocks of 128 registers, two per SM, sixteen queued, which even out what tiles
-// with more or fewer particles take; 16 bits, bound by instruction issue: three resident ones of 80.  The
-// tile is the largest, up to 2048 sites in FP32 and 1024 in 16 bits, that gives each resident block one:
-// larger ones leave blocks idle, smaller ones cost more tile contexts.  FP32, 14 sets of the serving
-// distribution (5 to 17 M sites with particles) against 1024 sites at three resident blocks, the
-// default before: 0.92 to 0.96 of its step time; 4096 sites at eight queued 0.91 to 0.99; 2048 and 1024 at two
-// resident 0.93 to 0.98 and 0.94 to 0.97.  Eight queued blocks for both storages with tiles of at most two a
-// block lost up to 27 % on sets of small replicas and 5 to 11 % in 16 bits.
-struct DefaultShape {
-  int tile_sites, collide_blocks, grid;  // most sites of a tile, blocks per SM resident, launched
+// with more or fewer particles take; 16 bits, bound by instruction issue: three of 80, resident, and sixteen
+// queued with larger tiles where there are enough of them.  The tile is the largest, up to 2048 sites in FP32
+// and 1024 in 16 bits, that gives each resident block one: larger ones leave blocks idle, smaller ones cost
+// more tile contexts.  FP32, 14 sets of the serving distribution (5 to 17 M sites with particles) against 1024
+// sites at three resident blocks, the default before: 0.92 to 0.96 of its step time; 4096 sites at eight
+// queued 0.91 to 0.99; 2048 and 1024 at two resident 0.93 to 0.98 and 0.94 to 0.97.  16 bits, the same sets:
+// 2048 sites at sixteen queued 0.92 to 1.03 (mean 0.97), 30 of 64^3 0.95, but 30 of 32^3 (480 tiles) 1.09 and
+// 40 of 24^3 1.29; 4096 sites from 10 M sites on 0.95 to 0.98, below 0.97 to 1.07.  Eight queued blocks for both storages with tiles of at most two a block lost up to 27 % on
+// sets of small replicas.
+constexpr int kQueuedTiles = 2000;
+struct Shape {
+  int tile_sites, grid;  // sites of a tile, blocks per SM launched
 };
-constexpr DefaultShape default_shape(int storage) {
-  return storage == LBMD_STORAGE_FP32 ? DefaultShape{2048, 2, 16} : DefaultShape{1024, 3, 3};
-}
+constexpr int default_collide_blocks(int storage) { return storage == LBMD_STORAGE_FP32 ? 2 : 3; }
 
-int default_tile(const lbmd_batch *b, const std::vector<int> &act) {
-  const DefaultShape D = default_shape(b->storage);
-  int ts = D.tile_sites;
-  for (; ts > kBThreads; ts /= 2) {
-    long long tiles = 0;
-    for (int s : act) tiles += (b->slots[s].P.N + ts - 1) / ts;
-    if (tiles >= (long long)D.collide_blocks * b->sms) break;
+Shape default_shape(const lbmd_batch *b, const std::vector<int> &act) {
+  auto tiles = [&](int ts) {
+    long long n = 0;
+    for (int s : act) n += (b->slots[s].P.N + ts - 1) / ts;
+    return n;
+  };
+  const int resident = default_collide_blocks(b->storage), queued = 16;
+  Shape S{2048, queued};
+  if (b->storage != LBMD_STORAGE_FP32) {
+    if (tiles(2048) < kQueuedTiles)
+      S = Shape{1024, resident};
+    else if (tiles(4096) >= (long long)queued * b->sms)
+      S.tile_sites = 4096;
   }
-  return ts;
+  while (S.tile_sites > kBThreads && tiles(S.tile_sites) < (long long)resident * b->sms)
+    S.tile_sites /= 2;
+  return S;
 }
 
 // Lay the tables out again after replicas joined or left or changed their particles: particle
@@ -972,7 +981,11 @@ int repack(lbmd_batch *b) {
   if (!rep_slot.empty())
     BK(cudaMemcpyAsync(b->d_rep_slot, rep_slot.data(), sizeof(int) * rep_slot.size(), cudaMemcpyHostToDevice, b->st),
        "upload replicas");
-  if (!b->shaped) b->tile_sites = default_tile(b, act);
+  if (!b->shaped) {
+    const Shape S = default_shape(b, act);
+    b->tile_sites = S.tile_sites;
+    b->grid_collide = S.grid * b->sms;
+  }
   int r = build_tiles(b, act);
   if (r) return r;
   b->mix = np > 0 ? kMixParticles : 0;
@@ -1090,10 +1103,10 @@ void drop_graphs(lbmd_batch *b) {
   b->graphs.clear();
 }
 
-// The graph of n steps for the current mix (captured once per n and mix);
+// The graph of n steps for the current mix and grid (captured once for each);
 // *launches receives its kernel launches.
 int graph_for(lbmd_batch *b, int n, cudaGraphExec_t *out, int *launches) {
-  const int key = 8 * n + b->mix;
+  const std::pair<int, int> key(8 * n + b->mix, b->grid_collide);
   auto it = b->graphs.find(key);
   *launches = n * step_launches(b);
   if (it != b->graphs.end()) {
@@ -1211,8 +1224,8 @@ int lbmd_batch_create(size_t mem_budget, int storage, int max_slots, void *strea
   b->max_slots = max_slots;
   b->slots.resize(max_slots);
   b->grid_moments = 4 * b->sms;
-  b->collide_blocks = default_shape(storage).collide_blocks;
-  b->grid_collide = default_shape(storage).grid * b->sms;
+  b->collide_blocks = default_collide_blocks(storage);
+  b->grid_collide = b->collide_blocks * b->sms;
   b->grid_particles = 8 * b->sms;
   b->hb.rep = b->d_rep;
   b->hb.state = b->d_state;
